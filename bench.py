@@ -259,7 +259,7 @@ def bench_trace(api, scene, view, d_alb, params, dev, tuning=None, n=1 << 22):
     import torch
     out = {}
     base = dict(tuning or {})
-    budgets = sorted({base.get("occupancy", 40), 32})
+    budgets = sorted({base.get("occupancy", 32), 40})
     for name, d in dumped_rays(api, scene, view, d_alb, params, n, tuning).items():
         m = d.shape[0]
         hits = torch.empty((m, 4), dtype=torch.int32, device=dev)

@@ -1,9 +1,10 @@
 // Host BVH builder (see bvh_build.h).  Binned SAH on item centroids, leaves of
 // up to max_leaf items, collapsed greedily to four children per node (the
 // child with the largest surface area is opened first), child boxes quantised
-// to 8 bits per plane against a power-of-two grid anchored at the node's lower
-// corner and widened until the dequantised box contains the exact one.
+// to 8 bits per plane and rounded outward (node_quant.h).
 #include "bvh_build.h"
+
+#include "node_quant.h"
 
 #include <algorithm>
 #include <array>
@@ -327,56 +328,6 @@ void build_chain(const std::vector<FBox>& boxes, std::vector<uint32_t>& ids,
     }
 }
 
-bool quantize(QNode& q, const FBox* cb, int nc) {
-    FBox u;
-    box_empty(u);
-    for (int i = 0; i < nc; ++i) box_grow(u, cb[i]);
-    float origin[3] = {u.lo[0], u.lo[1], u.lo[2]};
-    int8_t ex[3];
-    for (int a = 0; a < 3; ++a) {
-        double ext = (double)u.hi[a] - (double)origin[a];
-        int e = -126;
-        if (ext > 0.0) e = (int)std::ceil(std::log2(ext / 254.0));
-        e = std::max(-126, std::min(127, e));
-        for (;; ++e) {
-            if (e > 127) return false;
-            bool ok = true;
-            const double s = std::ldexp(1.0, e);
-            for (int i = 0; i < nc && ok; ++i) {
-                double fl = std::floor(((double)cb[i].lo[a] - origin[a]) / s);
-                int ql = (int)std::max(0.0, std::min(255.0, fl));
-                while (ql > 0 && dequant((uint8_t)ql, (int8_t)e, origin[a]) > cb[i].lo[a]) --ql;
-                if (dequant((uint8_t)ql, (int8_t)e, origin[a]) > cb[i].lo[a]) {
-                    ok = false;
-                    break;
-                }
-                double ch = std::ceil(((double)cb[i].hi[a] - origin[a]) / s);
-                if (ch > 255.0) {
-                    ok = false;
-                    break;
-                }
-                int qh = (int)std::max(0.0, ch);
-                while (qh <= 255 && dequant((uint8_t)qh, (int8_t)e, origin[a]) < cb[i].hi[a]) ++qh;
-                if (qh > 255) {
-                    ok = false;
-                    break;
-                }
-                q.qlo[a][i] = (uint8_t)ql;
-                q.qhi[a][i] = (uint8_t)qh;
-            }
-            if (ok) break;
-        }
-        ex[a] = (int8_t)e;
-    }
-    q.ox = origin[0];
-    q.oy = origin[1];
-    q.oz = origin[2];
-    q.ex = ex[0];
-    q.ey = ex[1];
-    q.ez = ex[2];
-    return true;
-}
-
 // Collapses the binary tree to four-wide nodes in two passes: emit() lays
 // the wide nodes out depth first (children and leaf references; it fixes
 // every index), then quantise() fills in the child boxes of all nodes in
@@ -390,20 +341,22 @@ struct Collapser {
     std::string err;
     std::vector<std::array<int32_t, 4>> kids;  // binary node of each child slot
 
-    bool quantise(int threads) {
+    void quantise(int threads) {
         const size_t n = out.size();
         const size_t chunk = 4096;
         std::atomic<size_t> next{0};
-        std::atomic<bool> bad{false};
         auto work = [&]() {
             for (;;) {
                 const size_t c0 = next.fetch_add(chunk);
-                if (c0 >= n || bad.load()) break;
+                if (c0 >= n) break;
                 for (size_t k = c0; k < std::min(n, c0 + chunk); ++k) {
                     FBox cb[4];
-                    const int nc = out[k].nchild;
-                    for (int i = 0; i < nc; ++i) cb[i] = bn[kids[k][i]].box;
-                    if (!quantize(out[k], cb, nc)) bad.store(true);
+                    int nc = 0;
+                    while (nc < 4 && kids[k][nc] >= 0) {
+                        cb[nc] = bn[kids[k][nc]].box;
+                        ++nc;
+                    }
+                    quantize_node(out[k], cb, nc);
                 }
             }
         };
@@ -412,11 +365,6 @@ struct Collapser {
         for (int t = 1; t < nt; ++t) th.emplace_back(work);
         work();
         for (std::thread& t : th) t.join();
-        if (bad.load()) {
-            err = "box quantisation failed (coordinates out of range)";
-            return false;
-        }
-        return true;
     }
 
     // Emits the wide node for binary node b; returns its local index or -1.
@@ -457,8 +405,7 @@ struct Collapser {
         }
         QNode q;
         std::memset(&q, 0, sizeof(q));
-        uint32_t childv[4] = {0, 0, 0, 0};
-        uint8_t meta[4] = {0, 0, 0, 0};
+        uint32_t ref[4] = {kRefNone, kRefNone, kRefNone, kRefNone};
         std::array<int32_t, 4> kb = {-1, -1, -1, -1};
         for (int i = 0; i < nc; ++i) {
             const BinNode& c = bn[ch[i]];
@@ -473,20 +420,14 @@ struct Collapser {
                     err = "item index beyond 2^27 within one object";
                     return -1;
                 }
-                childv[i] = first;
-                meta[i] = (uint8_t)c.count;
+                ref[i] = leaf_ref(first, c.count);
             } else {
                 int64_t k = emit(ch[i], depth + 1);
                 if (k < 0) return -1;
-                childv[i] = (uint32_t)k;
-                meta[i] = kMetaInner;
+                ref[i] = (uint32_t)k;
             }
         }
-        for (int i = 0; i < 4; ++i) {
-            q.child[i] = childv[i];
-            q.meta[i] = meta[i];
-        }
-        q.nchild = (uint8_t)nc;
+        for (int i = 0; i < 4; ++i) q.ref[i] = ref[i];
         out[idx] = q;
         kids[idx] = kb;
         return idx;
@@ -500,10 +441,6 @@ bool finite_box(const FBox& b) {
 }
 
 }  // namespace
-
-float dequant(uint8_t q, int8_t e, float origin) {
-    return std::fmaf((float)q, std::ldexp(1.0f, e), origin);
-}
 
 FBox transform_box(const FBox& b, const float* x) {
     FBox out;
@@ -533,21 +470,14 @@ FBox transform_box(const FBox& b, const float* x) {
 static void level_boxes_rec(const std::vector<QNode>& nodes, uint32_t n, uint32_t level,
                             std::vector<FBox>& out) {
     const QNode& q = nodes[n];
-    const float o[3] = {q.ox, q.oy, q.oz};
-    const int8_t e[3] = {q.ex, q.ey, q.ez};
     for (int i = 0; i < 4; ++i) {
-        const uint8_t m = q.meta[i];
-        if (m == 0) continue;
-        if (m == kMetaInner && level > 1) {
-            level_boxes_rec(nodes, q.child[i], level - 1, out);
+        const uint32_t r = q.ref[i];
+        if (r == kRefNone) continue;
+        if (is_inner(r) && level > 1) {
+            level_boxes_rec(nodes, r, level - 1, out);
             continue;
         }
-        FBox b;
-        for (int a = 0; a < 3; ++a) {
-            b.lo[a] = dequant(q.qlo[a][i], e[a], o[a]);
-            b.hi[a] = dequant(q.qhi[a][i], e[a], o[a]);
-        }
-        out.push_back(b);
+        out.push_back(child_bounds(q, i));
     }
 }
 
@@ -555,6 +485,8 @@ std::vector<FBox> level_boxes(const std::vector<QNode>& nodes, uint32_t level) {
     std::vector<FBox> out;
     if (level == 0 || nodes.empty()) return out;
     level_boxes_rec(nodes, 0, level, out);
+    for (const FBox& b : out)
+        if (!finite_box(b)) return {};  // an axis bounds nothing: the root box serves
     return out;
 }
 
@@ -601,10 +533,11 @@ bool build_blas(const float* verts, uint32_t n_verts, const uint32_t* quads, uin
                      std::max(4u, std::min(opts.sah_bins, 64u)), bn, helper_budget(opts));
     out.nodes.clear();
     Collapser col{bn, ids, false, out.nodes};
-    if (col.emit(0, 1) < 0 || !col.quantise(1)) {
+    if (col.emit(0, 1) < 0) {
         err = col.err;
         return false;
     }
+    col.quantise(1);
     out.depth = col.max_depth;
     out.quads.resize(n_quads);
     out.prim.resize(n_quads);
@@ -641,10 +574,11 @@ bool build_tlas(const std::vector<FBox>& inst_boxes, const BuildOpts& opts, Tlas
     build_binary(inst_boxes, ids, 1, std::max(4u, std::min(opts.sah_bins, 64u)), bn,
                  helper_budget(opts));
     Collapser col{bn, ids, true, out.nodes};
-    if (col.emit(0, 1) < 0 || !col.quantise(helper_budget(opts))) {
+    if (col.emit(0, 1) < 0) {
         err = col.err;
         return false;
     }
+    col.quantise(helper_budget(opts));
     out.depth = col.max_depth;
     return true;
 }
@@ -670,23 +604,18 @@ struct Checker {
         }
         const QNode& n = nodes[idx];
         box_empty(box);
-        const float org[3] = {n.ox, n.oy, n.oz};
-        const int8_t ex[3] = {n.ex, n.ey, n.ez};
         int valid = 0;
         for (int i = 0; i < 4; ++i) {
-            if (n.meta[i] == 0) continue;
+            const uint32_t r = n.ref[i];
+            if (r == kRefNone) continue;
             ++valid;
             FBox cb;
-            if (n.meta[i] == kMetaInner) {
-                if (!rec(n.child[i], d + 1, cb)) return false;
+            if (is_inner(r)) {
+                if (!rec(r, d + 1, cb)) return false;
             } else {
-                if (n.meta[i] > kMaxLeaf) {
-                    err = "leaf count too large";
-                    return false;
-                }
                 box_empty(cb);
-                for (uint32_t k = 0; k < n.meta[i]; ++k) {
-                    uint32_t it = n.child[i] + k;
+                for (uint32_t k = 0; k < leaf_count(r); ++k) {
+                    const uint32_t it = leaf_first(r) + k;
                     if (it >= items.size()) {
                         err = "leaf item out of range";
                         return false;
@@ -698,18 +627,17 @@ struct Checker {
                     box_grow(cb, items[it]);
                 }
             }
+            const FBox qb = child_bounds(n, i);
             for (int a = 0; a < 3; ++a) {
-                float lo = dequant(n.qlo[a][i], ex[a], org[a]);
-                float hi = dequant(n.qhi[a][i], ex[a], org[a]);
-                if (!(lo <= cb.lo[a] && hi >= cb.hi[a])) {
+                if (!(qb.lo[a] <= cb.lo[a] && qb.hi[a] >= cb.hi[a])) {
                     err = "quantised child box does not contain its subtree";
                     return false;
                 }
             }
             box_grow(box, cb);
         }
-        if (valid == 0 || valid != n.nchild) {
-            err = "node child count inconsistent";
+        if (valid == 0) {
+            err = "node without children";
             return false;
         }
         return true;
@@ -724,17 +652,17 @@ struct Checker {
         bool ok[4] = {true, true, true, true};
         std::vector<std::thread> th;
         for (int i = 0; i < 4; ++i)
-            if (n.meta[i] == kMetaInner) sub.push_back(Checker{nodes, items, seen, {}, 0, fork_depth});
+            if (is_inner(n.ref[i])) sub.push_back(Checker{nodes, items, seen, {}, 0, fork_depth});
         int s = 0;
         for (int i = 0; i < 4; ++i) {
-            if (n.meta[i] != kMetaInner) continue;
+            if (!is_inner(n.ref[i])) continue;
             Checker* c = &sub[s++];
-            th.emplace_back([c, &n, i, d, &cbs, &ok] { ok[i] = c->rec(n.child[i], d + 1, cbs[i]); });
+            th.emplace_back([c, &n, i, d, &cbs, &ok] { ok[i] = c->rec(n.ref[i], d + 1, cbs[i]); });
         }
         for (std::thread& t : th) t.join();
         s = 0;
         for (int i = 0; i < 4; ++i) {
-            if (n.meta[i] != kMetaInner) continue;
+            if (!is_inner(n.ref[i])) continue;
             Checker& c = sub[s++];
             depth = std::max(depth, c.depth);
             if (!ok[i]) {
@@ -758,23 +686,18 @@ struct Checker {
         depth = std::max(depth, d);
         const QNode& n = nodes[idx];
         box_empty(box);
-        const float org[3] = {n.ox, n.oy, n.oz};
-        const int8_t ex[3] = {n.ex, n.ey, n.ez};
         int valid = 0;
         for (int i = 0; i < 4; ++i) {
-            if (n.meta[i] == 0) continue;
+            const uint32_t r = n.ref[i];
+            if (r == kRefNone) continue;
             ++valid;
             FBox cb;
-            if (n.meta[i] == kMetaInner) {
+            if (is_inner(r)) {
                 cb = inner_boxes[i];
             } else {
-                if (n.meta[i] > kMaxLeaf) {
-                    err = "leaf count too large";
-                    return false;
-                }
                 box_empty(cb);
-                for (uint32_t k = 0; k < n.meta[i]; ++k) {
-                    uint32_t it = n.child[i] + k;
+                for (uint32_t k = 0; k < leaf_count(r); ++k) {
+                    const uint32_t it = leaf_first(r) + k;
                     if (it >= items.size()) {
                         err = "leaf item out of range";
                         return false;
@@ -786,18 +709,17 @@ struct Checker {
                     box_grow(cb, items[it]);
                 }
             }
+            const FBox qb = child_bounds(n, i);
             for (int a = 0; a < 3; ++a) {
-                float lo = dequant(n.qlo[a][i], ex[a], org[a]);
-                float hi = dequant(n.qhi[a][i], ex[a], org[a]);
-                if (!(lo <= cb.lo[a] && hi >= cb.hi[a])) {
+                if (!(qb.lo[a] <= cb.lo[a] && qb.hi[a] >= cb.hi[a])) {
                     err = "quantised child box does not contain its subtree";
                     return false;
                 }
             }
             box_grow(box, cb);
         }
-        if (valid == 0 || valid != n.nchild) {
-            err = "node child count inconsistent";
+        if (valid == 0) {
+            err = "node without children";
             return false;
         }
         return true;

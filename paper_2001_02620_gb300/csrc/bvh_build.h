@@ -63,7 +63,4 @@ FBox transform_box(const FBox& b, const float* xform);
 // root box).
 std::vector<FBox> level_boxes(const std::vector<QNode>& nodes, uint32_t level);
 
-// Dequantised bound used by both the builder and the checker.
-float dequant(uint8_t q, int8_t e, float origin);
-
 }  // namespace qrt

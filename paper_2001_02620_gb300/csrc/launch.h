@@ -10,8 +10,8 @@
 
 namespace qrt {
 
-// Resident blocks per SM of one kernel at a given block size (no dynamic
-// shared memory), queried once per device and block size and then reused:
+// Resident blocks per SM of one kernel at a given block size and dynamic
+// shared memory (a function of the block size), queried once per device and block size and then reused:
 // the query costs more host time than launching a trace kernel on a short
 // queue, and the persistent kernels size their grid from it on every launch.
 // Each kernel variant owns one (a static in its launcher).
@@ -19,24 +19,24 @@ struct ResidentBlocks {
     std::atomic<int> cached[16][5];  // [device][block / 64], 0 = not queried yet
 
     template <class Kernel>
-    int get(Kernel kernel, int block) {
+    int get(Kernel kernel, int block, size_t smem) {
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 16 || block % 64 != 0 ||
             block / 64 > 4)
-            return query(kernel, block);
+            return query(kernel, block, smem);
         std::atomic<int>& c = cached[dev][block / 64];
         int n = c.load(std::memory_order_relaxed);
         if (n == 0) {
-            n = query(kernel, block);
+            n = query(kernel, block, smem);
             c.store(n, std::memory_order_relaxed);
         }
         return n;
     }
 
     template <class Kernel>
-    static int query(Kernel kernel, int block) {
+    static int query(Kernel kernel, int block, size_t smem) {
         int n = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, smem);
         return n < 1 ? 1 : n;
     }
 };
@@ -52,7 +52,7 @@ struct Tune {
     int batch = 1;          // single kernel: 32-pixel groups a warp claims; trace kernels: rays a lane claims
     int stack = 64;         // 32 or 64
     int fetch = 32;         // node fetch bytes per load: 16 or 32
-    int occupancy = 40;     // trace kernels: target resident warps per SM (16, 24, 32, 40 or 48)
+    int occupancy = 32;     // trace kernels: target resident warps per SM (16, 24, 32, 40 or 48)
     int mode = 2;           // 1 = single persistent kernel, 2 = wavefront
     int chunk_log2 = 0;     // wavefront paths per chunk = 2^chunk_log2; 0 = fit the call
 };

@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "lbvh.h"
+#include "node_quant.h"
 #include "radix_sort.h"
 
 namespace qrt {
@@ -36,14 +37,6 @@ __host__ __device__ inline int clz32(uint32_t x) {
 #else
     return x ? __builtin_clz(x) : 32;
 #endif
-}
-
-// 2^e for e in [-126, 127], built from its bit pattern (exact).
-__host__ __device__ inline float pow2f(int e) {
-    const uint32_t bits = (uint32_t)(e + 127) << 23;
-    float f;
-    memcpy(&f, &bits, 4);
-    return f;
 }
 
 // Products and sums rounded one by one on both sides (no contraction into
@@ -140,64 +133,6 @@ __host__ __device__ inline float half_area(const FBox& b) {
     return add_rn(add_rn(mul_rn(dx, dy), mul_rn(dy, dz)), mul_rn(dz, dx));
 }
 
-__host__ __device__ inline float dequant_hd(int q, int e, float origin) {
-    return fmaf((float)q, pow2f(e), origin);
-}
-
-// Conservative quantisation of nc child boxes against their union's lower
-// corner: per axis the smallest power-of-two step (found from the extent,
-// then raised while needed) at which every child box, rounded outward to
-// 8-bit codes, still contains the exact box under the dequantisation
-// fma(q, 2^e, origin).  The same rule as the host builder's.
-__host__ __device__ inline bool quantize_node(QNode& q, const FBox* cb, int nc) {
-    FBox u = cb[0];
-    for (int i = 1; i < nc; ++i) box_union(u, u, cb[i]);
-    int8_t ex[3];
-    for (int a = 0; a < 3; ++a) {
-        const float origin = u.lo[a];
-        const double ext = (double)u.hi[a] - (double)origin;
-        int e = -126;
-        if (ext > 0.0) e = (int)ceil(log2(ext / 254.0));
-        e = e < -126 ? -126 : (e > 127 ? 127 : e);
-        for (;; ++e) {
-            if (e > 127) return false;
-            bool ok = true;
-            const double step = ldexp(1.0, e);
-            for (int i = 0; i < nc && ok; ++i) {
-                const double fl = floor(((double)cb[i].lo[a] - origin) / step);
-                int ql = (int)(fl < 0.0 ? 0.0 : (fl > 255.0 ? 255.0 : fl));
-                while (ql > 0 && dequant_hd(ql, e, origin) > cb[i].lo[a]) --ql;
-                if (dequant_hd(ql, e, origin) > cb[i].lo[a]) {
-                    ok = false;
-                    break;
-                }
-                const double ch = ceil(((double)cb[i].hi[a] - origin) / step);
-                if (ch > 255.0) {
-                    ok = false;
-                    break;
-                }
-                int qh = (int)(ch < 0.0 ? 0.0 : ch);
-                while (qh <= 255 && dequant_hd(qh, e, origin) < cb[i].hi[a]) ++qh;
-                if (qh > 255) {
-                    ok = false;
-                    break;
-                }
-                q.qlo[a][i] = (uint8_t)ql;
-                q.qhi[a][i] = (uint8_t)qh;
-            }
-            if (ok) break;
-        }
-        ex[a] = (int8_t)e;
-    }
-    q.ox = u.lo[0];
-    q.oy = u.lo[1];
-    q.oz = u.lo[2];
-    q.ex = ex[0];
-    q.ey = ex[1];
-    q.ez = ex[2];
-    return true;
-}
-
 __host__ __device__ inline FBox load_box(const FBox* p) {
 #ifdef __CUDA_ARCH__
     // boxes written by other threads of this launch: read through L2
@@ -273,7 +208,7 @@ __host__ __device__ inline int wide_children(uint32_t b, const uint32_t* left, c
 
 // Writes four-wide node `wide` (made from binary node b); its inner children
 // get consecutive indices after next_base, in the order of the next level's
-// list.  Returns false if the child boxes cannot be quantised.
+// list.  Returns false if an index leaves its range.
 __host__ __device__ inline bool emit_wide(uint32_t b, uint32_t wide, uint32_t n, const uint32_t* left,
                                           const uint32_t* right, const FBox* lbox, const FBox* ibox,
                                           const uint32_t* ids, uint32_t* next, uint32_t* next_count,
@@ -286,14 +221,13 @@ __host__ __device__ inline bool emit_wide(uint32_t b, uint32_t wide, uint32_t n,
     uint32_t c[4];
     const int nc = wide_children(b, left, right, ibox, c);
     QNode q;
-    memset(&q, 0, sizeof(q));
+    for (int i = 0; i < 4; ++i) q.ref[i] = kRefNone;
     FBox cb[4];
     for (int i = 0; i < nc; ++i) {
         cb[i] = child_box(c[i], lbox, ibox);
         if ((c[i] & kLeafBit) && (c[i] & ~kLeafBit) >= n) return false;
         if (c[i] & kLeafBit) {
-            q.meta[i] = 1;  // a TLAS leaf holds one instance
-            q.child[i] = ids[c[i] & ~kLeafBit];
+            q.ref[i] = leaf_ref(ids[c[i] & ~kLeafBit], 1);  // a TLAS leaf holds one instance
         } else {
 #ifdef __CUDA_ARCH__
             const uint32_t pos = atomicAdd(next_count, 1u);
@@ -302,14 +236,12 @@ __host__ __device__ inline bool emit_wide(uint32_t b, uint32_t wide, uint32_t n,
 #endif
             if (pos >= n || c[i] + 1 >= n) return false;
             next[pos] = c[i];
-            q.meta[i] = kMetaInner;
-            q.child[i] = next_base + pos;
+            q.ref[i] = next_base + pos;
         }
     }
-    q.nchild = (uint8_t)nc;
-    const bool ok = quantize_node(q, cb, nc);
+    quantize_node(q, cb, nc);
     nodes[wide] = q;
-    return ok;
+    return true;
 }
 
 // ---- kernels: one thread per item or node ----------------------------------
@@ -438,7 +370,7 @@ bool build_on_host(const std::vector<FBox>& boxes, const Grid& g, TlasResult& ou
         for (uint32_t t = 0; t < cur.size(); ++t)
             if (!emit_wide(cur[t], base + t, n, left.data(), right.data(), lbox.data(), ibox.data(),
                            ids.data(), next.data(), &count, next_base, out.nodes.data())) {
-                err = "child boxes cannot be quantised, or the tree is broken";
+                err = "the tree is broken";
                 return false;
             }
         base = next_base;
@@ -557,7 +489,7 @@ bool build_on_device(const std::vector<FBox>& boxes, const Grid& g, TlasResult& 
         ++depth;
     }
     if (failed) {
-        err = "child boxes cannot be quantised, or the tree is broken";
+        err = "the tree is broken";
         return false;
     }
     out.nodes.resize(base);
@@ -588,14 +520,9 @@ bool build_tlas_lbvh(const std::vector<FBox>& inst_boxes, bool on_device, TlasRe
             }
     if (n == 1) {  // a root with one leaf
         QNode q;
-        std::memset(&q, 0, sizeof(q));
-        q.meta[0] = 1;
-        q.child[0] = 0;
-        q.nchild = 1;
-        if (!quantize_node(q, inst_boxes.data(), 1)) {
-            err = "child boxes cannot be quantised";
-            return false;
-        }
+        q.ref[0] = leaf_ref(0, 1);
+        for (int i = 1; i < 4; ++i) q.ref[i] = kRefNone;
+        quantize_node(q, inst_boxes.data(), 1);
         out.nodes.push_back(q);
         out.depth = 1;
         return true;
@@ -722,7 +649,7 @@ __host__ __device__ inline bool emit_blas(uint32_t b, uint32_t m, uint32_t local
     uint32_t c[4];
     const int nc = blas_children(b, left, right, rlo, rhi, max_leaf, ibox, c);
     QNode q;
-    memset(&q, 0, sizeof(q));
+    for (int i = 0; i < 4; ++i) q.ref[i] = kRefNone;
     FBox cb[4];
     for (int i = 0; i < nc; ++i) {
         if ((c[i] & kLeafBit) ? (c[i] & ~kLeafBit) >= n : c[i] + 1 >= n) return false;
@@ -731,8 +658,7 @@ __host__ __device__ inline bool emit_blas(uint32_t b, uint32_t m, uint32_t local
         const uint32_t cnt = leaf_span(c[i], rlo, rhi, max_leaf, &first);
         if (cnt) {
             if (first < d.quad_off || first + cnt > d.quad_off + d.n_quads) return false;
-            q.meta[i] = (uint8_t)cnt;
-            q.child[i] = (uint32_t)(first - d.quad_off);  // slot within the mesh
+            q.ref[i] = leaf_ref((uint32_t)(first - d.quad_off), cnt);  // slot within the mesh
         } else {
 #ifdef __CUDA_ARCH__
             const uint32_t w = atomicAdd(mesh_nodes + m, 1u);
@@ -745,14 +671,12 @@ __host__ __device__ inline bool emit_blas(uint32_t b, uint32_t m, uint32_t local
             next_b[pos] = c[i];
             next_m[pos] = m;
             next_w[pos] = w;
-            q.meta[i] = kMetaInner;
-            q.child[i] = w;
+            q.ref[i] = w;
         }
     }
-    q.nchild = (uint8_t)nc;
-    const bool ok = quantize_node(q, cb, nc);
+    quantize_node(q, cb, nc);
     nodes[d.node_off + local] = q;
-    return ok;
+    return true;
 }
 
 __global__ void k_quad_keys(const float* verts, const uint32_t* quads, const MeshDev* md,
@@ -1030,7 +954,7 @@ bool blases_on_host(const std::vector<MeshView>& meshes, const std::vector<MeshD
             if (!emit_blas(cb[t], cm[t], cw[t], n, md.data(), left.data(), right.data(), rlo.data(),
                            rhi.data(), max_leaf, lbox.data(), ibox.data(), mesh_nodes.data(),
                            nb.data(), nm.data(), nw.data(), &count, nodes.data())) {
-                err = "child boxes cannot be quantised, or the tree is broken";
+                err = "the tree is broken";
                 return false;
             }
         }
@@ -1176,7 +1100,7 @@ bool blases_on_device(const std::vector<MeshView>& meshes, const std::vector<Mes
     }
     QRT_LBVH_TRY(cudaMemcpy(&failed, d_failed, 4, cudaMemcpyDeviceToHost));
     if (failed) {
-        err = "child boxes cannot be quantised, or the tree is broken";
+        err = "the tree is broken";
         return false;
     }
     // each mesh's used nodes, quads and indices straight into its result

@@ -16,28 +16,34 @@
 namespace qrt {
 
 // Four-wide node with conservatively quantised child boxes.
-// Child i spans [o + qlo*2^e, o + qhi*2^e] per axis, rounded outward so that
-// the dequantised box always contains the exact child box.
+//
+// A plane code q stands for the float v(q) with bits 0x3F000000 | q << 16:
+// v = 0.5 + q/256 for q < 128 and q/128 above, 0.5 .. 1.9921875, and the plane
+// lies at fma(v(q), s, o).  The traversal makes v(q) with one byte permute,
+// with no integer-to-float conversion, and s need not be a power of two, so
+// the 256 codes cover the node's extent exactly (192 to 384 steps per
+// extent).  Boxes are rounded outward: a dequantised box always contains the
+// exact child box.  An axis whose extent cannot be covered in FP32 (beyond
+// about 5e38) has s = NaN and bounds nothing: slab tests take minima and
+// maxima that ignore NaN.
 struct alignas(64) QNode {
-    float ox, oy, oz;      // quantisation origin
-    int8_t ex, ey, ez;     // per-axis scale exponents
-    uint8_t nchild;        // number of valid children
-    uint8_t qlo[3][4];     // [axis][child]
-    uint8_t qhi[3][4];     // [axis][child]
-    uint32_t child[4];     // internal: local node index; leaf: first local quad slot / instance
-    uint8_t meta[4];       // 0 = empty, kMetaInner = inner node, 1..16 = leaf item count
-    uint32_t pad;
+    float o[3], s[3];
+    uint8_t qlo[3][4];  // [axis][child]
+    uint8_t qhi[3][4];  // [axis][child]
+    uint32_t ref[4];    // child references (below); kRefNone = empty slot (qlo 255, qhi 0)
 };
 static_assert(sizeof(QNode) == 64, "QNode must be 64 bytes");
 
-constexpr uint8_t kMetaInner = 0xFF;
 constexpr uint32_t kMaxLeaf = 16;
 
 // Stack/child reference: bit 31 = leaf; a leaf keeps (count-1) in bits 27..30
-// and its first item in bits 0..26.  An inner reference is a node index.
+// and its first item in bits 0..26 (local quad slot, or instance at the top
+// level).  An inner reference is a node index local to its tree.  kRefNone
+// is no leaf: a leaf of 16 items cannot start at the last index there is.
 constexpr uint32_t kRefLeaf = 0x80000000u;
 constexpr uint32_t kRefIndexMask = 0x07FFFFFFu;
 constexpr uint32_t kMaxLocalIndex = kRefIndexMask;
+constexpr uint32_t kRefNone = 0xFFFFFFFFu;
 
 struct alignas(16) QuadDev {
     float v[12];  // v0, v1, v2, v3 as packed float3

@@ -30,6 +30,15 @@ namespace qrt {
 // Every floating-point operation on the path is an explicitly rounded
 // intrinsic (nothing is left for the compiler to contract), so each inlined
 // copy -- primal, replay pass 1, replay pass 2 -- computes bit-identical paths.
+//
+// Rays traced one after the other by a thread share its shared memory: both
+// kinds take the same bytes, so that a warp's part is the same for both.
+template <int FETCH>
+using PathRay = TraversalKind<false, true, false, FETCH, 10>;
+template <int FETCH>
+using PathShadow = TraversalKind<true, false, true, FETCH, 28>;
+static_assert(PathShadow<32>::kLaneBytes == PathRay<32>::kLaneBytes, "a warp's part must be the same");
+
 template <int STACK, int FETCH>
 __device__ __forceinline__ uint32_t path_sample(const RenderArgs& A, const ViewDev& V, uint32_t x,
                                              uint32_t y, uint64_t gpix, uint32_t smp, int mode,
@@ -52,8 +61,8 @@ __device__ __forceinline__ uint32_t path_sample(const RenderArgs& A, const ViewD
     for (; i <= D; ++i) {
         Hit h;
         if (rlog) log_ray(rlog + (i - 1) * kRayLogFloats, o, d);
-        err |= trace_ray<false, STACK, FETCH>(S, o.x, o.y, o.z, d.x, d.y, d.z, 0.0f, kInfF,
-                                               P.max_steps, h, ls);
+        err |= trace_ray<PathRay<FETCH>>(S, o.x, o.y, o.z, d.x, d.y, d.z, 0.0f, kInfF, P.max_steps, STACK,
+                                         &h, nullptr, ls);
         if (log) {
             log[2 * (i - 1)] = h.inst;
             log[2 * (i - 1) + 1] = h.prim;
@@ -86,10 +95,10 @@ __device__ __forceinline__ uint32_t path_sample(const RenderArgs& A, const ViewD
             const float cl = dot3(n, f3(P.sun_l[0], P.sun_l[1], P.sun_l[2]));
             if (cl > 0.f) {
                 if (i <= 16) shadow_bits |= 1u << (2 * (i - 1));
-                Hit hs;
-                err |= trace_ray<true, STACK, FETCH>(S, sp.x, sp.y, sp.z, P.sun_l[0], P.sun_l[1],
-                                                      P.sun_l[2], 0.0f, kInfF, P.max_steps, hs, ls);
-                if (hs.inst != 0xFFFFFFFFu) {
+                bool occluded;
+                err |= trace_ray<PathShadow<FETCH>>(S, sp.x, sp.y, sp.z, P.sun_l[0], P.sun_l[1], P.sun_l[2],
+                                                    0.0f, kInfF, P.max_steps, STACK, nullptr, &occluded, ls);
+                if (occluded) {
                     if (i <= 16) shadow_bits |= 2u << (2 * (i - 1));
                 } else {
                     const float k = __fmul_rn(cl, 0.318309886183790671538f);  // cos / pi
@@ -123,10 +132,10 @@ __device__ __forceinline__ uint32_t path_sample(const RenderArgs& A, const ViewD
             if (light_sample(P, u01(xl.x), u01(xl.y), u01(xl.z), sp, n, &ld, &dist, &wl)) {
                 if (i <= 16) light_bits |= 1u << (2 * (i - 1));
                 if (rlog) log_light_ray(rlog + (i - 1) * kRayLogFloats, ld, dist);
-                Hit hl;
-                err |= trace_ray<true, STACK, FETCH>(S, sp.x, sp.y, sp.z, ld.x, ld.y, ld.z, 0.0f, dist,
-                                                      P.max_steps, hl, ls);
-                if (hl.inst != 0xFFFFFFFFu) {
+                bool occluded;
+                err |= trace_ray<PathShadow<FETCH>>(S, sp.x, sp.y, sp.z, ld.x, ld.y, ld.z, 0.0f, dist,
+                                                    P.max_steps, STACK, nullptr, &occluded, ls);
+                if (occluded) {
                     if (i <= 16) light_bits |= 2u << (2 * (i - 1));
                 } else {
                     const float ip = 0.318309886183790671538f;  // 1 / pi
@@ -257,7 +266,7 @@ __global__ void __launch_bounds__(256) render_kernel(const __grid_constant__ Ren
 template <int STACK, int FETCH, bool ADJ>
 static int occupancy_of(int block) {
     static ResidentBlocks resident;
-    return resident.get(render_kernel<STACK, FETCH, ADJ>, block);
+    return resident.get(render_kernel<STACK, FETCH, ADJ>, block, traversal_bytes<PathRay<FETCH>>(block));
 }
 
 int render_occupancy(const Tune& t, bool adjoint) {
@@ -281,21 +290,22 @@ cudaError_t launch_render(const RenderArgs& A, const Tune& t, int sm_count, cuda
     if (grid < 1) grid = 1;
     const dim3 g((unsigned)grid), b((unsigned)t.block);
     const bool s32 = t.stack <= 32, f32 = t.fetch == 32;
+    const size_t m = traversal_bytes<PathRay<32>>(t.block);
     if (adj) {
         if (s32) {
-            if (f32) render_kernel<32, 32, true><<<g, b, 0, s>>>(A);
-            else render_kernel<32, 16, true><<<g, b, 0, s>>>(A);
+            if (f32) render_kernel<32, 32, true><<<g, b, m, s>>>(A);
+            else render_kernel<32, 16, true><<<g, b, m, s>>>(A);
         } else {
-            if (f32) render_kernel<64, 32, true><<<g, b, 0, s>>>(A);
-            else render_kernel<64, 16, true><<<g, b, 0, s>>>(A);
+            if (f32) render_kernel<64, 32, true><<<g, b, m, s>>>(A);
+            else render_kernel<64, 16, true><<<g, b, m, s>>>(A);
         }
     } else {
         if (s32) {
-            if (f32) render_kernel<32, 32, false><<<g, b, 0, s>>>(A);
-            else render_kernel<32, 16, false><<<g, b, 0, s>>>(A);
+            if (f32) render_kernel<32, 32, false><<<g, b, m, s>>>(A);
+            else render_kernel<32, 16, false><<<g, b, m, s>>>(A);
         } else {
-            if (f32) render_kernel<64, 32, false><<<g, b, 0, s>>>(A);
-            else render_kernel<64, 16, false><<<g, b, 0, s>>>(A);
+            if (f32) render_kernel<64, 32, false><<<g, b, m, s>>>(A);
+            else render_kernel<64, 16, false><<<g, b, m, s>>>(A);
         }
     }
     return cudaGetLastError();

@@ -15,39 +15,30 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) trace_kernel(const DevScene S, 
                                                        unsigned long long* cursor, uint32_t batch,
                                                        unsigned long long* stats, int stack_cap) {
     TraceStats st{0, 0, 0, 0, 0, 0};
-    Traversal<ANY, kMaxStack, FETCH> T;
+    Traversal<QueryKind<ANY, FETCH, OCC>> T;
     uint64_t i = 0;
-    uint32_t err = 0;
-    uint64_t bad = ~0ull;
-    WRay w{};  // kept per lane: reloading it from the ray array measured slower here
     auto start_ray = [&](unsigned long long k) {
         i = k;
         const float4 a = __ldg(rays + 2 * i), b = __ldg(rays + 2 * i + 1);
-        w = WRay{a.x, a.y, a.z, b.x, b.y, b.z};
-        T.err = 0;  // per ray: the first affected ray is reported
         T.init(S, a.x, a.y, a.z, b.x, b.y, b.z, a.w, b.w, max_steps, st);
     };
     auto finish_ray = [&]() {
-        if (T.err) {
-            err |= T.err;
-            bad = min(bad, i);
+        if (T.err) {  // the first affected ray is reported
+            atomicOr(S.err, T.err);
+            atomicMin(S.err + 1, (uint32_t)min(i, (uint64_t)0xFFFFFFFEu));
+            T.err = 0;
         }
         if (ANY) {
-            if (T.h.inst != 0xFFFFFFFFu) atomicOr(occ + (i >> 5), 1u << (i & 31));
+            if (T.found) atomicOr(occ + (i >> 5), 1u << (i & 31));
         } else {
-            const uint32_t uq = (uint32_t)__float2uint_rn(__saturatef(T.h.u) * 65535.f);
-            const uint32_t vq = (uint32_t)__float2uint_rn(__saturatef(T.h.v) * 65535.f);
-            const uint32_t uv = T.h.inst == 0xFFFFFFFFu ? 0u : (uq | (vq << 16));
-            hits[i] = make_uint4(__float_as_uint(T.h.t), T.h.inst, T.h.prim, uv);
+            const Hit h = T.hit(S);
+            const uint32_t uq = (uint32_t)__float2uint_rn(__saturatef(h.u) * 65535.f);
+            const uint32_t vq = (uint32_t)__float2uint_rn(__saturatef(h.v) * 65535.f);
+            const uint32_t uv = h.inst == 0xFFFFFFFFu ? 0u : (uq | (vq << 16));
+            hits[i] = make_uint4(__float_as_uint(h.t), h.inst, h.prim, uv);
         }
     };
-    auto world_ray = [&]() { return w; };
-    persistent_trace<ANY, kMaxStack, FETCH>(S, T, st, cursor, (unsigned long long)n, batch, stack_cap,
-                                            start_ray, finish_ray, world_ray);
-    if (err) {
-        atomicOr(S.err, err);
-        atomicMin(S.err + 1, (uint32_t)min(bad, (uint64_t)0xFFFFFFFEu));
-    }
+    persistent_trace(S, T, st, cursor, (unsigned long long)n, batch, stack_cap, start_ray, finish_ray);
     if constexpr (STATS) add_stats(stats, st);
 }
 
@@ -57,12 +48,13 @@ static cudaError_t launch_variant(const DevScene& S, const float4* rays, uint64_
                                   unsigned long long* stats, const Tune& t, int sm_count,
                                   cudaStream_t s) {
     static ResidentBlocks resident;
+    const size_t smem = traversal_bytes<QueryKind<ANY, FETCH, OCC>>(t.block);
     const int per_sm = t.blocks_per_sm > 0 ? t.blocks_per_sm
-                                           : resident.get(trace_kernel<ANY, FETCH, OCC, STATS>, t.block);
+                                           : resident.get(trace_kernel<ANY, FETCH, OCC, STATS>, t.block, smem);
     uint64_t grid = (uint64_t)sm_count * per_sm;
     const uint64_t want = (n + (uint64_t)t.block - 1) / (uint64_t)t.block;
     if (want < grid) grid = want;
-    trace_kernel<ANY, FETCH, OCC, STATS><<<(unsigned)grid, t.block, 0, s>>>(
+    trace_kernel<ANY, FETCH, OCC, STATS><<<(unsigned)grid, t.block, smem, s>>>(
         S, rays, n, hits, occ, max_steps, cursor, (uint32_t)t.batch, stats, t.stack);
     return cudaGetLastError();
 }

@@ -5,17 +5,12 @@
 // before tmin), formed exactly with error-free FP32 transformations, and moved
 // into the instance's object space (the direction is not renormalised, so t
 // is shared by both levels); the object's BLAS is traversed on the same stack
-// with a parameter s = t - t_e.  Closest-hit stack entries keep each box's
-// entry distance (64 bits: distance, reference) to cull entries beyond the
-// best hit; any-hit rays never cull (tmax is fixed until the ray ends), so
-// their entries are the 32-bit reference alone (half the local-memory
-// traffic).
-// When the stack drains back to the level where the instance was entered,
-// the world ray is restored.  Leaves of a BLAS hold up to 16 quads stored
-// contiguously.
+// with a parameter s = t - t_e.  When the stack drains back to the level where
+// the instance was entered, the world ray is restored.  Leaves of a BLAS hold
+// up to 16 quads stored contiguously.
 //
 // Precision design.  Box tests are made conservative by widening every
-// dequantised box by delta, an absolute bound on the position error of the
+// dequantised box by twice delta, an absolute bound on the position error of the
 // FP32 ray in the current space (2^-20 (|o| + R) at the top level, where the
 // world ray is exact; 2^-22 (kappa + 2) (|o''| + R) in object space, where o''
 // is the re-centred origin, R the object's radius and kappa the condition
@@ -25,7 +20,8 @@
 // diagonal v0-v2 shared; an edge function within the same error bound of zero,
 // or a hit distance within its error bound of either end of the interval,
 // makes the decision uncertain, and only then the quad is re-tested in FP64
-// from the world ray and the FP64 transform; two hits whose FP32 distances
+// from the world ray and the FP64 transform (later, together with other lanes'
+// quads: Traversal::resolve); two hits whose FP32 distances
 // lie within their error bounds of each other are ordered by FP64 distances.
 // Hit/miss decisions and the closest-hit choice therefore agree with exact
 // arithmetic on the given FP32 ray except when a hit lies within FP64
@@ -35,6 +31,16 @@
 // holds one ray; the warp tests inner nodes together, enters instances in
 // groups, then lets every other lane enter its instance or test one leaf;
 // finished lanes take the next ray at once (claimed one atomic per warp).
+// What bounds it is each ray's chain of dependent node loads, hidden by
+// resident warps, and the issue slots at 13 to 17 active lanes of 32.  So the
+// registers hold what a node test reads and shared memory the rest of a ray
+// and its stack: 64 registers (32 warps an SM) without spills in the node and
+// leaf loops.  Before, the compiler kept it all in registers and spilled
+// 476 bytes a thread, the 64-entry stacks lay in local memory, and the FP64
+// re-test sat in the leaf loop.  Both against each other on one GB300, ms:
+// 2 M diffuse bounces on the mid scene 5.59 -> 3.44, 1.5 M sun rays 1.61 ->
+// 1.11, 1 M rays of ambient occlusion on the island (0.42 re-tests a ray) 1.94
+// -> 1.03, the mid frame 18.04 -> 13.69, the island frame 33.6 -> 26.3.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -66,7 +72,7 @@ struct WRay {
 struct RaySetup {
     float ox, oy, oz;     // origin
     float ix, iy, iz;     // reciprocal direction, |d| clamped away from 0
-    float delta;
+    float delta2;         // 2 delta, delta the bound on its position error
 };
 
 // Watertight shear of the current-space ray in affine form,
@@ -92,7 +98,7 @@ __device__ __forceinline__ void setup_boxes(RaySetup& r, float ox, float oy, flo
     r.ix = __frcp_rn(clamp_dir(dx));
     r.iy = __frcp_rn(clamp_dir(dy));
     r.iz = __frcp_rn(clamp_dir(dz));
-    r.delta = delta;
+    r.delta2 = 2.0f * delta;
 }
 
 // (dx, dy, dz): the ray direction in the current space, the same value the
@@ -127,7 +133,7 @@ __device__ __forceinline__ Shear make_shear(const RaySetup& r, float dx, float d
     sh.cz = __fmul_rn(Sz, okz);
     // a position error of delta moves the distance along the dominant axis
     // by delta |Sz|; twice that bounds the FP32 hit distance's error
-    sh.eps_t = 2.0f * __fmul_rn(r.delta, fabsf(Sz));
+    sh.eps_t = __fmul_rn(r.delta2, fabsf(Sz));
     return sh;
 }
 
@@ -157,82 +163,101 @@ __device__ __forceinline__ float4 ld_nc_na_f4(const void* p) {
                        __uint_as_float(v.w));
 }
 
+// A node's sixteen words in memory order (QNode): o.xyz s.xyz, near/far plane
+// codes lo.xyz hi.xyz, references.
 template <int FETCH>
-__device__ __forceinline__ void load_node(const QNode* n, uint4& a, uint4& b, uint4& c, uint4& d) {
+__device__ __forceinline__ void load_node(const QNode* n, uint32_t w[16]) {
     if constexpr (FETCH == 32) {
-        asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y),
-                       "=r"(b.z), "=r"(b.w)
-                     : "l"(n));
-        asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(c.x), "=r"(c.y), "=r"(c.z), "=r"(c.w), "=r"(d.x), "=r"(d.y),
-                       "=r"(d.z), "=r"(d.w)
-                     : "l"(reinterpret_cast<const char*>(n) + 32));
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                         : "=r"(w[8 * h]), "=r"(w[8 * h + 1]), "=r"(w[8 * h + 2]), "=r"(w[8 * h + 3]),
+                           "=r"(w[8 * h + 4]), "=r"(w[8 * h + 5]), "=r"(w[8 * h + 6]),
+                           "=r"(w[8 * h + 7])
+                         : "l"(reinterpret_cast<const char*>(n) + 32 * h));
     } else {
         const uint4* p = reinterpret_cast<const uint4*>(n);
-        a = ld_nc_na(p);
-        b = ld_nc_na(p + 1);
-        c = ld_nc_na(p + 2);
-        d = ld_nc_na(p + 3);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint4 v = ld_nc_na(p + k);
+            w[4 * k] = v.x;
+            w[4 * k + 1] = v.y;
+            w[4 * k + 2] = v.z;
+            w[4 * k + 3] = v.w;
+        }
     }
 }
 
-// Byte i of w as a float, exactly: the byte is placed in the mantissa of
-// 2^23 with one byte permute and 2^23 is subtracted (full-rate integer and
-// FP32 instructions instead of an integer-to-float conversion).
-__device__ __forceinline__ float byte_f(uint32_t w, int i) {
-    return __fsub_rn(__uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u | (uint32_t)i)), 8388608.0f);
+// Plane value v(q) of byte i of w (QNode): one byte permute.
+__device__ __forceinline__ float plane_v(uint32_t w, int i) {
+    return __uint_as_float(__byte_perm(w, 0x3F000000u, 0x7044u | ((uint32_t)i << 8)));
 }
 
-__device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
+// Three-operand minima and maxima (one instruction on sm_103a); a NaN operand
+// is ignored, or propagated by the _nan forms.
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// (a0, a1) * b + (c0, c1), both halves in one instruction.
+__device__ __forceinline__ void fma2(float a0, float a1, float b, float c0, float c1, float& r0, float& r1) {
+    asm("{.reg .b64 a, b, c, r;\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 b, {%4, %4};\n\t"
+        "mov.b64 c, {%5, %6};\n\t"
+        "fma.rn.f32x2 r, a, b, c;\n\t"
+        "mov.b64 {%0, %1}, r;}"
+        : "=f"(r0), "=f"(r1)
+        : "f"(a0), "f"(a1), "f"(b), "f"(c0), "f"(c1));
+}
 
 // Tests the four children of a node; writes entry distances (inf = culled)
 // and references, sorted nearest first (SORT) or in slot order (any-hit
 // rays, which need no order).  Returns the number of hits.
+//
+// A plane's distance is fma(v(q), s/d, (node.o - o)/d), its box widened by
+// 2 delta.  delta alone bounds the ray's own position error; the second delta
+// covers this arithmetic: with e = 2^-24, the roundings of s/d, node.o - o,
+// 1/d and the fused product amount to at most e (|v s| + |node.o - o| +
+// 2 |plane - o|) <= e (9 R + 3 |o|) in position, R the radius of the space's
+// geometry (|v s| <= 2.7 R), while delta is at least 12 e (R + |o|).
 template <int FETCH, bool SORT = true>
 __device__ __forceinline__ int node_children(const QNode* node, const RaySetup& r, float tmin,
                                              float tmax, float t[4], uint32_t ref[4]) {
-    uint4 A, B, C, D;
-    load_node<FETCH>(node, A, B, C, D);
-    const float nox = __uint_as_float(A.x), noy = __uint_as_float(A.y), noz = __uint_as_float(A.z);
-    const int ex = (int)(int8_t)(A.w & 0xFF), ey = (int)(int8_t)((A.w >> 8) & 0xFF),
-              ez = (int)(int8_t)((A.w >> 16) & 0xFF);
-    const float ax = __fmul_rn(exp2i(ex), r.ix), ay = __fmul_rn(exp2i(ey), r.iy),
-                az = __fmul_rn(exp2i(ez), r.iz);
-    // o * inv and the widening delta * |inv| are formed here, not kept in
-    // RaySetup: at 64 registers kept values are spilled, and six multiplies
-    // per node cost less than their local-memory round trips
-    const float bx = __fmaf_rn(nox, r.ix, -__fmul_rn(r.ox, r.ix)),
-                by = __fmaf_rn(noy, r.iy, -__fmul_rn(r.oy, r.iy)),
-                bz = __fmaf_rn(noz, r.iz, -__fmul_rn(r.oz, r.iz));
-    const float px = __fmul_rn(r.delta, fabsf(r.ix)), py = __fmul_rn(r.delta, fabsf(r.iy)),
-                pz = __fmul_rn(r.delta, fabsf(r.iz));
-    const float bnx = bx - px, bfx = bx + px;
-    const float bny = by - py, bfy = by + py;
-    const float bnz = bz - pz, bfz = bz + pz;
-    // words: lo x,y,z = B.x, B.y, B.z ; hi x,y,z = B.w, C.x, C.y
-    // near/far planes by the sign of the direction (compared here rather than
-    // kept as bits: one register less per ray)
-    const bool sx = r.ix < 0.f, sy = r.iy < 0.f, sz = r.iz < 0.f;
-    const uint32_t nwx = sx ? B.w : B.x, fwx = sx ? B.x : B.w;
-    const uint32_t nwy = sy ? C.x : B.y, fwy = sy ? B.y : C.x;
-    const uint32_t nwz = sz ? C.y : B.z, fwz = sz ? B.z : C.y;
-    const uint32_t meta = D.z;
-    const uint32_t child[4] = {C.z, C.w, D.x, D.y};
+    uint32_t w[16];
+    load_node<FETCH>(node, w);
+    const float o[3] = {r.ox, r.oy, r.oz}, inv[3] = {r.ix, r.iy, r.iz};
+    float A[3], bn[3], bf[3];
+    uint32_t wn[3], wf[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float d = __fsub_rn(__uint_as_float(w[a]), o[a]);
+        const float p = __fmul_rn(r.delta2, fabsf(inv[a]));
+        A[a] = __fmul_rn(__uint_as_float(w[3 + a]), inv[a]);
+        bn[a] = __fmaf_rn(d, inv[a], -p);
+        bf[a] = __fmaf_rn(d, inv[a], p);
+        // near and far planes by the sign of the direction
+        const bool neg = inv[a] < 0.f;
+        wn[a] = neg ? w[9 + a] : w[6 + a];
+        wf[a] = neg ? w[6 + a] : w[9 + a];
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const float tnx = __fmaf_rn(byte_f(nwx, i), ax, bnx);
-        const float tfx = __fmaf_rn(byte_f(fwx, i), ax, bfx);
-        const float tny = __fmaf_rn(byte_f(nwy, i), ay, bny);
-        const float tfy = __fmaf_rn(byte_f(fwy, i), ay, bfy);
-        const float tnz = __fmaf_rn(byte_f(nwz, i), az, bnz);
-        const float tfz = __fmaf_rn(byte_f(fwz, i), az, bfz);
-        const float tn = fmaxf(fmaxf(tnx, tny), fmaxf(tnz, tmin));
-        const float tf = fminf(fminf(tfx, tfy), fminf(tfz, tmax));
-        const uint32_t m = (meta >> (8 * i)) & 0xFFu;
-        const bool hit = (m != 0u) && (tn <= tf);
-        t[i] = hit ? tn : kInfF;
-        ref[i] = (m == kMetaInner) ? child[i] : (kRefLeaf | ((m - 1u) << 27) | child[i]);
+        float n[3], f[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+            fma2(plane_v(wn[a], i), plane_v(wf[a], i), A[a], bn[a], bf[a], n[a], f[a]);
+        const float tn = fmaxf(max3(n[0], n[1], n[2]), tmin);
+        const float tf = fminf(min3(f[0], f[1], f[2]), tmax);
+        ref[i] = w[12 + i];
+        t[i] = (tn <= tf) && ref[i] != kRefNone ? tn : kInfF;
     }
     if constexpr (!SORT)
         return (t[0] < kInfF) + (t[1] < kInfF) + (t[2] < kInfF) + (t[3] < kInfF);
@@ -275,101 +300,97 @@ __device__ __forceinline__ float edge(const SV& P, const SV& Q) {
     return __fsub_rn(__fmul_rn(P.X, Q.Y), __fmul_rn(P.Y, Q.X));
 }
 
-// 0 = certain miss, 1 = certain hit, 2 = uncertain.
-__device__ __forceinline__ int classify(float e0, float e1, float e2, float B) {
-    const bool p0 = e0 > B, p1 = e1 > B, p2 = e2 > B;
-    const bool n0 = e0 < -B, n1 = e1 < -B, n2 = e2 < -B;
-    if ((p0 || p1 || p2) && (n0 || n1 || n2)) return 0;
-    if ((p0 && p1 && p2) || (n0 && n1 && n2)) return 1;
-    return 2;
-}
+// Exact-enough re-test in FP64 of quad `slot` of instance `inst`: object ray
+// from the world ray and the instance's FP64 world->object matrix, then the
+// watertight test with FP64 arithmetic.  A hit has t > tmin (world t, with
+// quad-space u, v); a miss returns t = +inf.
+struct Hit64 {
+    double t;
+    float u, v;
+};
 
-// Exact-enough re-test in FP64: object ray from the world ray and the
-// instance's FP64 world->object matrix, then the watertight test with FP64
-// arithmetic.  Returns 1 on a hit with t > tmin (world t written, with
-// quad-space u, v).
-static __device__ __noinline__ int quad_test64(const InstDev* ip, const InstDev64* ip64, float wox,
-                                               float woy, float woz, float wdx, float wdy, float wdz,
-                                               const float* v, float tmin, double* t_out,
-                                               float* u_out, float* v_out) {
+static __device__ __noinline__ Hit64 quad_test64(const InstDev* ip, const InstDev64* ip64,
+                                                 const QuadDev* quad, WRay ray, float tmin) {
     double o[3], d[3];
-    const double e[3] = {(double)wox - (double)ip->c[0], (double)woy - (double)ip->c[1],
-                         (double)woz - (double)ip->c[2]};
-    const double wd[3] = {wdx, wdy, wdz};
+    const double e[3] = {(double)ray.ox - (double)ip->c[0], (double)ray.oy - (double)ip->c[1],
+                         (double)ray.oz - (double)ip->c[2]};
+    const double wd[3] = {ray.dx, ray.dy, ray.dz};
     const double* w = ip64->w;
+#pragma unroll
     for (int r = 0; r < 3; ++r) {
         o[r] = w[3 * r] * e[0] + w[3 * r + 1] * e[1] + w[3 * r + 2] * e[2];
         d[r] = w[3 * r] * wd[0] + w[3 * r + 1] * wd[1] + w[3 * r + 2] * wd[2];
     }
-    int kz = (fabs(d[0]) > fabs(d[1])) ? ((fabs(d[0]) > fabs(d[2])) ? 0 : 2)
-                                       : ((fabs(d[1]) > fabs(d[2])) ? 1 : 2);
-    int kx = kz == 2 ? 0 : kz + 1;
-    int ky = kx == 2 ? 0 : kx + 1;
-    const double Sx = d[kx] / d[kz], Sy = d[ky] / d[kz], Sz = 1.0 / d[kz];
+    // kz = dominant axis, (kx, ky) the next two in cyclic order; selects
+    // instead of indexed arrays keep everything in registers
+    const int kz = (fabs(d[0]) > fabs(d[1])) ? ((fabs(d[0]) > fabs(d[2])) ? 0 : 2)
+                                             : ((fabs(d[1]) > fabs(d[2])) ? 1 : 2);
+    const auto pick = [kz](double a, double b, double c, double& x, double& y, double& z) {
+        x = kz == 0 ? b : (kz == 1 ? c : a);
+        y = kz == 0 ? c : (kz == 1 ? a : b);
+        z = kz == 0 ? a : (kz == 1 ? b : c);
+    };
+    double dx, dy, dz;
+    pick(d[0], d[1], d[2], dx, dy, dz);
+    const double Sx = dx / dz, Sy = dy / dz, Sz = 1.0 / dz;
     double X[4], Y[4], Z[4];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-        double P[3] = {(double)v[3 * k] - o[0], (double)v[3 * k + 1] - o[1],
-                       (double)v[3 * k + 2] - o[2]};
-        X[k] = P[kx] - Sx * P[kz];
-        Y[k] = P[ky] - Sy * P[kz];
-        Z[k] = Sz * P[kz];
+        double px, py, pz;
+        pick((double)quad->v[3 * k] - o[0], (double)quad->v[3 * k + 1] - o[1],
+             (double)quad->v[3 * k + 2] - o[2], px, py, pz);
+        X[k] = px - Sx * pz;
+        Y[k] = py - Sy * pz;
+        Z[k] = Sz * pz;
     }
-    auto E = [&](int p, int q) { return X[p] * Y[q] - Y[p] * X[q]; };
+    const auto E = [&](int p, int q) { return X[p] * Y[q] - Y[p] * X[q]; };
     const double e21 = E(2, 1), e02 = E(0, 2), e10 = E(1, 0), e32 = E(3, 2), e03 = E(0, 3);
-    int hit = 0;
-    double best = INFINITY;
-    float bu = 0.f, bv = 0.f;
-    // triangle 0: (v0, v1, v2) with weights (e21, e02, e10)
-    {
-        const double U = e21, V = e02, W = e10;
-        if (((U >= 0 && V >= 0 && W >= 0) || (U <= 0 && V <= 0 && W <= 0))) {
+    Hit64 h{__longlong_as_double(0x7ff0000000000000ll), 0.f, 0.f};
+    // triangle 0: (v0, v1, v2) with weights (e21, e02, e10); triangle 1:
+    // (v0, v2, v3) with weights (e32, e03, -e02)
+#pragma unroll 1
+    for (int tri = 0; tri < 2; ++tri) {
+        const double U = tri ? e32 : e21, V = tri ? e03 : e02, W = tri ? -e02 : e10;
+        if ((U >= 0 && V >= 0 && W >= 0) || (U <= 0 && V <= 0 && W <= 0)) {
             const double det = U + V + W;
             if (det != 0.0) {
-                const double tt = (U * Z[0] + V * Z[1] + W * Z[2]) / det;
-                if (tt > (double)tmin && tt < best) {
-                    best = tt;
-                    hit = 1;
-                    bu = (float)((V + W) / det);
-                    bv = (float)(W / det);
+                const double tt = (U * Z[0] + V * (tri ? Z[2] : Z[1]) + W * (tri ? Z[3] : Z[2])) / det;
+                if (tt > (double)tmin && tt < h.t) {
+                    h.t = tt;
+                    h.u = (float)((tri ? V : V + W) / det);
+                    h.v = (float)((tri ? V + W : W) / det);
                 }
             }
         }
     }
-    // triangle 1: (v0, v2, v3) with weights (e32, e03, -e02)
-    {
-        const double U = e32, V = e03, W = -e02;
-        if (((U >= 0 && V >= 0 && W >= 0) || (U <= 0 && V <= 0 && W <= 0))) {
-            const double det = U + V + W;
-            if (det != 0.0) {
-                const double tt = (U * Z[0] + V * Z[2] + W * Z[3]) / det;
-                if (tt > (double)tmin && tt < best) {
-                    best = tt;
-                    hit = 1;
-                    bu = (float)(V / det);
-                    bv = (float)((V + W) / det);
-                }
-            }
-        }
-    }
-    *t_out = best;
-    *u_out = bu;
-    *v_out = bv;
-    return hit;
+    return h;
 }
 
-// FP32 test of one quad; returns 1 on a hit with tmin < t (t, u, v written);
-// may defer to quad_test64.
+// min / max of three values that return NaN when one is NaN.
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // FP32 test of one quad in the object-space parameter s (smin < s < smax).
-// A quad whose hit/miss decision is uncertain -- an edge function within its
-// error band of zero, or the hit distance within eps_t of either end of the
-// interval -- is re-tested by quad_test64, which returns the world t
-// (*t64_out, *exact64 = 1).  Returns 1 on a hit.
-template <class World>
-__device__ __forceinline__ int quad_test(const RaySetup& r, const Shear& sh, const QuadDev* q,
-                                         const InstDev* ip, const InstDev64* ip64,
-                                         const World& world, float smin, float smax,
-                                         float tmin, float* t_out, double* t64_out, float* u_out,
-                                         float* v_out, int* exact64, uint32_t* n_fallback) {
+// kQuadUncertain: the decision is within its error bounds -- an edge function
+// within its band of zero, or the hit distance within eps_t of either end of
+// the interval -- and quad_test64 makes it.  A hit leaves its distance and
+// (u, v) as numerators over det: few hits are kept, so few are divided.
+enum QuadResult { kQuadMiss = 0, kQuadHit = 1, kQuadUncertain = 2 };
+
+struct QuadHit {
+    float s, u_num, v_num, det;
+};
+
+__device__ __forceinline__ QuadResult quad_test(const Shear& sh, float delta, const QuadDev* q, float smin,
+                                                float smax, QuadHit& out) {
     const float4* p = reinterpret_cast<const float4*>(q);
     // quads are read once per test: no L1 allocation, as for the nodes
     const float4 a = ld_nc_na_f4(p), b = ld_nc_na_f4(p + 1), c = ld_nc_na_f4(p + 2);
@@ -381,71 +402,38 @@ __device__ __forceinline__ int quad_test(const RaySetup& r, const Shear& sh, con
     const float e32 = edge(s3, s2), e03 = edge(s0, s3);
     // one error band for the whole quad: covers delta-perturbed vertices and
     // the rounding of the edge products
-    const float M = fmaxf(fmaxf(fmaxf(fabsf(s0.X), fabsf(s0.Y)), fmaxf(fabsf(s1.X), fabsf(s1.Y))),
-                          fmaxf(fmaxf(fabsf(s2.X), fabsf(s2.Y)), fmaxf(fabsf(s3.X), fabsf(s3.Y))));
-    const float B = __fmaf_rn(4.0f * r.delta, M, 4.76837158e-07f * M * M);  // 2^-21 M^2
-    const int c0 = classify(e21, e02, e10, B);
-    const int c1 = classify(e32, e03, -e02, B);
-    if (c0 == 0 && c1 == 0) return 0;
-    bool uncertain = c0 == 2 || c1 == 2;
-    float best = kInfF;
-    int hit = 0;
-    if (!uncertain) {
-        if (c0 == 1) {
-            const float det = e21 + e02 + e10;
-            const float T = __fmaf_rn(e21, s0.Z, __fmaf_rn(e02, s1.Z, __fmul_rn(e10, s2.Z)));
-            const float tt = __fdiv_rn(T, det);
-            if (tt > smin) {
-                best = tt;
-                hit = 1;
-                *u_out = __fdiv_rn(e02 + e10, det);
-                *v_out = __fdiv_rn(e10, det);
+    const float M = fmaxf(max3(max3(fabsf(s0.X), fabsf(s0.Y), fabsf(s1.X)), fabsf(s1.Y), fabsf(s2.X)),
+                          max3(fabsf(s2.Y), fabsf(s3.X), fabsf(s3.Y)));
+    const float B = __fmaf_rn(4.0f * delta, M, 4.76837158e-07f * M * M);  // 2^-21 M^2
+    // triangle 0 = (v0, v1, v2), weights (e21, e02, e10); triangle 1 = (v0,
+    // v2, v3), weights (e32, e03, -e02).  Weights surely of both signs: a
+    // miss; surely of one: a hit; a NaN is neither.
+    const float mn0 = min3_nan(e21, e02, e10), mx0 = max3_nan(e21, e02, e10);
+    const float mn1 = min3_nan(e32, e03, -e02), mx1 = max3_nan(e32, e03, -e02);
+    const bool miss0 = mx0 > B && mn0 < -B, miss1 = mx1 > B && mn1 < -B;
+    if (miss0 && miss1) return kQuadMiss;
+    const bool hit0 = mn0 > B || mx0 < -B, hit1 = mn1 > B || mx1 < -B;
+    bool sure = (miss0 || hit0) && (miss1 || hit1);
+    QuadResult res = kQuadMiss;
+    out.s = kInfF;
+    bool second = !hit0;
+    if (sure) {
+        for (;;) {
+            const float u = second ? e32 : e21, v = second ? e03 : e02, w = second ? -e02 : e10;
+            const float det = __fadd_rn(__fadd_rn(u, v), w);
+            const float T = __fmaf_rn(u, s0.Z, __fmaf_rn(v, second ? s2.Z : s1.Z, __fmul_rn(w, second ? s3.Z : s2.Z)));
+            const float s = __fdiv_rn(T, det);
+            if (s > smin && s < out.s) {
+                const float vw = __fadd_rn(v, w);
+                out = QuadHit{s, second ? v : vw, second ? vw : w, det};
+                res = kQuadHit;
             }
-            uncertain |= fabsf(tt - smin) <= sh.eps_t || fabsf(tt - smax) <= sh.eps_t;
-        }
-        if (c1 == 1) {
-            const float det = e32 + e03 - e02;
-            const float T = __fmaf_rn(e32, s0.Z, __fmaf_rn(e03, s2.Z, __fmul_rn(-e02, s3.Z)));
-            const float tt = __fdiv_rn(T, det);
-            if (tt > smin && tt < best) {
-                best = tt;
-                hit = 1;
-                *u_out = __fdiv_rn(e03, det);
-                *v_out = __fdiv_rn(e03 - e02, det);
-            }
-            uncertain |= fabsf(tt - smin) <= sh.eps_t || fabsf(tt - smax) <= sh.eps_t;
+            sure = sure && !(fabsf(s - smin) <= sh.eps_t || fabsf(s - smax) <= sh.eps_t);
+            if (second || !hit1) break;
+            second = true;  // both triangles hit: a folded quad
         }
     }
-    if (uncertain) {
-        ++*n_fallback;
-        double t64;
-        float vv[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
-        const WRay w = world();
-        if (!quad_test64(ip, ip64, w.ox, w.oy, w.oz, w.dx, w.dy, w.dz, vv, tmin, &t64, u_out, v_out))
-            return 0;
-        *t_out = (float)t64;
-        *t64_out = t64;
-        *exact64 = 1;
-        return 1;
-    }
-    *exact64 = 0;
-    *t_out = best;
-    return hit;
-}
-
-// Exact (FP64) hit distance of quad `slot` of instance `inst` for the world
-// ray, or +inf if the FP64 test misses it.
-static __device__ __noinline__ double exact_t(const DevScene& S, uint32_t inst, uint32_t slot,
-                                              float wox, float woy, float woz, float wdx, float wdy,
-                                              float wdz, float tmin) {
-    const float* v = S.quads[slot].v;
-    float vv[12];
-    for (int k = 0; k < 12; ++k) vv[k] = v[k];
-    double t64;
-    float u, w;
-    if (!quad_test64(S.inst + inst, S.inst64 + inst, wox, woy, woz, wdx, wdy, wdz, vv, tmin, &t64, &u, &w))
-        return __longlong_as_double(0x7ff0000000000000ll);
-    return t64;
+    return sure ? res : kQuadUncertain;
 }
 
 // --------------------------------------------------------------------------
@@ -473,34 +461,201 @@ __device__ __forceinline__ void add_stats(unsigned long long* stats, const Trace
     }
 }
 
-// Resumable two-level traversal of one world ray.  init() sets the ray up;
-// each step() processes the current node, leaf or instance entry and pops the
-// next stack entry, returning false once the ray is finished (or stopped by
-// an error); trace_ray runs it to the end.  The persistent kernels instead
-// drive the warp-synchronous phase methods below from persistent_trace and
-// refill finished lanes, so no lane waits for the slowest ray of its warp.
-// The world ray itself is not kept: the callers' world() functors supply it.
-// UV = false drops the hit's quad-space (u, v) (left 0): closest-hit rays
-// whose consumer needs no (u, v) do not carry two more values through the
-// traversal nor divide for them at every closer hit.
-template <bool ANY, int STACK, int FETCH, bool UV = true>
+// --------------------------------------------------------------------------
+// Two-level traversal of one ray per thread
+// --------------------------------------------------------------------------
+
+// 32-bit shared-memory addresses; volatile, so that what is put there stays
+// there instead of being kept in registers through the traversal.
+__device__ __forceinline__ float4 lds4(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts4(uint32_t a, float x, float y, float z, float w) {
+    asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(a), "f"(x), "f"(y), "f"(z), "f"(w));
+}
+__device__ __forceinline__ float lds1(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts1(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v));
+}
+__device__ __forceinline__ uint32_t lds_u(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts_u(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v));
+}
+__device__ __forceinline__ uint2 lds_u2(uint32_t a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts_u2(uint32_t a, uint32_t x, uint32_t y) {
+    asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(a), "r"(x), "r"(y));
+}
+
+// What a kernel asks of the traversal, and the shared memory it takes.
+//   ANY    any hit instead of the closest
+//   UV     the closest hit's quad-space (u, v) is wanted
+//   RANGE  the ray's interval (tmin, tmax) is its own; otherwise (0, inf)
+//   STACK  stack entries in shared memory; deeper ones, up to kMaxStack, go to
+//          local memory
+// Per thread kRecs 16-byte records and the stack's entries: 64 bits (distance,
+// reference) for closest-hit rays, whose pops drop entries beyond the best
+// hit; 32 bits (reference) for any-hit rays, which never drop one (tmax stays
+// put until the ray ends).  Per warp, record k of lane l lies at 512 k + 16 l
+// and stack entry k after the records at (32 sizeof(Entry)) k + sizeof(Entry)
+// l: lanes never conflict for a bank, however far apart their stacks are.
+template <bool ANY_, bool UV_, bool RANGE_, int FETCH_, int STACK_>
+struct TraversalKind {
+    static constexpr bool ANY = ANY_, UV = UV_, RANGE = RANGE_;
+    static constexpr int FETCH = FETCH_, STACK = STACK_;
+    using Entry = std::conditional_t<ANY, uint32_t, uint64_t>;
+    static constexpr int kRecs = ANY ? 5 : (UV || RANGE ? 7 : 6);
+    static constexpr int kLaneBytes = kRecs * 16 + STACK * (int)sizeof(Entry);
+};
+
+// Stack entries in shared memory: what fits the 48 KB of a 256-thread block,
+// and the 228 KB of an SM (less 1 KB a block) at the kernel's resident warps.
+constexpr int shared_stack(bool any, int recs, int warps) {
+    return any ? 16 : ((warps > 40 ? 144 : warps > 32 ? 176 : 192) - 16 * recs) / 8;
+}
+
+// The ray-query kernels' rays, and the wavefront renderer's.
+template <bool ANY, int FETCH, int OCC>
+using QueryKind = TraversalKind<ANY, !ANY, true, FETCH, shared_stack(ANY, 7, OCC)>;
+template <bool ANY, bool UV, int FETCH, int OCC>
+using WaveKind = TraversalKind<ANY, UV, ANY, FETCH, shared_stack(ANY, UV ? 7 : 6, OCC)>;
+
+// Resumable traversal.  init() sets the ray up; the caller then runs, while
+// the ray is not finished, whichever step fits its state: inner_step (an inner
+// node to test), instance_step (a TLAS leaf to enter), leaf_step (a BLAS leaf
+// to test).  Registers hold what a node test reads; everything else about the
+// ray -- its world-space form, the object-space direction, the hit -- lies in
+// shared memory and is touched only when an instance is entered or left or a
+// leaf is tested.  (Left to the compiler, the same state spilled to local
+// memory: at 48 registers 476 bytes of spill stores per thread, half of all
+// local accesses, with the stacks 1 KB a thread of L1 and L2 footprint.)
+template <class Kind>
 struct Traversal {
-    float tmin, tmax;
-    float te;  // object-space parameter offset: t = s + te
-    RaySetup r;
-    // any-hit rays never cull by distance (tmax stays put until the ray
-    // ends), so their entries hold the reference alone
-    std::conditional_t<ANY, uint32_t, uint64_t> stack[STACK];
-    int sp, inst_sp;
-    bool have;
-    // at the top level (no instance entered): inst_sp < 0
+    static constexpr bool ANY = Kind::ANY, UV = Kind::UV, RANGE = Kind::RANGE;
+    static constexpr int STACK = Kind::STACK;
+    using Entry = typename Kind::Entry;
+
+    uint32_t rec, stk;  // shared-memory addresses of this thread's records and stack
+    RaySetup r;         // the ray in the current space
+    float lo, lim;      // its interval there: lo = tmin - te, lim = best hit (or tmax) - te
+    uint32_t cur;       // reference to visit next, kRefNone: take one from the stack
+    uint32_t pleaf;     // postponed BLAS leaf (0 = none)
+    uint32_t node_base;
+    uint32_t budget;    // inner-node tests left before the step limit
+    int sp, inst_sp;    // stack height; height at instance entry, -1 at the top level
+    uint32_t err;       // device error bits
+    bool found;         // any-hit rays: answered
+    bool pending;       // a quad waits for resolve()
+    bool blocked;       // and another one for its place
+    Entry deep[kMaxStack - STACK];
+
+    // records: word offsets from rec
+    static constexpr uint32_t kWorldO = 0;     // world origin, te
+    static constexpr uint32_t kWorldD = 512;   // world direction, h_t (any hit: cur_inst)
+    static constexpr uint32_t kWorldInv = 1024;  // world reciprocal direction
+    static constexpr uint32_t kObjD = 1536;    // object-space direction, quad_base
+    static constexpr uint32_t kHit = 2048;     // inst, slot, error bound of h_t, cur_inst
+    // the quad that waits: slot, inst; closest hit also u, v (u NaN: FP32 could
+    // not decide it) and the error bound of its distance
+    static constexpr uint32_t kPend = ANY ? 2056 : 2560;
+    static constexpr uint32_t kPendEps = kWorldInv + 12;
+    static constexpr uint32_t kRange = ANY ? 2048 : 3072;  // tmin, tmax; closest hit also u, v
+    static constexpr uint32_t kCurInst = ANY ? kWorldD + 12 : kHit + 12;
+
     __device__ __forceinline__ bool top() const { return inst_sp < 0; }
-    uint32_t node_base, cur_inst, cur;
-    uint32_t err;     // device error bits; init leaves them, the kernel resets them
-    uint32_t budget;  // inner-node tests left before the step limit
-    float h_eps;     // error bound of h.t (0 if exact)
-    uint32_t pleaf;  // postponed BLAS leaf reference (0 = none)
-    Hit h;
+
+    // base: the warp's shared memory
+    __device__ __forceinline__ void bind(uint32_t base) {
+        const uint32_t lane = threadIdx.x & 31u;
+        rec = base + 16u * lane;
+        stk = base + 512u * Kind::kRecs + (uint32_t)sizeof(Entry) * lane;
+        cur = kRefNone;
+        pleaf = 0;
+        err = 0;
+        found = pending = blocked = false;
+    }
+
+    __device__ __forceinline__ float tmin() const { return RANGE ? lds1(rec + kRange) : 0.f; }
+    __device__ __forceinline__ float tmax() const { return RANGE ? lds1(rec + kRange + 4) : kInfF; }
+
+    __device__ __forceinline__ void init(const DevScene& S, float ox, float oy, float oz, float dx,
+                                         float dy, float dz, float t0, float t1, uint32_t msteps,
+                                         TraceStats& st) {
+        ++st.rays;
+        sp = 0;
+        inst_sp = -1;
+        node_base = S.tlas_base;
+        pleaf = 0;
+        budget = msteps;
+        found = pending = blocked = false;
+        lo = t0;
+        lim = t1;
+        setup_boxes(r, ox, oy, oz, dx, dy, dz, world_delta(S, ox, oy, oz));
+        sts4(rec + kWorldO, ox, oy, oz, 0.f);
+        sts4(rec + kWorldD, dx, dy, dz, t1);
+        sts4(rec + kWorldInv, r.ix, r.iy, r.iz, 0.f);
+        if constexpr (!ANY) sts4(rec + kHit, __uint_as_float(0xFFFFFFFFu), 0.f, 0.f, 0.f);
+        if constexpr (RANGE) sts_u2(rec + kRange, __float_as_uint(t0), __float_as_uint(t1));
+        if constexpr (UV) sts_u2(rec + kRange + 8, 0u, 0u);
+        cur = S.n_inst > 0 ? 0u : kRefNone;  // TLAS root, an inner reference
+    }
+
+    // 2^-20 (|o| + R_top): the world ray is exact, so this covers only the
+    // rounding of the slab arithmetic at the top level.
+    static __device__ __forceinline__ float world_delta(const DevScene& S, float ox, float oy, float oz) {
+        return 9.5367431640625e-07f * (maxabs3(ox, oy, oz) + S.R_top);
+    }
+
+    __device__ __forceinline__ WRay world() const {
+        const float4 o = lds4(rec + kWorldO), d = lds4(rec + kWorldD);
+        return WRay{o.x, o.y, o.z, d.x, d.y, d.z};
+    }
+
+    // Far end of the interval in object space (s units, widened by the
+    // rounding of t - te).
+    static __device__ __forceinline__ float object_limit(float t, float te) {
+        return __fadd_rn(__fsub_rn(t, te), 1.9073486328125e-06f * (fabsf(t) + fabsf(te)));
+    }
+
+    __device__ __forceinline__ void put(int i, float t, uint32_t ref) {
+        if constexpr (ANY) {
+            if (i < STACK) sts_u(stk + 128u * (uint32_t)i, ref);
+            else deep[i - STACK] = ref;
+        } else {
+            if (i < STACK) sts_u2(stk + 256u * (uint32_t)i, ref, __float_as_uint(t));
+            else deep[i - STACK] = ((uint64_t)__float_as_uint(t) << 32) | ref;
+        }
+    }
+
+    // Pops an entry into cur unless it lies beyond the best hit.
+    __device__ __forceinline__ void pop() {
+        const int i = --sp;
+        if constexpr (ANY) {
+            cur = i < STACK ? lds_u(stk + 128u * (uint32_t)i) : deep[i - STACK];
+        } else {
+            uint2 e;
+            if (i < STACK) {
+                e = lds_u2(stk + 256u * (uint32_t)i);
+            } else {
+                const uint64_t v = deep[i - STACK];
+                e = make_uint2((uint32_t)v, (uint32_t)(v >> 32));
+            }
+            cur = __uint_as_float(e.y) <= lim ? e.x : kRefNone;
+        }
+    }
 
     // Pushes the hit children other than the one visited next and makes that
     // one current (nh > 0).  Closest hit: children sorted nearest first, the
@@ -514,161 +669,58 @@ struct Traversal {
             const int first = h0 ? 0 : (h1 ? 1 : (h2 ? 2 : 3));
 #pragma unroll
             for (int k = 3; k >= 0; --k)
-                if (t[k] < kInfF && k != first) stack[sp++] = ref[k];
+                if (t[k] < kInfF && k != first) put(sp++, t[k], ref[k]);
             cur = h0 ? ref[0] : (h1 ? ref[1] : (h2 ? ref[2] : ref[3]));
         } else {
 #pragma unroll
             for (int k = 3; k >= 1; --k)
-                if (k < nh) stack[sp++] = ((uint64_t)__float_as_uint(t[k]) << 32) | ref[k];
+                if (k < nh) put(sp++, t[k], ref[k]);
             cur = ref[0];
         }
     }
 
-    __device__ __forceinline__ void init(const DevScene& S, float ox, float oy, float oz, float dx,
-                                         float dy, float dz, float t0, float t1, uint32_t msteps,
-                                         TraceStats& st) {
-        tmin = t0;
-        tmax = t1;
-        h.t = t1;
-        h.inst = 0xFFFFFFFFu;
-        h.prim = 0xFFFFFFFFu;
-        h.u = h.v = 0.f;
-        h.slot = 0;
-        ++st.rays;
-        sp = 0;
-        inst_sp = -1;
-        node_base = S.tlas_base;
-        cur_inst = 0;
-        te = 0.f;
-        cur = 0;  // TLAS root, an inner reference
-        h_eps = 0.f;
-        have = S.n_inst > 0;
-        budget = msteps;
-        pleaf = 0;
-        setup_world(S, WRay{ox, oy, oz, dx, dy, dz});
-    }
-
-    // The world ray's box-test setup, widened by 2^-20 (|o| + R_top): the
-    // world ray is exact, so this covers only the rounding of the slab
-    // arithmetic at the top level.  Recomputed on every return to the TLAS
-    // rather than kept live: at 64 registers that shrinks the closest-hit
-    // kernel's spill stores from 500 to 384 bytes per thread.
-    __device__ __forceinline__ void setup_world(const DevScene& S, const WRay& w) {
-        setup_boxes(r, w.ox, w.oy, w.oz, w.dx, w.dy, w.dz,
-                    9.5367431640625e-07f * (maxabs3(w.ox, w.oy, w.oz) + S.R_top));
-    }
-
-    // far end of the interval in the current space (object space: s units,
-    // widened by the rounding of h.t - te)
-    __device__ __forceinline__ float limit() const {
-        return top() ? h.t
-                   : __fadd_rn(__fsub_rn(h.t, te), 1.9073486328125e-06f * (fabsf(h.t) + fabsf(te)));
-    }
-
-    template <class World>
-    __device__ __forceinline__ bool step(const DevScene& S, TraceStats& st, const World& world) {
-        if (have) {
-            if (!(cur & kRefLeaf)) {
-                if (budget == 0) {
-                    err |= kErrStepLimit;
-                    return false;
-                }
-                --budget;
-                ++st.nodes;
-                float t[4];
-                uint32_t ref[4];
-                const float lo = top() ? tmin : __fsub_rn(tmin, te);
-                const int nh = node_children<FETCH, !ANY>(S.nodes + node_base + cur, r, lo, limit(), t, ref);
-                if (nh == 0) {
-                    have = false;
-                } else {
-                    if (sp + nh - 1 > STACK) {
-                        err |= kErrStackOverflow;
-                        return false;
-                    }
-                    push_children(nh, t, ref);
-                    return true;
-                }
-            } else if (top()) {
-                enter_instance(S, st, world);
-                return true;
-            } else {
-                if (leaf(S, st, world)) return false;  // any hit found
-                have = false;
-            }
-        }
-        // pop
-        if (!top() && sp == inst_sp) {
-            inst_sp = -1;
-            node_base = S.tlas_base;
-            te = 0.f;
-            setup_world(S, world());
-        }
-        if (sp == 0) return false;
-        const uint64_t e = stack[--sp];
-        const float tn = ANY ? tmin : __uint_as_float((uint32_t)(e >> 32));
-        if (ANY || tn <= limit()) {
-            cur = (uint32_t)e;
-            have = true;
-        }
-        return true;
-    }
-
-    // ---- warp-synchronous phases (used by the persistent kernels) --------
     // A lane is in exactly one of: an inner node to test (wants_inner), a TLAS
     // leaf to enter (at_instance), a BLAS leaf to test (at_leaf: postponed or
     // current), or finished.
-
-    __device__ __forceinline__ bool wants_inner() const { return have && !(cur & kRefLeaf); }
-    __device__ __forceinline__ bool at_instance() const { return have && (cur & kRefLeaf) && top(); }
+    __device__ __forceinline__ bool wants_inner() const { return (int)cur >= 0; }
+    __device__ __forceinline__ bool at_instance() const { return (int)cur < 0 && cur != kRefNone && top(); }
     __device__ __forceinline__ bool at_leaf() const {
-        return pleaf != 0 || (have && (cur & kRefLeaf) && !top());
+        return pleaf != 0 || ((int)cur < 0 && cur != kRefNone && !top());
     }
-    __device__ __forceinline__ bool finished() const { return !have && pleaf == 0; }
+    // nothing left to visit (a quad may still wait), and the ray's end
+    __device__ __forceinline__ bool visited() const { return cur == kRefNone && pleaf == 0; }
+    __device__ __forceinline__ bool finished() const { return visited() && !pending; }
 
     __device__ __forceinline__ void stop(uint32_t e) {
         err |= e;
-        have = false;
+        cur = kRefNone;
         pleaf = 0;
         sp = 0;
+        pending = blocked = false;
     }
 
-    // Pops until cur holds an entry, the stack is empty, or the instance
+    // Pops until cur holds a reference, the stack is empty, or the instance
     // boundary is reached while a leaf of this instance is still postponed.
     // BLAS leaves met on the way are postponed (one at a time) so that the
     // lane keeps traversing inner nodes with the rest of its warp.
-    template <class World>
-    __device__ __forceinline__ void advance(const DevScene& S, const World& world) {
+    __device__ __forceinline__ void advance(const DevScene& S) {
         for (;;) {
-            if (have) {
-                if (pleaf == 0 && !top() && (cur & kRefLeaf)) {
-                    pleaf = cur;
-                    have = false;
-                } else {
-                    return;
-                }
+            if (cur != kRefNone) {
+                if (pleaf != 0 || top() || (int)cur >= 0) return;
+                pleaf = cur;
+                cur = kRefNone;
             }
-            if (!top() && sp == inst_sp) {
+            if (sp == inst_sp) {
                 if (pleaf) return;
-                inst_sp = -1;
-                node_base = S.tlas_base;
-                te = 0.f;
-                setup_world(S, world());
+                leave_instance(S);
             }
             if (sp == 0) return;
-            const uint64_t e = stack[--sp];
-            const float tn = ANY ? tmin : __uint_as_float((uint32_t)(e >> 32));
-            if (ANY || tn <= limit()) {
-                cur = (uint32_t)e;
-                have = true;
-            }
+            pop();
         }
     }
 
     // Tests the inner node cur and moves on (precondition: wants_inner()).
-    template <class World>
-    __device__ __forceinline__ void inner_step(const DevScene& S, TraceStats& st, int cap,
-                                               const World& world) {
+    __device__ __forceinline__ void inner_step(const DevScene& S, TraceStats& st, int cap) {
         if (budget == 0) {
             stop(kErrStepLimit);
             return;
@@ -677,10 +729,9 @@ struct Traversal {
         ++st.nodes;
         float t[4];
         uint32_t ref[4];
-        const float lo = top() ? tmin : __fsub_rn(tmin, te);
-        const int nh = node_children<FETCH, !ANY>(S.nodes + node_base + cur, r, lo, limit(), t, ref);
+        const int nh = node_children<Kind::FETCH, !ANY>(S.nodes + (size_t)(node_base + cur), r, lo, lim, t, ref);
         if (nh == 0) {
-            have = false;
+            cur = kRefNone;
         } else {
             if (sp + nh - 1 > cap) {
                 stop(kErrStackOverflow);
@@ -688,93 +739,95 @@ struct Traversal {
             }
             push_children(nh, t, ref);
         }
-        advance(S, world);
+        advance(S);
     }
 
-    // Tests one BLAS leaf (the postponed one first); returns true when an
-    // any-hit query is answered (precondition: at_leaf()).
-    template <class World>
-    __device__ __forceinline__ bool leaf_step(const DevScene& S, TraceStats& st, const World& world) {
-        if (pleaf) {
-            const uint32_t keep = cur;
-            cur = pleaf;
+    // Tests one BLAS leaf (the postponed one first; precondition: at_leaf()).
+    __device__ __forceinline__ void leaf_step(const DevScene& S, TraceStats& st) {
+        uint32_t ref = pleaf;
+        if (ref) {
             pleaf = 0;
-            const bool done = leaf(S, st, world);
-            cur = keep;
-            if (done) return true;
         } else {
-            if (leaf(S, st, world)) return true;
-            have = false;
+            ref = cur;
+            cur = kRefNone;
         }
-        advance(S, world);
-        return false;
+        if (leaf(S, st, ref)) {
+            answer();
+        } else {
+            advance(S);
+        }
     }
 
-    // Enters the instance of the TLAS leaf cur (precondition: at_instance()).
-    template <class World>
-    __device__ __forceinline__ void instance_step(const DevScene& S, TraceStats& st,
-                                                  const World& world) {
-        enter_instance(S, st, world);
+    __device__ __forceinline__ void answer() {
+        found = true;
+        cur = kRefNone;
+        pleaf = 0;
+        pending = blocked = false;
     }
 
-    // Moves the ray into the instance's object space.  The world point
-    // p = o + te d where the ray enters the instance's box and its offset
-    // p - c from the object origin are formed exactly as float pairs
-    // (two-product / two-sum), so the FP32 object-space origin W (p - c)
-    // carries an error proportional to the object's size only; the BLAS then
-    // works in s = t - te.
-    template <class World>
-    __device__ __forceinline__ void enter_instance(const DevScene& S, TraceStats& st,
-                                                   const World& world) {
-        cur_inst = cur & kRefIndexMask;
-        const WRay w = world();
-        const float wox = w.ox, woy = w.oy, woz = w.oz, wdx = w.dx, wdy = w.dy, wdz = w.dz;
-        const float4* ip = reinterpret_cast<const float4*>(S.inst + cur_inst);
+    // Moves the ray into the object space of the instance of the TLAS leaf cur
+    // (precondition: at_instance()).  The world point p = o + te d where the
+    // ray passes closest to the object origin and its offset p - c from that
+    // origin are formed exactly as float pairs (two-product / two-sum), so the
+    // FP32 object-space origin W (p - c) carries an error proportional to the
+    // object's size only; the BLAS then works in s = t - te.
+    __device__ __forceinline__ void instance_step(const DevScene& S, TraceStats& st) {
+        const uint32_t inst = cur & kRefIndexMask;
+        const float4* ip = reinterpret_cast<const float4*>(S.inst + inst);
         const float4 m0 = __ldg(ip), m1 = __ldg(ip + 1), m2 = __ldg(ip + 2), m3 = __ldg(ip + 3);
         // m0 = (c, R); m1 = (w0 w1 w2 w3); m2 = (w4 w5 w6 w7); m3 = (w8, node_base, quad_base, kappa)
+        const float4 wo = lds4(rec + kWorldO), wd = lds4(rec + kWorldD);
+        const float tmin_ = lo;  // at the top level
         // Re-centre where the ray passes closest to the object origin (never
         // before tmin), so the re-centred origin lies within the object's
         // reach; hits before that point have s < 0.  (Re-centring at the
         // instance box's entry distance instead needs that distance kept per
         // stack entry and per ray, and measured slower with more FP64
         // re-tests.)
+        float te;
         {
-            const float cx = __fsub_rn(m0.x, wox), cy = __fsub_rn(m0.y, woy), cz = __fsub_rn(m0.z, woz);
-            const float dd = __fmaf_rn(wdx, wdx, __fmaf_rn(wdy, wdy, __fmul_rn(wdz, wdz)));
-            const float tc = __fdiv_rn(__fmaf_rn(cx, wdx, __fmaf_rn(cy, wdy, __fmul_rn(cz, wdz))), dd);
-            te = (tc > tmin && tc < kInfF) ? tc : tmin;
+            const float cx = __fsub_rn(m0.x, wo.x), cy = __fsub_rn(m0.y, wo.y), cz = __fsub_rn(m0.z, wo.z);
+            const float dd = __fmaf_rn(wd.x, wd.x, __fmaf_rn(wd.y, wd.y, __fmul_rn(wd.z, wd.z)));
+            const float tc = __fdiv_rn(__fmaf_rn(cx, wd.x, __fmaf_rn(cy, wd.y, __fmul_rn(cz, wd.z))), dd);
+            te = (tc > tmin_ && tc < kInfF) ? tc : tmin_;
         }
         float exl, eyl, ezl;
-        const float ex = exact_offset(wox, wdx, te, m0.x, &exl);
-        const float ey = exact_offset(woy, wdy, te, m0.y, &eyl);
-        const float ez = exact_offset(woz, wdz, te, m0.z, &ezl);
+        const float ex = exact_offset(wo.x, wd.x, te, m0.x, &exl);
+        const float ey = exact_offset(wo.y, wd.y, te, m0.y, &eyl);
+        const float ez = exact_offset(wo.z, wd.z, te, m0.z, &ezl);
         const float rox = __fmaf_rn(m1.x, ex, __fmaf_rn(m1.y, ey, __fmaf_rn(m1.z, ez,
                               __fmaf_rn(m1.x, exl, __fmaf_rn(m1.y, eyl, __fmul_rn(m1.z, ezl))))));
         const float roy = __fmaf_rn(m1.w, ex, __fmaf_rn(m2.x, ey, __fmaf_rn(m2.y, ez,
                               __fmaf_rn(m1.w, exl, __fmaf_rn(m2.x, eyl, __fmul_rn(m2.y, ezl))))));
         const float roz = __fmaf_rn(m2.z, ex, __fmaf_rn(m2.w, ey, __fmaf_rn(m3.x, ez,
                               __fmaf_rn(m2.z, exl, __fmaf_rn(m2.w, eyl, __fmul_rn(m3.x, ezl))))));
-        float fdx, fdy, fdz;
-        object_dir(m1, m2, m3, wdx, wdy, wdz, fdx, fdy, fdz);
+        // W d: the world direction in object space
+        const float fdx = __fmaf_rn(m1.x, wd.x, __fmaf_rn(m1.y, wd.y, __fmul_rn(m1.z, wd.z)));
+        const float fdy = __fmaf_rn(m1.w, wd.x, __fmaf_rn(m2.x, wd.y, __fmul_rn(m2.y, wd.z)));
+        const float fdz = __fmaf_rn(m2.z, wd.x, __fmaf_rn(m2.w, wd.y, __fmul_rn(m3.x, wd.z)));
         node_base = __float_as_uint(m3.y);
         // 2^-22 (kappa + 2) (|o''| + R): rounding of W, of W (p - c), of W d and
-        // of the slab and shear arithmetic, with a factor-two margin
-        const float delta = __fmul_rn(2.384185791015625e-07f * (m3.w + 2.0f),
-                                      maxabs3(rox, roy, roz) + m0.w);
-        setup_boxes(r, rox, roy, roz, fdx, fdy, fdz, delta);
+        // of the shear arithmetic, with a factor-two margin
+        setup_boxes(r, rox, roy, roz, fdx, fdy, fdz,
+                    __fmul_rn(2.384185791015625e-07f * (m3.w + 2.0f), maxabs3(rox, roy, roz) + m0.w));
+        sts1(rec + kWorldO + 12, te);
+        sts4(rec + kObjD, fdx, fdy, fdz, m3.z);
+        sts_u(rec + kCurInst, inst);
+        lim = object_limit(ANY ? tmax() : wd.w, te);
+        lo = __fsub_rn(tmin_, te);
         inst_sp = sp;
         ++st.insts;
         cur = 0;
     }
 
-    // W d: the world direction in the instance's object space (m1..m3 hold
-    // W row by row).  Recomputed at each leaf rather than kept per ray.
-    static __device__ __forceinline__ void object_dir(const float4& m1, const float4& m2,
-                                                      const float4& m3, float wdx, float wdy,
-                                                      float wdz, float& fdx, float& fdy, float& fdz) {
-        fdx = __fmaf_rn(m1.x, wdx, __fmaf_rn(m1.y, wdy, __fmul_rn(m1.z, wdz)));
-        fdy = __fmaf_rn(m1.w, wdx, __fmaf_rn(m2.x, wdy, __fmul_rn(m2.y, wdz)));
-        fdz = __fmaf_rn(m2.z, wdx, __fmaf_rn(m2.w, wdy, __fmul_rn(m3.x, wdz)));
+    // Back to the world-space ray and the top level.
+    __device__ __forceinline__ void leave_instance(const DevScene& S) {
+        const float4 o = lds4(rec + kWorldO), inv = lds4(rec + kWorldInv);
+        r = RaySetup{o.x, o.y, o.z, inv.x, inv.y, inv.z, 2.0f * world_delta(S, o.x, o.y, o.z)};
+        lo = tmin();
+        lim = ANY ? tmax() : lds1(rec + kWorldD + 12);
+        inst_sp = -1;
+        node_base = S.tlas_base;
     }
 
     // (o + te d) - c per axis as a float pair hi + *lo, exact up to the
@@ -792,109 +845,155 @@ struct Traversal {
         return hi;
     }
 
-    // The closest hit's original quad index, looked up from its slot once the
-    // ray has ended (ties during traversal read it on demand), so it is not
-    // live through the traversal.  Any-hit results carry no quad index.
-    __device__ __forceinline__ void resolve_prim(const DevScene& S) {
-        if constexpr (!ANY) h.prim = h.inst == 0xFFFFFFFFu ? 0xFFFFFFFFu : __ldg(S.prim + h.slot);
+    // The hit, read back once the ray has ended.  The original quad index is
+    // looked up from the slot here (any-hit results carry none).
+    __device__ __forceinline__ Hit hit(const DevScene& S) const {
+        Hit h;
+        const float4 a = lds4(rec + kHit);
+        h.t = lds1(rec + kWorldD + 12);
+        h.inst = __float_as_uint(a.x);
+        h.slot = __float_as_uint(a.y);
+        h.prim = h.inst == 0xFFFFFFFFu ? 0xFFFFFFFFu : __ldg(S.prim + h.slot);
+        h.u = h.v = 0.f;
+        if constexpr (UV) {
+            h.u = lds1(rec + kRange + 8);
+            h.v = lds1(rec + kRange + 12);
+        }
+        return h;
     }
 
-    // Tests the quads of the current BLAS leaf; returns true when an any-hit
-    // query is answered.  Two candidates whose FP32 distances are within
-    // their error bounds of each other are ordered by their FP64 distances.
-    template <class World>
-    __device__ __forceinline__ bool leaf(const DevScene& S, TraceStats& st, const World& world) {
-        Shear sh;
-        {
-            const float4* mp = reinterpret_cast<const float4*>(S.inst + cur_inst);
-            const float4 m1 = __ldg(mp + 1), m2 = __ldg(mp + 2), m3 = __ldg(mp + 3);
-            const WRay w = world();
-            float dx, dy, dz;
-            object_dir(m1, m2, m3, w.dx, w.dy, w.dz, dx, dy, dz);
-            sh = make_shear(r, dx, dy, dz);
-        }
-        const uint32_t first = cur & kRefIndexMask;
-        const uint32_t cnt = ((cur >> 27) & 0xFu) + 1u;
-        const float smin = __fsub_rn(tmin, te);
-        const float smax = __fsub_rn(tmax, te);
-        const InstDev* ip = S.inst + cur_inst;
-        const InstDev64* ip64 = S.inst64 + cur_inst;
-        // read here (an L1 hit after the instance entry) rather than kept
-        // live for the whole BLAS traversal
-        const uint32_t quad_base = __ldg(&ip->quad_base);
-        for (uint32_t k = 0; k < cnt; ++k) {
-            const uint32_t slot = quad_base + first + k;
-            float tt, uu, vv;
-            double t64;
-            int ex64;
+    // Makes (t, inst, slot) the best hit.
+    __device__ __forceinline__ void keep(float t, float te, uint32_t inst, uint32_t slot, float eps, float u,
+                                         float v) {
+        sts1(rec + kWorldD + 12, t);
+        sts_u2(rec + kHit, inst, slot);
+        sts1(rec + kHit + 8, eps);
+        if constexpr (UV) sts_u2(rec + kRange + 8, __float_as_uint(u), __float_as_uint(v));
+        lim = top() ? t : object_limit(t, te);
+    }
+
+    // Tests the quads of BLAS leaf ref; returns true when an any-hit query is
+    // answered.  A quad that FP32 cannot decide, or whose distance is within
+    // its error bound of the best hit's, waits for resolve(); while one waits
+    // the traversal goes on, and a second one puts the rest of its leaf back.
+    __device__ __forceinline__ bool leaf(const DevScene& S, TraceStats& st, uint32_t ref) {
+        const float4 od = lds4(rec + kObjD);
+        const Shear sh = make_shear(r, od.x, od.y, od.z);
+        const float te = lds1(rec + kWorldO + 12);
+        const float t1 = tmax();
+        uint32_t slot = __float_as_uint(od.w) + (ref & kRefIndexMask);
+        for (;;) {
+            QuadHit q;
+            const QuadResult res = quad_test(sh, 0.5f * r.delta2, S.quads + slot, lo, __fsub_rn(t1, te), q);
+            if (res != kQuadMiss) {
+                const float t = __fadd_rn(q.s, te);
+                bool wait = res == kQuadUncertain;
+                float u = __int_as_float(0x7fffffff), v = 0.f;
+                if constexpr (ANY) {
+                    if (!wait && t > tmin() && t < t1) return true;
+                } else if (!wait && t > tmin() && t < t1) {
+                    const float ht = lds1(rec + kWorldD + 12);
+                    const float4 hr = lds4(rec + kHit);
+                    const uint32_t inst = lds_u(rec + kCurInst);
+                    const uint32_t hinst = __float_as_uint(hr.x), hslot = __float_as_uint(hr.y);
+                    wait = fabsf(t - ht) <= fmaxf(sh.eps_t, hr.z) && hinst != 0xFFFFFFFFu &&
+                           !(hslot == slot && hinst == inst);
+                    if (wait || t <= ht) {
+                        if constexpr (UV) {
+                            u = __fdiv_rn(q.u_num, q.det);
+                            v = __fdiv_rn(q.v_num, q.det);
+                        } else {
+                            u = 0.f;
+                        }
+                        if (!wait && (t < ht || before(S, inst, slot, hinst, hslot)))
+                            keep(t, te, inst, slot, sh.eps_t, u, v);
+                    }
+                }
+                if (wait) {
+                    if (pending) {
+                        blocked = true;
+                        pleaf = ref;
+                        return false;
+                    }
+                    pending = true;
+                    const float inst = lds1(rec + kCurInst);
+                    if constexpr (ANY) {
+                        sts_u2(rec + kPend, slot, __float_as_uint(inst));
+                    } else {
+                        sts4(rec + kPend, __uint_as_float(slot), inst, u, v);
+                        sts1(rec + kPendEps, sh.eps_t);
+                    }
+                }
+            }
             ++st.quads;
-            if (!quad_test(r, sh, S.quads + slot, ip, ip64, world, smin, smax, tmin, &tt, &t64, &uu,
-                           &vv, &ex64, &st.fallbacks))
-                continue;
-            if (!ex64) tt = __fadd_rn(tt, te);
-            if (!(tt > tmin && tt < tmax)) continue;
-            if (ANY) {
-                h.t = tt;
-                h.inst = cur_inst;
-                h.slot = slot;
-                return true;
-            }
-            const float eps = fmaxf(sh.eps_t, h_eps);
-            if (h.inst != 0xFFFFFFFFu && fabsf(tt - h.t) <= eps &&
-                !(h.slot == slot && h.inst == cur_inst)) {
-                // near tie with the current best: decide on FP64 distances
-                ++st.fallbacks;
-                const WRay w = world();
-                const double tb = exact_t(S, h.inst, h.slot, w.ox, w.oy, w.oz, w.dx, w.dy, w.dz, tmin);
-                const double tc =
-                    ex64 ? t64 : exact_t(S, cur_inst, slot, w.ox, w.oy, w.oz, w.dx, w.dy, w.dz, tmin);
-                const bool better =
-                    tc < tb || (tc == tb && (cur_inst < h.inst ||
-                                             (cur_inst == h.inst &&
-                                              __ldg(S.prim + slot) < __ldg(S.prim + h.slot))));
-                if (better && tc < (double)tmax) {
-                    h.t = (float)tc;
-                    h.inst = cur_inst;
-                    if constexpr (UV) {
-                        h.u = uu;
-                        h.v = vv;
-                    }
-                    h.slot = slot;
-                    h_eps = sh.eps_t;
-                }
-                continue;
-            }
-            if (tt < h.t) {
-                h.t = tt;
-                h.inst = cur_inst;
-                if constexpr (UV) {
-                    h.u = uu;
-                    h.v = vv;
-                }
-                h.slot = slot;
-                h_eps = ex64 ? 0.f : sh.eps_t;
-            } else if (tt == h.t) {
-                if (cur_inst < h.inst ||
-                    (cur_inst == h.inst && __ldg(S.prim + slot) < __ldg(S.prim + h.slot))) {
-                    h.inst = cur_inst;
-                    if constexpr (UV) {
-                        h.u = uu;
-                        h.v = vv;
-                    }
-                    h.slot = slot;
-                    h_eps = ex64 ? 0.f : sh.eps_t;
-                }
-            }
+            if ((ref & 0x78000000u) == 0) return false;
+            // the rest of the leaf: one item further, one fewer
+            ref -= (1u << 27) - 1u;
+            ++slot;
         }
-        return false;
+    }
+
+    // Decides the waiting quad in FP64: two candidates whose distances are
+    // within their error bounds of each other are ordered by their FP64
+    // distances, equal distances by (instance, quad).  Rare, and slow on this
+    // GPU (FP64 runs at 1/64 of FP32, and a warp pays for one lane what it
+    // pays for all), so the caller gathers lanes for it.
+    __device__ __forceinline__ void resolve(const DevScene& S, TraceStats& st) {
+        pending = blocked = false;
+        ++st.fallbacks;
+        const WRay w = world();
+        const float t0 = tmin(), t1 = tmax();
+        if constexpr (ANY) {
+            const uint2 p = lds_u2(rec + kPend);
+            const float t = (float)quad_test64(S.inst + p.y, S.inst64 + p.y, S.quads + p.x, w, t0).t;
+            if (t > t0 && t < t1) answer();
+        } else {
+            const float4 p = lds4(rec + kPend);
+            const uint32_t slot = __float_as_uint(p.x), inst = __float_as_uint(p.y);
+            const Hit64 c = quad_test64(S.inst + inst, S.inst64 + inst, S.quads + slot, w, t0);
+            const float t = (float)c.t;
+            if (!(t > t0 && t < t1 && c.t < (double)t1)) return;
+            const float ht = lds1(rec + kWorldD + 12);
+            const float4 hr = lds4(rec + kHit);
+            const uint32_t hinst = __float_as_uint(hr.x), hslot = __float_as_uint(hr.y);
+            float eps = lds1(rec + kPendEps);
+            bool better;
+            if (fabsf(t - ht) <= fmaxf(eps, hr.z) && hinst != 0xFFFFFFFFu && !(hslot == slot && hinst == inst)) {
+                ++st.fallbacks;
+                const double tb = quad_test64(S.inst + hinst, S.inst64 + hinst, S.quads + hslot, w, t0).t;
+                better = c.t < tb || (c.t == tb && before(S, inst, slot, hinst, hslot));
+            } else {
+                better = t < ht || (t == ht && before(S, inst, slot, hinst, hslot));
+                eps = 0.f;
+            }
+            const bool decided = p.z == p.z;  // FP32 hit: its own (u, v)
+            if (better)
+                keep(t, lds1(rec + kWorldO + 12), inst, slot, eps, decided ? p.z : c.u, decided ? p.w : c.v);
+        }
+    }
+
+    // Order of two hits at the same distance.
+    static __device__ __forceinline__ bool before(const DevScene& S, uint32_t inst, uint32_t slot,
+                                                  uint32_t hinst, uint32_t hslot) {
+        return inst < hinst || (inst == hinst && __ldg(S.prim + slot) < __ldg(S.prim + hslot));
     }
 };
 
+// Shared memory of a block of `threads` threads, and a warp's part of it.
+template <class Kind>
+constexpr size_t traversal_bytes(int threads) {
+    return (size_t)threads * Kind::kLaneBytes;
+}
+template <class Kind>
+__device__ __forceinline__ uint32_t traversal_base() {
+    extern __shared__ __align__(512) unsigned char qrt_smem[];
+    return (uint32_t)__cvta_generic_to_shared(qrt_smem) + (threadIdx.x >> 5) * 32u * Kind::kLaneBytes;
+}
+
 // Persistent warp-synchronous traversal loop over work items [0, count)
 // claimed from *cursor.  Each lane holds one ray; start(k) sets item k up in
-// T (T.init), done() consumes the finished ray in T, world() gives the world
-// ray of the lane's current item; a ray may use cap (<=
-// STACK) stack entries, a launch-wide value passed down rather than kept per
+// T (T.init), done() consumes the finished ray in T; a ray may use cap (<=
+// kMaxStack) stack entries, a launch-wide value passed down rather than kept per
 // ray.  A lane claims `batch`
 // items at a time; the idle lanes of a warp claim theirs with one atomic
 // (warp-aggregated), so a launch costs about one atomic per warp and
@@ -904,17 +1003,18 @@ struct Traversal {
 // groups) until few lanes are left with an inner node, then lanes enter
 // instances or test one leaf each.  Finished lanes refill
 // immediately, so no lane waits for the slowest ray of its warp.
-template <bool ANY, int STACK, int FETCH, bool UV, class Idx, class Start, class Done, class World>
-__device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<ANY, STACK, FETCH, UV>& T,
-                                                 TraceStats& st, Idx* cursor, Idx count,
-                                                 uint32_t batch, int cap, Start start, Done done,
-                                                 World world) {
+template <class Kind, class Idx, class Start, class Done>
+__device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Kind>& T, TraceStats& st,
+                                                 Idx* cursor, Idx count, uint32_t batch, int cap,
+                                                 Start start, Done done) {
     const unsigned FULL = 0xFFFFFFFFu;
     const unsigned lane = threadIdx.x & 31u;
     // [next, end) = this lane's claimed items not yet started; a claim that
     // lands at or past count leaves end == count, which ends the claiming
     bool busy = false;
     Idx next = 0, end = 0;
+    int waited = 0;  // iterations lanes have sat with nothing left but a waiting quad
+    T.bind(traversal_base<Kind>());
     for (;;) {
         const bool need = !busy && next >= end && end < count;
         const unsigned want = __ballot_sync(FULL, need);
@@ -938,13 +1038,13 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<AN
             // enter it together and go on with the inner nodes of its BLAS
             // in this phase, instead of idling until the next outer
             // iteration.  Each such step enters at least eight instances.
-            const bool wt = busy && T.at_instance();
+            const bool wt = T.at_instance();
             const unsigned bt = __ballot_sync(FULL, wt);
             if (__popc(bt) >= 8) {
-                if (wt) T.instance_step(S, st, world);
+                if (wt) T.instance_step(S, st);
                 continue;
             }
-            const bool w = busy && T.wants_inner();
+            const bool w = T.wants_inner();
             const unsigned bw = __ballot_sync(FULL, w);
             if (!bw) break;
             // Leave the inner-node phase early once the lanes still in it are
@@ -955,19 +1055,30 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<AN
             // outer iteration makes progress.
             const unsigned bo = __ballot_sync(FULL, busy && !w);
             if (bo && 2 * __popc(bw) <= __popc(bo)) break;
-            if (w) T.inner_step(S, st, cap, world);
+            if (w) T.inner_step(S, st, cap);
         }
         if (busy) {
             if (T.at_instance()) {
-                T.instance_step(S, st, world);
+                T.instance_step(S, st);
             } else if (T.at_leaf()) {
-                if (T.leaf_step(S, st, world)) {
-                    T.have = false;
-                    T.pleaf = 0;
-                }
+                T.leaf_step(S, st);
             }
-            if (T.finished() || (ANY && T.h.inst != 0xFFFFFFFFu)) {
-                T.resolve_prim(S);
+        }
+        // Waiting quads are decided together: when a lane cannot go on, when
+        // eight wait, or when the lanes that wait for nothing else have cost
+        // about as much as the FP64 test does.
+        const unsigned bp = __ballot_sync(FULL, T.pending);
+        if (bp) {
+            const bool idle = T.pending && T.visited();
+            waited += __popc(__ballot_sync(FULL, idle));
+            if (__popc(bp) >= 8 || waited >= 16 || __any_sync(FULL, T.blocked) ||
+                !__any_sync(FULL, busy && !idle)) {
+                if (T.pending) T.resolve(S, st);
+                waited = 0;
+            }
+        }
+        if (busy) {
+            if (T.finished()) {
                 done();
                 busy = false;
             }
@@ -975,22 +1086,31 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<AN
     }
 }
 
-// Closest hit (ANY = false) or any hit (ANY = true) of the world ray, run to
-// completion.  Returns device error bits (0 = fine); h holds the best hit
-// found (inst = 0xFFFFFFFF if none).
-template <bool ANY, int STACK, int FETCH>
+// Closest hit or any hit (Kind::ANY) of the world ray, run to completion by
+// one thread.  Returns device error bits (0 = fine); a closest hit is left in
+// *h (inst = 0xFFFFFFFF if none), an any-hit answer in *found.
+template <class Kind>
 __device__ __forceinline__ uint32_t trace_ray(const DevScene& S, float wox, float woy, float woz,
-                                              float wdx, float wdy, float wdz, float tmin,
-                                              float tmax, uint32_t max_steps, Hit& h,
+                                              float wdx, float wdy, float wdz, float tmin, float tmax,
+                                              uint32_t max_steps, int cap, Hit* h, bool* found,
                                               TraceStats& st) {
-    Traversal<ANY, STACK, FETCH> T;
-    T.err = 0;
+    Traversal<Kind> T;
+    T.bind(traversal_base<Kind>());
     T.init(S, wox, woy, woz, wdx, wdy, wdz, tmin, tmax, max_steps, st);
-    const auto world = [=] { return WRay{wox, woy, woz, wdx, wdy, wdz}; };
-    while (T.step(S, st, world)) {
+    while (!T.finished()) {
+        if (T.blocked || T.visited())
+            T.resolve(S, st);
+        else if (T.wants_inner())
+            T.inner_step(S, st, cap);
+        else if (T.at_instance())
+            T.instance_step(S, st);
+        else
+            T.leaf_step(S, st);
     }
-    T.resolve_prim(S);
-    h = T.h;
+    if constexpr (Kind::ANY)
+        *found = T.found;
+    else
+        *h = T.hit(S);
     return T.err;
 }
 

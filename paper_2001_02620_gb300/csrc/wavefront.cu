@@ -118,8 +118,7 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
     const uint32_t* queue = ANY ? A.B.qs : A.B.q[depth & 1];
     const uint32_t batch = A.batch;
     TraceStats st{0, 0, 0, 0, 0, 0};
-    Traversal<ANY, kMaxStack, FETCH, UV> T;
-    T.err = 0;  // accumulated over this thread's rays
+    Traversal<WaveKind<ANY, UV, FETCH, OCC>> T;
     uint32_t j = 0;
     // any-hit entries of key-light shadow rays carry kLightRay
     auto start_ray = [&](uint32_t k) {
@@ -134,9 +133,7 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
                        A.P.max_steps, st);
             }
         } else {
-            // path rays span (0, inf) (the spawn point is offset off the
-            // surface): constant bounds fold into the traversal instead of
-            // occupying two registers per ray
+            // path rays span (0, inf) (the spawn point is offset off the surface)
             const float4 o = A.B.ray_o[j], d = A.B.ray_d[j];
             T.init(A.S, o.x, o.y, o.z, d.x, d.y, d.z, 0.f, kInfF, A.P.max_steps, st);
         }
@@ -148,7 +145,7 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
         }
         if (ANY) {
             const bool light = j & kLightRay;
-            if (T.h.inst == 0xFFFFFFFFu) {
+            if (!T.found) {
                 if (light) {
                     // the sun's shadow ray of the same vertex may add into L
                     // in this launch: flag the term, fold_light adds it later
@@ -168,26 +165,12 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
                     2u << (2 * (depth - 1));
             }
         } else {
-            A.B.hit[j] = make_uint4(__float_as_uint(T.h.t), T.h.inst, T.h.prim, T.h.slot);
-            if constexpr (UV) A.B.hit_uv[j] = make_float2(T.h.u, T.h.v);
+            const Hit h = T.hit(A.S);
+            A.B.hit[j] = make_uint4(__float_as_uint(h.t), h.inst, h.prim, h.slot);
+            if constexpr (UV) A.B.hit_uv[j] = make_float2(h.u, h.v);
         }
     };
-    // the world ray is read back from the queue buffers where the traversal
-    // needs it, not kept live per lane
-    auto world_ray = [&]() {
-        if (ANY) {
-            const float4 o = __ldg(A.B.sray_o + (j & ~kLightRay));
-            if (j & kLightRay) {
-                const float4 ld = __ldg(A.B.lray_d + (j & ~kLightRay));
-                return WRay{o.x, o.y, o.z, ld.x, ld.y, ld.z};
-            }
-            return WRay{o.x, o.y, o.z, A.P.sun_l[0], A.P.sun_l[1], A.P.sun_l[2]};
-        }
-        const float4 o = __ldg(A.B.ray_o + j), d = __ldg(A.B.ray_d + j);
-        return WRay{o.x, o.y, o.z, d.x, d.y, d.z};
-    };
-    persistent_trace<ANY, kMaxStack, FETCH>(A.S, T, st, fetch, count, batch, stack_cap, start_ray,
-                                            finish_ray, world_ray);
+    persistent_trace(A.S, T, st, fetch, count, batch, stack_cap, start_ray, finish_ray);
     if (T.err) atomicOr(A.S.err, T.err);
     if constexpr (STATS) add_stats(A.stats + (ANY ? 6 : 0), st);
 }
@@ -370,9 +353,11 @@ template <bool ANY, int FETCH, int OCC, bool STATS, bool UV>
 static cudaError_t launch_wave_trace_v(const WaveArgs& A, int depth, const Tune& t, int sm_count,
                                        cudaStream_t s) {
     static ResidentBlocks resident;
-    const int per_sm = t.blocks_per_sm > 0 ? t.blocks_per_sm
-                                           : resident.get(wave_trace<ANY, FETCH, OCC, STATS, UV>, t.block);
-    wave_trace<ANY, FETCH, OCC, STATS, UV><<<(unsigned)(sm_count * per_sm), t.block, 0, s>>>(
+    const size_t smem = traversal_bytes<WaveKind<ANY, UV, FETCH, OCC>>(t.block);
+    const int per_sm = t.blocks_per_sm > 0
+                           ? t.blocks_per_sm
+                           : resident.get(wave_trace<ANY, FETCH, OCC, STATS, UV>, t.block, smem);
+    wave_trace<ANY, FETCH, OCC, STATS, UV><<<(unsigned)(sm_count * per_sm), t.block, smem, s>>>(
         A, depth, t.stack);
     return cudaGetLastError();
 }
