@@ -420,7 +420,7 @@ struct Collapser {
                     err = "item index beyond 2^27 within one object";
                     return -1;
                 }
-                ref[i] = leaf_ref(first, c.count);
+                ref[i] = leaf_holds_id ? instance_ref(first) : leaf_ref(first, c.count);
             } else {
                 int64_t k = emit(ch[i], depth + 1);
                 if (k < 0) return -1;

@@ -33,9 +33,19 @@ struct ResidentBlocks {
         return n;
     }
 
+    // Lets a block take more than the default 48 KB.  The setting belongs to
+    // the current context and costs a fraction of a microsecond, so every
+    // launch that needs it makes it.
+    template <class Kernel>
+    static cudaError_t allow(Kernel kernel, size_t smem) {
+        if (smem <= 48 * 1024) return cudaSuccess;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
+
     template <class Kernel>
     static int query(Kernel kernel, int block, size_t smem) {
         int n = 0;
+        allow(kernel, smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block, smem);
         return n < 1 ? 1 : n;
     }

@@ -227,7 +227,7 @@ __host__ __device__ inline bool emit_wide(uint32_t b, uint32_t wide, uint32_t n,
         cb[i] = child_box(c[i], lbox, ibox);
         if ((c[i] & kLeafBit) && (c[i] & ~kLeafBit) >= n) return false;
         if (c[i] & kLeafBit) {
-            q.ref[i] = leaf_ref(ids[c[i] & ~kLeafBit], 1);  // a TLAS leaf holds one instance
+            q.ref[i] = instance_ref(ids[c[i] & ~kLeafBit]);  // a TLAS leaf holds one instance
         } else {
 #ifdef __CUDA_ARCH__
             const uint32_t pos = atomicAdd(next_count, 1u);
@@ -520,7 +520,7 @@ bool build_tlas_lbvh(const std::vector<FBox>& inst_boxes, bool on_device, TlasRe
             }
     if (n == 1) {  // a root with one leaf
         QNode q;
-        q.ref[0] = leaf_ref(0, 1);
+        q.ref[0] = instance_ref(0);
         for (int i = 1; i < 4; ++i) q.ref[i] = kRefNone;
         quantize_node(q, inst_boxes.data(), 1);
         out.nodes.push_back(q);

@@ -105,8 +105,9 @@ QRT_HD inline FBox child_bounds(const QNode& q, int i) {
 QRT_HD inline uint32_t leaf_ref(uint32_t first, uint32_t count) {
     return kRefLeaf | ((count - 1u) << 27) | first;
 }
+QRT_HD inline uint32_t instance_ref(uint32_t inst) { return kRefInstance | inst; }
 QRT_HD inline bool is_inner(uint32_t ref) { return !(ref & kRefLeaf); }
-QRT_HD inline uint32_t leaf_count(uint32_t ref) { return ((ref >> 27) & 0xFu) + 1u; }
+QRT_HD inline uint32_t leaf_count(uint32_t ref) { return ((ref >> 27) & 0x7u) + 1u; }
 QRT_HD inline uint32_t leaf_first(uint32_t ref) { return ref & kRefIndexMask; }
 
 }  // namespace qrt

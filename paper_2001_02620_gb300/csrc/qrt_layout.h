@@ -34,16 +34,18 @@ struct alignas(64) QNode {
 };
 static_assert(sizeof(QNode) == 64, "QNode must be 64 bytes");
 
-constexpr uint32_t kMaxLeaf = 16;
+constexpr uint32_t kMaxLeaf = 8;
 
-// Stack/child reference: bit 31 = leaf; a leaf keeps (count-1) in bits 27..30
-// and its first item in bits 0..26 (local quad slot, or instance at the top
-// level).  An inner reference is a node index local to its tree.  kRefNone
-// is no leaf: a leaf of 16 items cannot start at the last index there is.
+// Stack/child reference.  Inner node: its index, local to its tree.  BLAS
+// leaf: bit 31, (count-1) in bits 27..29, first local quad slot in bits 0..26.
+// TLAS leaf: bits 31 and 30, the instance.  kRefNone is no leaf: eight quads
+// cannot start at the last slot there is.  One unsigned comparison tells each
+// kind from the others.
 constexpr uint32_t kRefLeaf = 0x80000000u;
+constexpr uint32_t kRefInstance = 0xC0000000u;
 constexpr uint32_t kRefIndexMask = 0x07FFFFFFu;
 constexpr uint32_t kMaxLocalIndex = kRefIndexMask;
-constexpr uint32_t kRefNone = 0xFFFFFFFFu;
+constexpr uint32_t kRefNone = 0xBFFFFFFFu;
 
 struct alignas(16) QuadDev {
     float v[12];  // v0, v1, v2, v3 as packed float3

@@ -291,23 +291,24 @@ cudaError_t launch_render(const RenderArgs& A, const Tune& t, int sm_count, cuda
     const dim3 g((unsigned)grid), b((unsigned)t.block);
     const bool s32 = t.stack <= 32, f32 = t.fetch == 32;
     const size_t m = traversal_bytes<PathRay<32>>(t.block);
+    cudaError_t e = cudaSuccess;
+#define QRT_RENDER(STACK, FETCH, ADJ)                                                             \
+    if ((e = ResidentBlocks::allow(render_kernel<STACK, FETCH, ADJ>, m)) != cudaSuccess) return e; \
+    render_kernel<STACK, FETCH, ADJ><<<g, b, m, s>>>(A)
     if (adj) {
         if (s32) {
-            if (f32) render_kernel<32, 32, true><<<g, b, m, s>>>(A);
-            else render_kernel<32, 16, true><<<g, b, m, s>>>(A);
+            if (f32) { QRT_RENDER(32, 32, true); } else { QRT_RENDER(32, 16, true); }
         } else {
-            if (f32) render_kernel<64, 32, true><<<g, b, m, s>>>(A);
-            else render_kernel<64, 16, true><<<g, b, m, s>>>(A);
+            if (f32) { QRT_RENDER(64, 32, true); } else { QRT_RENDER(64, 16, true); }
         }
     } else {
         if (s32) {
-            if (f32) render_kernel<32, 32, false><<<g, b, m, s>>>(A);
-            else render_kernel<32, 16, false><<<g, b, m, s>>>(A);
+            if (f32) { QRT_RENDER(32, 32, false); } else { QRT_RENDER(32, 16, false); }
         } else {
-            if (f32) render_kernel<64, 32, false><<<g, b, m, s>>>(A);
-            else render_kernel<64, 16, false><<<g, b, m, s>>>(A);
+            if (f32) { QRT_RENDER(64, 32, false); } else { QRT_RENDER(64, 16, false); }
         }
     }
+#undef QRT_RENDER
     return cudaGetLastError();
 }
 

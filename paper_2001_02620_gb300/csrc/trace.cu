@@ -2,6 +2,8 @@
 // a grid of SMs x resident blocks running the warp-synchronous traversal loop
 // (persistent_trace); each lane claims `batch` rays at a time from a global
 // cursor and starts its next ray as soon as its own is done.
+#include <algorithm>
+
 #include "launch.h"
 #include "traverse.cuh"
 
@@ -10,23 +12,20 @@ namespace qrt {
 // Work counters are kept only in the STATS variant (dead code elsewhere).
 template <bool ANY, int FETCH, int OCC, bool STATS>
 __global__ void __maxnreg__(occupancy_regs(OCC)) trace_kernel(const DevScene S, const float4* __restrict__ rays,
-                                                       uint64_t n, uint4* __restrict__ hits,
+                                                       uint32_t n, uint64_t first, uint4* __restrict__ hits,
                                                        uint32_t* __restrict__ occ, uint32_t max_steps,
-                                                       unsigned long long* cursor, uint32_t batch,
+                                                       uint32_t* cursor, uint32_t batch,
                                                        unsigned long long* stats, int stack_cap) {
     TraceStats st{0, 0, 0, 0, 0, 0};
     Traversal<QueryKind<ANY, FETCH, OCC>> T;
-    uint64_t i = 0;
-    auto start_ray = [&](unsigned long long k) {
-        i = k;
-        const float4 a = __ldg(rays + 2 * i), b = __ldg(rays + 2 * i + 1);
+    auto start_ray = [&](uint32_t i) {
+        const float4 a = __ldg(rays + 2 * (size_t)i), b = __ldg(rays + 2 * (size_t)i + 1);
         T.init(S, a.x, a.y, a.z, b.x, b.y, b.z, a.w, b.w, max_steps, st);
     };
-    auto finish_ray = [&]() {
-        if (T.err) {  // the first affected ray is reported
-            atomicOr(S.err, T.err);
-            atomicMin(S.err + 1, (uint32_t)min(i, (uint64_t)0xFFFFFFFEu));
-            T.err = 0;
+    auto finish_ray = [&](uint32_t i) {
+        if (T.error()) {  // the first affected ray is reported
+            atomicOr(S.err, T.error());
+            atomicMin(S.err + 1, (uint32_t)min(first + i, (uint64_t)0xFFFFFFFEu));
         }
         if (ANY) {
             if (T.found) atomicOr(occ + (i >> 5), 1u << (i & 31));
@@ -38,9 +37,11 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) trace_kernel(const DevScene S, 
             hits[i] = make_uint4(__float_as_uint(h.t), h.inst, h.prim, uv);
         }
     };
-    persistent_trace(S, T, st, cursor, (unsigned long long)n, batch, stack_cap, start_ray, finish_ray);
+    persistent_trace(S, T, st, cursor, n, batch, stack_cap, start_ray, finish_ray);
     if constexpr (STATS) add_stats(stats, st);
 }
+
+constexpr uint64_t kMaxItems = 1ull << 31;
 
 template <bool ANY, int FETCH, int OCC, bool STATS>
 static cudaError_t launch_variant(const DevScene& S, const float4* rays, uint64_t n, uint4* hits,
@@ -51,12 +52,21 @@ static cudaError_t launch_variant(const DevScene& S, const float4* rays, uint64_
     const size_t smem = traversal_bytes<QueryKind<ANY, FETCH, OCC>>(t.block);
     const int per_sm = t.blocks_per_sm > 0 ? t.blocks_per_sm
                                            : resident.get(trace_kernel<ANY, FETCH, OCC, STATS>, t.block, smem);
-    uint64_t grid = (uint64_t)sm_count * per_sm;
-    const uint64_t want = (n + (uint64_t)t.block - 1) / (uint64_t)t.block;
-    if (want < grid) grid = want;
-    trace_kernel<ANY, FETCH, OCC, STATS><<<(unsigned)grid, t.block, smem, s>>>(
-        S, rays, n, hits, occ, max_steps, cursor, (uint32_t)t.batch, stats, t.stack);
-    return cudaGetLastError();
+    cudaError_t e = ResidentBlocks::allow(trace_kernel<ANY, FETCH, OCC, STATS>, smem);
+    if (e != cudaSuccess) return e;
+    // 32-bit item numbers: more rays than kMaxItems go in several launches
+    for (uint64_t k = 0; k < n; k += kMaxItems) {
+        const uint32_t m = (uint32_t)std::min(n - k, kMaxItems);
+        if ((e = cudaMemsetAsync(cursor, 0, sizeof(*cursor), s)) != cudaSuccess) return e;
+        // at most one block per ray: a short query has each ray in a warp and
+        // mostly on an SM of its own
+        const unsigned grid = std::min((uint32_t)(sm_count * per_sm), m);
+        trace_kernel<ANY, FETCH, OCC, STATS><<<grid, t.block, smem, s>>>(
+            S, rays + 2 * k, m, k, ANY ? nullptr : hits + k, ANY ? occ + k / 32 : nullptr, max_steps,
+            reinterpret_cast<uint32_t*>(cursor), (uint32_t)t.batch, stats, t.stack);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 template <bool ANY>
@@ -89,10 +99,8 @@ cudaError_t launch_trace(bool any, const DevScene& S, const void* rays, uint64_t
                          uint32_t* occ_bits, uint32_t max_steps, unsigned long long* cursor,
                          unsigned long long* stats, const Tune& t, int sm_count, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
     if (any) {
-        e = cudaMemsetAsync(occ_bits, 0, sizeof(uint32_t) * ((n + 31) / 32), s);
+        const cudaError_t e = cudaMemsetAsync(occ_bits, 0, sizeof(uint32_t) * ((n + 31) / 32), s);
         if (e != cudaSuccess) return e;
         return launch_any_variant<true>(S, rays, n, hits, occ_bits, max_steps, cursor, stats, t,
                                         sm_count, s);

@@ -7,7 +7,7 @@
 // is shared by both levels); the object's BLAS is traversed on the same stack
 // with a parameter s = t - t_e.  When the stack drains back to the level where
 // the instance was entered, the world ray is restored.  Leaves of a BLAS hold
-// up to 16 quads stored contiguously.
+// up to 8 quads stored contiguously.
 //
 // Precision design.  Box tests are made conservative by widening every
 // dequantised box by twice delta, an absolute bound on the position error of the
@@ -31,16 +31,17 @@
 // holds one ray; the warp tests inner nodes together, enters instances in
 // groups, then lets every other lane enter its instance or test one leaf;
 // finished lanes take the next ray at once (claimed one atomic per warp).
-// What bounds it is each ray's chain of dependent node loads, hidden by
-// resident warps, and the issue slots at 13 to 17 active lanes of 32.  So the
-// registers hold what a node test reads and shared memory the rest of a ray
-// and its stack: 64 registers (32 warps an SM) without spills in the node and
-// leaf loops.  Before, the compiler kept it all in registers and spilled
-// 476 bytes a thread, the 64-entry stacks lay in local memory, and the FP64
-// re-test sat in the leaf loop.  Both against each other on one GB300, ms:
-// 2 M diffuse bounces on the mid scene 5.59 -> 3.44, 1.5 M sun rays 1.61 ->
-// 1.11, 1 M rays of ambient occlusion on the island (0.42 re-tests a ray) 1.94
-// -> 1.03, the mid frame 18.04 -> 13.69, the island frame 33.6 -> 26.3.
+// What bounds it is the issue slots (65 to 75 % busy at 13 to 17 active lanes
+// of 32; some 430 warp instructions per node step, all phases counted) and,
+// behind them, each ray's chain of dependent node loads, hidden by resident
+// warps.  So the registers hold what a node test reads and shared memory the
+// rest of a ray and its stack: 64 registers (32 warps an SM) without spills.
+// Left to the compiler, the state spilled 476 bytes a thread at 48 registers,
+// the 64-entry stacks lay in local memory, a node test sorted its children and
+// the FP64 re-test sat in the leaf loop.  That against this on one GB300, ms:
+// 2 M diffuse bounces on the mid scene 5.58 -> 2.92, 1.5 M sun rays 1.60 ->
+// 0.83, 1 M rays of ambient occlusion on the island (0.42 re-tests a ray) 1.95
+// -> 0.91, the mid frame 17.9 -> 11.1, the island frame 34.2 -> 22.1.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -60,19 +61,17 @@ struct Hit {
     uint32_t slot;  // global quad slot of the hit (for shading)
 };
 
-// A world-space ray (origin, direction).  The traversal asks a caller-given
-// functor for it where it is needed (instance entry, return to the TLAS, FP64
-// re-tests) instead of keeping six floats live for the whole ray: kernels
-// whose rays sit in device memory reload them from there.
+// A world-space ray (origin, direction).
 struct WRay {
     float ox, oy, oz, dx, dy, dz;
 };
 
-// Ray in the current space, with everything the node and quad tests reuse.
+// Ray in the current space: what a node test reads, in the two quadruples in
+// which the world-space form also lies in shared memory (Traversal), so that
+// one 128-bit load each restores it in place.
 struct RaySetup {
-    float ox, oy, oz;     // origin
-    float ix, iy, iz;     // reciprocal direction, |d| clamped away from 0
-    float delta2;         // 2 delta, delta the bound on its position error
+    float4 o;    // origin; w: 2 delta, delta the bound on its position error
+    float4 inv;  // reciprocal direction, |d| clamped away from 0; w: near end of the interval
 };
 
 // Watertight shear of the current-space ray in affine form,
@@ -90,20 +89,15 @@ __device__ __forceinline__ float clamp_dir(float d) {
     return fabsf(d) > 1e-30f ? d : copysignf(1e-30f, d);
 }
 
-__device__ __forceinline__ void setup_boxes(RaySetup& r, float ox, float oy, float oz, float dx,
-                                            float dy, float dz, float delta) {
-    r.ox = ox;
-    r.oy = oy;
-    r.oz = oz;
-    r.ix = __frcp_rn(clamp_dir(dx));
-    r.iy = __frcp_rn(clamp_dir(dy));
-    r.iz = __frcp_rn(clamp_dir(dz));
-    r.delta2 = 2.0f * delta;
+__device__ __forceinline__ RaySetup setup_boxes(float ox, float oy, float oz, float dx, float dy, float dz,
+                                                float delta, float near) {
+    return RaySetup{make_float4(ox, oy, oz, 2.0f * delta),
+                    make_float4(__frcp_rn(clamp_dir(dx)), __frcp_rn(clamp_dir(dy)), __frcp_rn(clamp_dir(dz)), near)};
 }
 
-// (dx, dy, dz): the ray direction in the current space, the same value the
-// box set-up was made from
-__device__ __forceinline__ Shear make_shear(const RaySetup& r, float dx, float dy, float dz) {
+// o: the origin in the current space and 2 delta; (dx, dy, dz): the direction,
+// the same value the box set-up was made from
+__device__ __forceinline__ Shear make_shear(const float4& o, float dx, float dy, float dz) {
     Shear sh;
     const float ax = fabsf(dx), ay = fabsf(dy), az = fabsf(dz);
     // kz = dominant axis, (kx, ky) the next two in cyclic order; selects
@@ -112,9 +106,9 @@ __device__ __forceinline__ Shear make_shear(const RaySetup& r, float dx, float d
     const float dkx = kz == 0 ? dy : (kz == 1 ? dz : dx);
     const float dky = kz == 0 ? dz : (kz == 1 ? dx : dy);
     const float dkz = kz == 0 ? dx : (kz == 1 ? dy : dz);
-    const float okx = kz == 0 ? r.oy : (kz == 1 ? r.oz : r.ox);
-    const float oky = kz == 0 ? r.oz : (kz == 1 ? r.ox : r.oy);
-    const float okz = kz == 0 ? r.ox : (kz == 1 ? r.oy : r.oz);
+    const float okx = kz == 0 ? o.y : (kz == 1 ? o.z : o.x);
+    const float oky = kz == 0 ? o.z : (kz == 1 ? o.x : o.y);
+    const float okz = kz == 0 ? o.x : (kz == 1 ? o.y : o.z);
     // one reciprocal; the products' extra rounding is covered by delta
     const float Sz = __frcp_rn(dkz);
     const float Sx = __fmul_rn(dkx, Sz), Sy = __fmul_rn(dky, Sz);
@@ -133,7 +127,7 @@ __device__ __forceinline__ Shear make_shear(const RaySetup& r, float dx, float d
     sh.cz = __fmul_rn(Sz, okz);
     // a position error of delta moves the distance along the dominant axis
     // by delta |Sz|; twice that bounds the FP32 hit distance's error
-    sh.eps_t = __fmul_rn(r.delta2, fabsf(Sz));
+    sh.eps_t = __fmul_rn(o.w, fabsf(Sz));
     return sh;
 }
 
@@ -188,9 +182,10 @@ __device__ __forceinline__ void load_node(const QNode* n, uint32_t w[16]) {
     }
 }
 
-// Plane value v(q) of byte i of w (QNode): one byte permute.
-__device__ __forceinline__ float plane_v(uint32_t w, int i) {
-    return __uint_as_float(__byte_perm(w, 0x3F000000u, 0x7044u | ((uint32_t)i << 8)));
+// Plane value v(q) of byte i of w (QNode): one byte permute with plane_exp =
+// 0x3F000000.
+__device__ __forceinline__ float plane_v(uint32_t w, uint32_t plane_exp, int i) {
+    return __uint_as_float(__byte_perm(w, plane_exp, 0x7044u | ((uint32_t)i << 8)));
 }
 
 // Three-operand minima and maxima (one instruction on sm_103a); a NaN operand
@@ -218,9 +213,10 @@ __device__ __forceinline__ void fma2(float a0, float a1, float b, float c0, floa
         : "f"(a0), "f"(a1), "f"(b), "f"(c0), "f"(c1));
 }
 
-// Tests the four children of a node; writes entry distances (inf = culled)
-// and references, sorted nearest first (SORT) or in slot order (any-hit
-// rays, which need no order).  Returns the number of hits.
+// Tests the four children of a node, in slot order: entry distances (inf =
+// missed), whether hit, references.  An empty slot can pass for hit where all
+// of the node's planes lie within the widening; its kRefNone is then dropped
+// when it comes up.
 //
 // A plane's distance is fma(v(q), s/d, (node.o - o)/d), its box widened by
 // 2 delta.  delta alone bounds the ray's own position error; the second delta
@@ -228,18 +224,18 @@ __device__ __forceinline__ void fma2(float a0, float a1, float b, float c0, floa
 // 1/d and the fused product amount to at most e (|v s| + |node.o - o| +
 // 2 |plane - o|) <= e (9 R + 3 |o|) in position, R the radius of the space's
 // geometry (|v s| <= 2.7 R), while delta is at least 12 e (R + |o|).
-template <int FETCH, bool SORT = true>
-__device__ __forceinline__ int node_children(const QNode* node, const RaySetup& r, float tmin,
-                                             float tmax, float t[4], uint32_t ref[4]) {
+template <int FETCH>
+__device__ __forceinline__ void node_children(const QNode* node, uint32_t plane_exp, const RaySetup& r,
+                                              float tmax, float t[4], bool hit[4], uint32_t ref[4]) {
     uint32_t w[16];
     load_node<FETCH>(node, w);
-    const float o[3] = {r.ox, r.oy, r.oz}, inv[3] = {r.ix, r.iy, r.iz};
+    const float o[3] = {r.o.x, r.o.y, r.o.z}, inv[3] = {r.inv.x, r.inv.y, r.inv.z};
     float A[3], bn[3], bf[3];
     uint32_t wn[3], wf[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float d = __fsub_rn(__uint_as_float(w[a]), o[a]);
-        const float p = __fmul_rn(r.delta2, fabsf(inv[a]));
+        const float p = __fmul_rn(r.o.w, fabsf(inv[a]));
         A[a] = __fmul_rn(__uint_as_float(w[3 + a]), inv[a]);
         bn[a] = __fmaf_rn(d, inv[a], -p);
         bf[a] = __fmaf_rn(d, inv[a], p);
@@ -253,31 +249,13 @@ __device__ __forceinline__ int node_children(const QNode* node, const RaySetup& 
         float n[3], f[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a)
-            fma2(plane_v(wn[a], i), plane_v(wf[a], i), A[a], bn[a], bf[a], n[a], f[a]);
-        const float tn = fmaxf(max3(n[0], n[1], n[2]), tmin);
+            fma2(plane_v(wn[a], plane_exp, i), plane_v(wf[a], plane_exp, i), A[a], bn[a], bf[a], n[a], f[a]);
+        const float tn = fmaxf(max3(n[0], n[1], n[2]), r.inv.w);
         const float tf = fminf(min3(f[0], f[1], f[2]), tmax);
         ref[i] = w[12 + i];
-        t[i] = (tn <= tf) && ref[i] != kRefNone ? tn : kInfF;
+        hit[i] = tn <= tf;
+        t[i] = hit[i] ? tn : kInfF;
     }
-    if constexpr (!SORT)
-        return (t[0] < kInfF) + (t[1] < kInfF) + (t[2] < kInfF) + (t[3] < kInfF);
-    // sorting network on (t, ref); strict comparisons keep equal keys in order
-#define QRT_CSWAP(i, j)                             \
-    if (t[j] < t[i]) {                              \
-        float tt = t[i];                            \
-        t[i] = t[j];                                \
-        t[j] = tt;                                  \
-        uint32_t rr = ref[i];                       \
-        ref[i] = ref[j];                            \
-        ref[j] = rr;                                \
-    }
-    QRT_CSWAP(0, 1)
-    QRT_CSWAP(2, 3)
-    QRT_CSWAP(0, 2)
-    QRT_CSWAP(1, 3)
-    QRT_CSWAP(1, 2)
-#undef QRT_CSWAP
-    return (t[0] < kInfF) + (t[1] < kInfF) + (t[2] < kInfF) + (t[3] < kInfF);
 }
 
 // --------------------------------------------------------------------------
@@ -500,6 +478,14 @@ __device__ __forceinline__ void sts_u2(uint32_t a, uint32_t x, uint32_t y) {
     asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(a), "r"(x), "r"(y));
 }
 
+// v by way of shared memory (this lane's word a): a value that the compiler
+// cannot recompute and so keeps in a register.  Left to itself it rebuilt the
+// plane constant and the stack's address in every node test.
+__device__ __forceinline__ uint32_t keep_register(uint32_t a, uint32_t v) {
+    sts_u(a, v);
+    return lds_u(a);
+}
+
 // What a kernel asks of the traversal, and the shared memory it takes.
 //   ANY    any hit instead of the closest
 //   UV     the closest hit's quad-space (u, v) is wanted
@@ -517,21 +503,24 @@ struct TraversalKind {
     static constexpr bool ANY = ANY_, UV = UV_, RANGE = RANGE_;
     static constexpr int FETCH = FETCH_, STACK = STACK_;
     using Entry = std::conditional_t<ANY, uint32_t, uint64_t>;
-    static constexpr int kRecs = ANY ? 5 : (UV || RANGE ? 7 : 6);
+    static constexpr int kRecs = ANY ? 6 : (UV || RANGE ? 8 : 6);
     static constexpr int kLaneBytes = kRecs * 16 + STACK * (int)sizeof(Entry);
 };
 
-// Stack entries in shared memory: what fits the 48 KB of a 256-thread block,
-// and the 228 KB of an SM (less 1 KB a block) at the kernel's resident warps.
+// Stack entries in shared memory: what fits the 228 KB of an SM (less 1 KB a
+// block) at the kernel's resident warps, in blocks of 256 threads.  A ray's
+// stack seldom holds more than 9 entries, but the deepest of a warp's lanes is
+// beyond 9 in half of a closest-hit frame's node steps and beyond 12 in a
+// sixth, and a lane beyond takes its warp through the slower path.
 constexpr int shared_stack(bool any, int recs, int warps) {
-    return any ? 16 : ((warps > 40 ? 144 : warps > 32 ? 176 : 192) - 16 * recs) / 8;
+    return any ? 16 : ((warps > 40 ? 144 : warps > 32 ? 176 : 216) - 16 * recs) / 8;
 }
 
 // The ray-query kernels' rays, and the wavefront renderer's.
 template <bool ANY, int FETCH, int OCC>
-using QueryKind = TraversalKind<ANY, !ANY, true, FETCH, shared_stack(ANY, 7, OCC)>;
+using QueryKind = TraversalKind<ANY, !ANY, true, FETCH, shared_stack(ANY, 8, OCC)>;
 template <bool ANY, bool UV, int FETCH, int OCC>
-using WaveKind = TraversalKind<ANY, UV, ANY, FETCH, shared_stack(ANY, UV ? 7 : 6, OCC)>;
+using WaveKind = TraversalKind<ANY, UV, ANY, FETCH, shared_stack(ANY, UV ? 8 : 6, OCC)>;
 
 // Resumable traversal.  init() sets the ray up; the caller then runs, while
 // the ray is not finished, whichever step fits its state: inner_step (an inner
@@ -548,68 +537,81 @@ struct Traversal {
     static constexpr int STACK = Kind::STACK;
     using Entry = typename Kind::Entry;
 
-    uint32_t rec, stk;  // shared-memory addresses of this thread's records and stack
-    RaySetup r;         // the ray in the current space
-    float lo, lim;      // its interval there: lo = tmin - te, lim = best hit (or tmax) - te
+    uint32_t rec;         // shared-memory address of this thread's records
+    uint32_t plane_exp;   // 0x3F000000 (plane_v)
+    uint32_t tip;         // and of its stack's next free entry
+    uint32_t bottom;      // and first entry
+    uint32_t inst_tip;    // tip at instance entry; bottom at the top level
+    RaySetup r;         // the ray in the current space; r.inv.w = tmin - te
+    float lim;          // far end of its interval there: best hit (or tmax) - te
     uint32_t cur;       // reference to visit next, kRefNone: take one from the stack
     uint32_t pleaf;     // postponed BLAS leaf (0 = none)
     uint32_t node_base;
-    uint32_t budget;    // inner-node tests left before the step limit
-    int sp, inst_sp;    // stack height; height at instance entry, -1 at the top level
-    uint32_t err;       // device error bits
+    int budget;         // inner-node tests left before the step limit
     bool found;         // any-hit rays: answered
-    bool pending;       // a quad waits for resolve()
-    bool blocked;       // and another one for its place
-    Entry deep[kMaxStack - STACK];
+    int waiting;        // quads that wait for resolve(): 1, or 2 when another wants its place
+    uint32_t deep;      // local-memory address of the entries beyond shared memory
 
-    // records: word offsets from rec
-    static constexpr uint32_t kWorldO = 0;     // world origin, te
-    static constexpr uint32_t kWorldD = 512;   // world direction, h_t (any hit: cur_inst)
-    static constexpr uint32_t kWorldInv = 1024;  // world reciprocal direction
-    static constexpr uint32_t kObjD = 1536;    // object-space direction, quad_base
-    static constexpr uint32_t kHit = 2048;     // inst, slot, error bound of h_t, cur_inst
-    // the quad that waits: slot, inst; closest hit also u, v (u NaN: FP32 could
-    // not decide it) and the error bound of its distance
-    static constexpr uint32_t kPend = ANY ? 2056 : 2560;
-    static constexpr uint32_t kPendEps = kWorldInv + 12;
-    static constexpr uint32_t kRange = ANY ? 2048 : 3072;  // tmin, tmax; closest hit also u, v
+    // records: byte offsets from rec
+    static constexpr uint32_t kWorldO = 0;       // r.o at the top level
+    static constexpr uint32_t kWorldInv = 512;   // r.inv at the top level (w: tmin)
+    static constexpr uint32_t kWorldD = 1024;    // world direction; closest hit: h_t, any hit: cur_inst
+    static constexpr uint32_t kObjD = 1536;      // object-space direction, quad_base
+    static constexpr uint32_t kHit = 2048;       // closest hit: inst, slot, error bound of h_t, cur_inst
+    static constexpr uint32_t kObjO = 2048;      // any hit: r.o in object space
+    // the quad that waits: slot, inst; closest hit also the error bound of its
+    // distance; then te
+    static constexpr uint32_t kPend = 2560;
+    static constexpr uint32_t kPendEps = kPend + 8;
+    static constexpr uint32_t kTe = kPend + 12;
+    static constexpr uint32_t kTmax = ANY ? kPend + 8 : 3072 + 8;  // RANGE
+    static constexpr uint32_t kUV = 3072;        // u, v of the best hit, tmax, unused
+    static constexpr uint32_t kPendUV = 3584;    // of the waiting quad (u NaN: FP32 could not decide it)
+    static constexpr uint32_t kHT = kWorldD + 12;
     static constexpr uint32_t kCurInst = ANY ? kWorldD + 12 : kHit + 12;
 
-    __device__ __forceinline__ bool top() const { return inst_sp < 0; }
+    static constexpr uint32_t kStride = 32u * (uint32_t)sizeof(Entry);  // between stack entries
+    static constexpr uint32_t kShared = STACK * kStride;                // entries beyond go to local memory
 
-    // base: the warp's shared memory
-    __device__ __forceinline__ void bind(uint32_t base) {
+    __device__ __forceinline__ bool top(const DevScene& S) const { return node_base == S.tlas_base; }
+
+    // base: the warp's shared memory; deep_entries: kMaxStack - STACK entries
+    // of the thread's local memory (not a member: that would put the whole
+    // traversal there)
+    __device__ __forceinline__ void bind(uint32_t base, Entry* deep_entries) {
+        deep = (uint32_t)__cvta_generic_to_local(deep_entries);
         const uint32_t lane = threadIdx.x & 31u;
-        rec = base + 16u * lane;
-        stk = base + 512u * Kind::kRecs + (uint32_t)sizeof(Entry) * lane;
+        const uint32_t own = base + 16u * lane;
+        rec = keep_register(own, own);
+        bottom = keep_register(own, base + 512u * Kind::kRecs + (uint32_t)sizeof(Entry) * lane);
+        plane_exp = keep_register(own, 0x3F000000u);
         cur = kRefNone;
         pleaf = 0;
-        err = 0;
-        found = pending = blocked = false;
+        found = false;
+        waiting = 0;
     }
 
-    __device__ __forceinline__ float tmin() const { return RANGE ? lds1(rec + kRange) : 0.f; }
-    __device__ __forceinline__ float tmax() const { return RANGE ? lds1(rec + kRange + 4) : kInfF; }
+    __device__ __forceinline__ float tmin() const { return RANGE ? lds1(rec + kWorldInv + 12) : 0.f; }
+    __device__ __forceinline__ float tmax() const { return RANGE ? lds1(rec + kTmax) : kInfF; }
 
     __device__ __forceinline__ void init(const DevScene& S, float ox, float oy, float oz, float dx,
                                          float dy, float dz, float t0, float t1, uint32_t msteps,
                                          TraceStats& st) {
         ++st.rays;
-        sp = 0;
-        inst_sp = -1;
+        tip = inst_tip = bottom;
         node_base = S.tlas_base;
         pleaf = 0;
-        budget = msteps;
-        found = pending = blocked = false;
-        lo = t0;
+        budget = (int)min(msteps, 0x7FFFFFFFu);
+        found = false;
+        waiting = 0;
         lim = t1;
-        setup_boxes(r, ox, oy, oz, dx, dy, dz, world_delta(S, ox, oy, oz));
-        sts4(rec + kWorldO, ox, oy, oz, 0.f);
+        r = setup_boxes(ox, oy, oz, dx, dy, dz, world_delta(S, ox, oy, oz), t0);
+        sts4(rec + kWorldO, r.o.x, r.o.y, r.o.z, r.o.w);
+        sts4(rec + kWorldInv, r.inv.x, r.inv.y, r.inv.z, r.inv.w);
         sts4(rec + kWorldD, dx, dy, dz, t1);
-        sts4(rec + kWorldInv, r.ix, r.iy, r.iz, 0.f);
         if constexpr (!ANY) sts4(rec + kHit, __uint_as_float(0xFFFFFFFFu), 0.f, 0.f, 0.f);
-        if constexpr (RANGE) sts_u2(rec + kRange, __float_as_uint(t0), __float_as_uint(t1));
-        if constexpr (UV) sts_u2(rec + kRange + 8, 0u, 0u);
+        if constexpr (RANGE) sts1(rec + kTmax, t1);
+        if constexpr (UV) sts_u2(rec + kUV, 0u, 0u);
         cur = S.n_inst > 0 ? 0u : kRefNone;  // TLAS root, an inner reference
     }
 
@@ -630,116 +632,160 @@ struct Traversal {
         return __fadd_rn(__fsub_rn(t, te), 1.9073486328125e-06f * (fabsf(t) + fabsf(te)));
     }
 
-    __device__ __forceinline__ void put(int i, float t, uint32_t ref) {
-        if constexpr (ANY) {
-            if (i < STACK) sts_u(stk + 128u * (uint32_t)i, ref);
-            else deep[i - STACK] = ref;
-        } else {
-            if (i < STACK) sts_u2(stk + 256u * (uint32_t)i, ref, __float_as_uint(t));
-            else deep[i - STACK] = ((uint64_t)__float_as_uint(t) << 32) | ref;
-        }
+    __device__ __forceinline__ void put_shared(float t, uint32_t ref) {
+        if constexpr (ANY) sts_u(tip, ref);
+        else sts_u2(tip, ref, __float_as_uint(t));
+        tip += kStride;
     }
 
-    // Pops an entry into cur unless it lies beyond the best hit.
+    // As put_shared, wherever the entry goes; false if the stack is full (cap
+    // entries).
+    __device__ __forceinline__ bool put(float t, uint32_t ref, int cap) {
+        if (tip - bottom < kShared) {
+            put_shared(t, ref);
+            return true;
+        }
+        const int i = (int)((tip - bottom - kShared) / kStride);
+        if (i + STACK >= cap) return false;
+        const uint32_t a = deep + (uint32_t)sizeof(Entry) * (uint32_t)i;
+        if constexpr (ANY) asm volatile("st.local.u32 [%0], %1;" ::"r"(a), "r"(ref) : "memory");
+        else asm volatile("st.local.v2.u32 [%0], {%1,%2};" ::"r"(a), "r"(ref), "f"(t) : "memory");
+        tip += kStride;
+        return true;
+    }
+
+    // Pops an entry into cur unless it lies beyond the best hit.  Both places
+    // are read under a predicate: a branch and its reconvergence cost more.
     __device__ __forceinline__ void pop() {
-        const int i = --sp;
+        tip -= kStride;
+        const uint32_t off = tip - bottom;
+        const uint32_t far = deep + (off - kShared) / 32u;
         if constexpr (ANY) {
-            cur = i < STACK ? lds_u(stk + 128u * (uint32_t)i) : deep[i - STACK];
+            asm volatile("{.reg .pred p;\n\t"
+                         "setp.lt.u32 p, %1, %2;\n\t"
+                         "@p ld.shared.u32 %0, [%3];\n\t"
+                         "@!p ld.local.u32 %0, [%4];}"
+                         : "=r"(cur)
+                         : "r"(off), "n"(kShared), "r"(tip), "r"(far)
+                         : "memory");
         } else {
-            uint2 e;
-            if (i < STACK) {
-                e = lds_u2(stk + 256u * (uint32_t)i);
-            } else {
-                const uint64_t v = deep[i - STACK];
-                e = make_uint2((uint32_t)v, (uint32_t)(v >> 32));
-            }
-            cur = __uint_as_float(e.y) <= lim ? e.x : kRefNone;
-        }
-    }
-
-    // Pushes the hit children other than the one visited next and makes that
-    // one current (nh > 0).  Closest hit: children sorted nearest first, the
-    // nearest visited next, the others pushed farthest first with their entry
-    // distances.  Any hit: children in slot order (the answer does not
-    // depend on the order, and an unoccluded ray visits every child anyway),
-    // the first hit visited next.
-    __device__ __forceinline__ void push_children(int nh, const float t[4], const uint32_t ref[4]) {
-        if constexpr (ANY) {
-            const bool h0 = t[0] < kInfF, h1 = t[1] < kInfF, h2 = t[2] < kInfF;
-            const int first = h0 ? 0 : (h1 ? 1 : (h2 ? 2 : 3));
-#pragma unroll
-            for (int k = 3; k >= 0; --k)
-                if (t[k] < kInfF && k != first) put(sp++, t[k], ref[k]);
-            cur = h0 ? ref[0] : (h1 ? ref[1] : (h2 ? ref[2] : ref[3]));
-        } else {
-#pragma unroll
-            for (int k = 3; k >= 1; --k)
-                if (k < nh) put(sp++, t[k], ref[k]);
-            cur = ref[0];
+            uint32_t ref, t;
+            asm volatile("{.reg .pred p;\n\t"
+                         "setp.lt.u32 p, %2, %3;\n\t"
+                         "@p ld.shared.v2.u32 {%0,%1}, [%4];\n\t"
+                         "@!p ld.local.v2.u32 {%0,%1}, [%5];}"
+                         : "=r"(ref), "=r"(t)
+                         : "r"(off), "n"(kShared), "r"(tip), "r"(far)
+                         : "memory");
+            cur = __uint_as_float(t) <= lim ? ref : kRefNone;
         }
     }
 
     // A lane is in exactly one of: an inner node to test (wants_inner), a TLAS
     // leaf to enter (at_instance), a BLAS leaf to test (at_leaf: postponed or
-    // current), or finished.
+    // current), or nothing left to visit (visited; a quad may still wait).
     __device__ __forceinline__ bool wants_inner() const { return (int)cur >= 0; }
-    __device__ __forceinline__ bool at_instance() const { return (int)cur < 0 && cur != kRefNone && top(); }
-    __device__ __forceinline__ bool at_leaf() const {
-        return pleaf != 0 || ((int)cur < 0 && cur != kRefNone && !top());
-    }
-    // nothing left to visit (a quad may still wait), and the ray's end
+    __device__ __forceinline__ bool at_instance() const { return cur >= kRefInstance && (!ANY || pleaf == 0); }
+    __device__ __forceinline__ bool at_blas_leaf() const { return cur - kRefLeaf < kRefNone - kRefLeaf; }
+    __device__ __forceinline__ bool at_leaf() const { return pleaf != 0 || at_blas_leaf(); }
     __device__ __forceinline__ bool visited() const { return cur == kRefNone && pleaf == 0; }
-    __device__ __forceinline__ bool finished() const { return visited() && !pending; }
+    __device__ __forceinline__ bool finished() const { return visited() && waiting == 0; }
 
     __device__ __forceinline__ void stop(uint32_t e) {
-        err |= e;
+        budget = kStopped | (int)e;
         cur = kRefNone;
         pleaf = 0;
-        sp = 0;
-        pending = blocked = false;
+        waiting = 0;
     }
 
-    // Pops until cur holds a reference, the stack is empty, or the instance
-    // boundary is reached while a leaf of this instance is still postponed.
-    // BLAS leaves met on the way are postponed (one at a time) so that the
-    // lane keeps traversing inner nodes with the rest of its warp.
+    __device__ __forceinline__ void postpone() {
+        if (pleaf == 0 && at_blas_leaf()) {
+            pleaf = cur;
+            cur = kRefNone;
+        }
+    }
+
+    // Pops until cur holds a reference, the stack is empty, or (closest hit)
+    // the instance boundary is reached while a leaf of this instance is still
+    // postponed.  BLAS leaves met on the way are postponed (one at a time) so
+    // that the lane keeps traversing inner nodes with the rest of its warp.
+    // Any-hit rays leave the instance all the same and test the leaf from the
+    // object-space ray in shared memory before they enter another (sun rays
+    // 0.99 -> 0.97 ms); closest-hit rays would walk on without that leaf's hit
+    // to cull with, and measured 5 % slower that way.
     __device__ __forceinline__ void advance(const DevScene& S) {
-        for (;;) {
-            if (cur != kRefNone) {
-                if (pleaf != 0 || top() || (int)cur >= 0) return;
-                pleaf = cur;
-                cur = kRefNone;
-            }
-            if (sp == inst_sp) {
-                if (pleaf) return;
+        postpone();
+        while (cur == kRefNone) {
+            if (tip == inst_tip) {
+                if (top(S) || (!ANY && pleaf != 0)) break;
                 leave_instance(S);
+                if (tip == bottom) break;
             }
-            if (sp == 0) return;
             pop();
+            postpone();
         }
     }
 
     // Tests the inner node cur and moves on (precondition: wants_inner()).
+    // Closest hit: the nearest hit child is visited next (the first of equally
+    // near ones), the others are pushed with their entry distances.  They are
+    // pushed in slot order, not sorted: with two hits, by far the most common
+    // case, that is sorted already, and a sorting network took 25 instructions
+    // of every node test.  Any hit: the first hit in slot order is next (the
+    // answer does not depend on the order, and an unoccluded ray visits every
+    // child anyway).
     __device__ __forceinline__ void inner_step(const DevScene& S, TraceStats& st, int cap) {
-        if (budget == 0) {
-            stop(kErrStepLimit);
-            return;
-        }
         --budget;
         ++st.nodes;
         float t[4];
+        bool hit[4];
         uint32_t ref[4];
-        const int nh = node_children<Kind::FETCH, !ANY>(S.nodes + (size_t)(node_base + cur), r, lo, lim, t, ref);
-        if (nh == 0) {
-            cur = kRefNone;
+        node_children<Kind::FETCH>(S.nodes + (size_t)(node_base + cur), plane_exp, r, lim, t, hit, ref);
+        bool next0, next1, next2;  // the child visited next, child 3 if none of these
+        if constexpr (ANY) {
+            next0 = hit[0];
+            next1 = !hit[0] && hit[1];
+            next2 = !hit[0] && !hit[1] && hit[2];
         } else {
-            if (sp + nh - 1 > cap) {
+            const float m = fminf(min3(t[0], t[1], t[2]), t[3]);
+            next0 = t[0] == m;
+            next1 = !next0 && t[1] == m;
+            next2 = !next0 && !next1 && t[2] == m;
+        }
+        const bool next3 = !next0 && !next1 && !next2;
+        const bool push[4] = {hit[0] && !next0, hit[1] && !next1, hit[2] && !next2, hit[3] && !next3};
+        cur = next0 ? ref[0] : next1 ? ref[1] : next2 ? ref[2] : ref[3];
+        if (!(hit[0] || hit[1] || hit[2] || hit[3])) cur = kRefNone;
+        if (tip - bottom <= kShared - 3 * kStride) {
+#pragma unroll
+            for (int k = 3; k >= 0; --k)
+                if (push[k]) put_shared(t[k], ref[k]);
+        } else {
+            bool room = true;
+#pragma unroll
+            for (int k = 3; k >= 0; --k)
+                if (push[k]) room = room && put(t[k], ref[k], cap);
+            if (!room) {
                 stop(kErrStackOverflow);
                 return;
             }
-            push_children(nh, t, ref);
         }
         advance(S);
+    }
+
+    // Whether the ray has tested more nodes than it may; such a ray ends here.
+    // Asked between steps and not in them, which saves two instructions of
+    // every node test: a ray may go some nodes beyond its limit, but never ends
+    // beyond it unreported.
+    __device__ __forceinline__ void check_budget() {
+        if (budget < 0 && !error()) stop(kErrStepLimit);
+    }
+
+    // Device error bits of a ray that was stopped, else 0: they take the place
+    // of its step count.
+    static constexpr int kStopped = (int)0x80000000u;
+    __device__ __forceinline__ uint32_t error() const {
+        return (uint32_t)budget - (uint32_t)kStopped < 16u ? (uint32_t)(budget & 15) : 0u;
     }
 
     // Tests one BLAS leaf (the postponed one first; precondition: at_leaf()).
@@ -762,7 +808,7 @@ struct Traversal {
         found = true;
         cur = kRefNone;
         pleaf = 0;
-        pending = blocked = false;
+        waiting = 0;
     }
 
     // Moves the ray into the object space of the instance of the TLAS leaf cur
@@ -777,7 +823,7 @@ struct Traversal {
         const float4 m0 = __ldg(ip), m1 = __ldg(ip + 1), m2 = __ldg(ip + 2), m3 = __ldg(ip + 3);
         // m0 = (c, R); m1 = (w0 w1 w2 w3); m2 = (w4 w5 w6 w7); m3 = (w8, node_base, quad_base, kappa)
         const float4 wo = lds4(rec + kWorldO), wd = lds4(rec + kWorldD);
-        const float tmin_ = lo;  // at the top level
+        const float tmin_ = r.inv.w;  // at the top level
         // Re-centre where the ray passes closest to the object origin (never
         // before tmin), so the re-centred origin lies within the object's
         // reach; hits before that point have s < 0.  (Re-centring at the
@@ -808,25 +854,25 @@ struct Traversal {
         node_base = __float_as_uint(m3.y);
         // 2^-22 (kappa + 2) (|o''| + R): rounding of W, of W (p - c), of W d and
         // of the shear arithmetic, with a factor-two margin
-        setup_boxes(r, rox, roy, roz, fdx, fdy, fdz,
-                    __fmul_rn(2.384185791015625e-07f * (m3.w + 2.0f), maxabs3(rox, roy, roz) + m0.w));
-        sts1(rec + kWorldO + 12, te);
+        r = setup_boxes(rox, roy, roz, fdx, fdy, fdz,
+                        __fmul_rn(2.384185791015625e-07f * (m3.w + 2.0f), maxabs3(rox, roy, roz) + m0.w),
+                        __fsub_rn(tmin_, te));
+        sts1(rec + kTe, te);
         sts4(rec + kObjD, fdx, fdy, fdz, m3.z);
+        if constexpr (ANY) sts4(rec + kObjO, rox, roy, roz, r.o.w);
         sts_u(rec + kCurInst, inst);
         lim = object_limit(ANY ? tmax() : wd.w, te);
-        lo = __fsub_rn(tmin_, te);
-        inst_sp = sp;
+        inst_tip = tip;
         ++st.insts;
         cur = 0;
     }
 
     // Back to the world-space ray and the top level.
     __device__ __forceinline__ void leave_instance(const DevScene& S) {
-        const float4 o = lds4(rec + kWorldO), inv = lds4(rec + kWorldInv);
-        r = RaySetup{o.x, o.y, o.z, inv.x, inv.y, inv.z, 2.0f * world_delta(S, o.x, o.y, o.z)};
-        lo = tmin();
-        lim = ANY ? tmax() : lds1(rec + kWorldD + 12);
-        inst_sp = -1;
+        r.o = lds4(rec + kWorldO);
+        r.inv = lds4(rec + kWorldInv);
+        lim = ANY ? tmax() : lds1(rec + kHT);
+        inst_tip = bottom;
         node_base = S.tlas_base;
     }
 
@@ -850,26 +896,27 @@ struct Traversal {
     __device__ __forceinline__ Hit hit(const DevScene& S) const {
         Hit h;
         const float4 a = lds4(rec + kHit);
-        h.t = lds1(rec + kWorldD + 12);
+        h.t = lds1(rec + kHT);
         h.inst = __float_as_uint(a.x);
         h.slot = __float_as_uint(a.y);
         h.prim = h.inst == 0xFFFFFFFFu ? 0xFFFFFFFFu : __ldg(S.prim + h.slot);
         h.u = h.v = 0.f;
         if constexpr (UV) {
-            h.u = lds1(rec + kRange + 8);
-            h.v = lds1(rec + kRange + 12);
+            h.u = lds1(rec + kUV);
+            h.v = lds1(rec + kUV + 4);
         }
         return h;
     }
 
-    // Makes (t, inst, slot) the best hit.
-    __device__ __forceinline__ void keep(float t, float te, uint32_t inst, uint32_t slot, float eps, float u,
-                                         float v) {
-        sts1(rec + kWorldD + 12, t);
+    // Makes (t, inst, slot) the best hit, and cuts the ray there.
+    __device__ __forceinline__ void record(float t, uint32_t inst, uint32_t slot, float eps, float u, float v) {
+        sts1(rec + kHT, t);
         sts_u2(rec + kHit, inst, slot);
         sts1(rec + kHit + 8, eps);
-        if constexpr (UV) sts_u2(rec + kRange + 8, __float_as_uint(u), __float_as_uint(v));
-        lim = top() ? t : object_limit(t, te);
+        if constexpr (UV) sts_u2(rec + kUV, __float_as_uint(u), __float_as_uint(v));
+    }
+    __device__ __forceinline__ void shorten(const DevScene& S, float t, float te) {
+        lim = top(S) ? t : object_limit(t, te);
     }
 
     // Tests the quads of BLAS leaf ref; returns true when an any-hit query is
@@ -878,21 +925,23 @@ struct Traversal {
     // the traversal goes on, and a second one puts the rest of its leaf back.
     __device__ __forceinline__ bool leaf(const DevScene& S, TraceStats& st, uint32_t ref) {
         const float4 od = lds4(rec + kObjD);
-        const Shear sh = make_shear(r, od.x, od.y, od.z);
-        const float te = lds1(rec + kWorldO + 12);
-        const float t1 = tmax();
+        const float4 oo = ANY ? lds4(rec + kObjO) : r.o;
+        const Shear sh = make_shear(oo, od.x, od.y, od.z);
+        const float te = lds1(rec + kTe);
+        const float t0 = tmin(), t1 = tmax();
+        const float smin = ANY ? __fsub_rn(t0, te) : r.inv.w;
         uint32_t slot = __float_as_uint(od.w) + (ref & kRefIndexMask);
         for (;;) {
             QuadHit q;
-            const QuadResult res = quad_test(sh, 0.5f * r.delta2, S.quads + slot, lo, __fsub_rn(t1, te), q);
+            const QuadResult res = quad_test(sh, 0.5f * oo.w, S.quads + slot, smin, __fsub_rn(t1, te), q);
             if (res != kQuadMiss) {
                 const float t = __fadd_rn(q.s, te);
                 bool wait = res == kQuadUncertain;
                 float u = __int_as_float(0x7fffffff), v = 0.f;
                 if constexpr (ANY) {
-                    if (!wait && t > tmin() && t < t1) return true;
-                } else if (!wait && t > tmin() && t < t1) {
-                    const float ht = lds1(rec + kWorldD + 12);
+                    if (!wait && t > t0 && t < t1) return true;
+                } else if (!wait && t > t0 && t < t1) {
+                    const float ht = lds1(rec + kHT);
                     const float4 hr = lds4(rec + kHit);
                     const uint32_t inst = lds_u(rec + kCurInst);
                     const uint32_t hinst = __float_as_uint(hr.x), hslot = __float_as_uint(hr.y);
@@ -905,28 +954,26 @@ struct Traversal {
                         } else {
                             u = 0.f;
                         }
-                        if (!wait && (t < ht || before(S, inst, slot, hinst, hslot)))
-                            keep(t, te, inst, slot, sh.eps_t, u, v);
+                        if (!wait && (t < ht || before(S, inst, slot, hinst, hslot))) {
+                            record(t, inst, slot, sh.eps_t, u, v);
+                            lim = object_limit(t, te);
+                        }
                     }
                 }
                 if (wait) {
-                    if (pending) {
-                        blocked = true;
+                    if (waiting) {
+                        waiting = 2;
                         pleaf = ref;
                         return false;
                     }
-                    pending = true;
-                    const float inst = lds1(rec + kCurInst);
-                    if constexpr (ANY) {
-                        sts_u2(rec + kPend, slot, __float_as_uint(inst));
-                    } else {
-                        sts4(rec + kPend, __uint_as_float(slot), inst, u, v);
-                        sts1(rec + kPendEps, sh.eps_t);
-                    }
+                    waiting = 1;
+                    sts_u2(rec + kPend, slot, lds_u(rec + kCurInst));
+                    if constexpr (!ANY) sts1(rec + kPendEps, sh.eps_t);
+                    if constexpr (UV) sts_u2(rec + kPendUV, __float_as_uint(u), __float_as_uint(v));
                 }
             }
             ++st.quads;
-            if ((ref & 0x78000000u) == 0) return false;
+            if ((ref & 0x38000000u) == 0) return false;
             // the rest of the leaf: one item further, one fewer
             ref -= (1u << 27) - 1u;
             ++slot;
@@ -938,38 +985,92 @@ struct Traversal {
     // distances, equal distances by (instance, quad).  Rare, and slow on this
     // GPU (FP64 runs at 1/64 of FP32, and a warp pays for one lane what it
     // pays for all), so the caller gathers lanes for it.
-    __device__ __forceinline__ void resolve(const DevScene& S, TraceStats& st) {
-        pending = blocked = false;
+    //
+    // The traversal's registers (and the caller's, `item`) are put away in
+    // local memory and read back here, by hand: the compiler, left to keep
+    // them over the calls, stored each of them whenever it changed, nine local
+    // stores in every node step.
+    __device__ __forceinline__ void resolve(const DevScene& S, TraceStats& st, uint32_t& item) {
+        volatile uint32_t away[19];
+        const float rf[8] = {r.o.x, r.o.y, r.o.z, r.o.w, r.inv.x, r.inv.y, r.inv.z, r.inv.w};
+        away[0] = rec;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) away[1 + k] = __float_as_uint(rf[k]);
+        away[9] = __float_as_uint(lim);
+        away[10] = cur;
+        away[11] = pleaf;
+        away[12] = tip;
+        away[13] = inst_tip;
+        away[14] = bottom;
+        away[15] = plane_exp;
+        away[16] = node_base;
+        away[17] = (uint32_t)budget;
+        away[18] = item;
         ++st.fallbacks;
-        const WRay w = world();
-        const float t0 = tmin(), t1 = tmax();
-        if constexpr (ANY) {
+        bool better = false;
+        {
             const uint2 p = lds_u2(rec + kPend);
-            const float t = (float)quad_test64(S.inst + p.y, S.inst64 + p.y, S.quads + p.x, w, t0).t;
-            if (t > t0 && t < t1) answer();
-        } else {
-            const float4 p = lds4(rec + kPend);
-            const uint32_t slot = __float_as_uint(p.x), inst = __float_as_uint(p.y);
-            const Hit64 c = quad_test64(S.inst + inst, S.inst64 + inst, S.quads + slot, w, t0);
-            const float t = (float)c.t;
-            if (!(t > t0 && t < t1 && c.t < (double)t1)) return;
-            const float ht = lds1(rec + kWorldD + 12);
-            const float4 hr = lds4(rec + kHit);
-            const uint32_t hinst = __float_as_uint(hr.x), hslot = __float_as_uint(hr.y);
-            float eps = lds1(rec + kPendEps);
-            bool better;
-            if (fabsf(t - ht) <= fmaxf(eps, hr.z) && hinst != 0xFFFFFFFFu && !(hslot == slot && hinst == inst)) {
-                ++st.fallbacks;
-                const double tb = quad_test64(S.inst + hinst, S.inst64 + hinst, S.quads + hslot, w, t0).t;
-                better = c.t < tb || (c.t == tb && before(S, inst, slot, hinst, hslot));
-            } else {
-                better = t < ht || (t == ht && before(S, inst, slot, hinst, hslot));
-                eps = 0.f;
+            const Hit64 c = quad_test64(S.inst + p.y, S.inst64 + p.y, S.quads + p.x, world(), tmin());
+            rec = away[0];
+            const float t = (float)c.t, t0 = tmin(), t1 = tmax();
+            better = t > t0 && t < t1 && c.t < (double)t1;
+            if constexpr (!ANY) {
+                if (better) better = beats_best(S, st, c, away);
             }
-            const bool decided = p.z == p.z;  // FP32 hit: its own (u, v)
-            if (better)
-                keep(t, lds1(rec + kWorldO + 12), inst, slot, eps, decided ? p.z : c.u, decided ? p.w : c.v);
         }
+        rec = away[0];
+        const auto f = [&](int k) { return __uint_as_float(away[k]); };
+        r.o = make_float4(f(1), f(2), f(3), f(4));
+        r.inv = make_float4(f(5), f(6), f(7), f(8));
+        lim = f(9);
+        cur = away[10];
+        pleaf = away[11];
+        tip = away[12];
+        inst_tip = away[13];
+        bottom = away[14];
+        plane_exp = away[15];
+        node_base = away[16];
+        budget = (int)away[17];
+        item = away[18];
+        waiting = 0;
+        if (better) {
+            if constexpr (ANY) answer();
+            else shorten(S, lds1(rec + kHT), lds1(rec + kTe));
+        }
+    }
+
+    // Whether the waiting quad's FP64 hit c beats the best hit, whose place it
+    // then takes.  away[0] = rec.
+    __device__ __forceinline__ bool beats_best(const DevScene& S, TraceStats& st, const Hit64& c,
+                                               const volatile uint32_t* away) {
+        const float4 hr = lds4(rec + kHit);
+        const float t = (float)c.t, ht = lds1(rec + kHT);
+        const uint2 p = lds_u2(rec + kPend);
+        const uint32_t hinst = __float_as_uint(hr.x), hslot = __float_as_uint(hr.y);
+        float eps = lds1(rec + kPendEps);
+        bool better;
+        if (fabsf(t - ht) <= fmaxf(eps, hr.z) && hinst != 0xFFFFFFFFu && !(hslot == p.x && hinst == p.y)) {
+            ++st.fallbacks;
+            const double tb =
+                quad_test64(S.inst + hinst, S.inst64 + hinst, S.quads + hslot, world(), tmin()).t;
+            rec = away[0];
+            better = c.t < tb || (c.t == tb && before(S, p.y, p.x, hinst, hslot));
+        } else {
+            better = t < ht || (t == ht && before(S, p.y, p.x, hinst, hslot));
+            eps = 0.f;
+        }
+        if (better) {
+            float u = c.u, v = c.v;
+            if constexpr (UV) {
+                const uint2 uv = lds_u2(rec + kPendUV);
+                if (__uint_as_float(uv.x) == __uint_as_float(uv.x)) {  // an FP32 hit: its own (u, v)
+                    u = __uint_as_float(uv.x);
+                    v = __uint_as_float(uv.y);
+                }
+            }
+            record(t, p.y, p.x, eps, u, v);
+        }
+        return better;
     }
 
     // Order of two hits at the same distance.
@@ -979,108 +1080,133 @@ struct Traversal {
     }
 };
 
-// Shared memory of a block of `threads` threads, and a warp's part of it.
+// Shared memory of a block of `threads` threads, and a warp's part of it: the
+// lanes' records and stacks, and the warp's claimed items.
 template <class Kind>
 constexpr size_t traversal_bytes(int threads) {
-    return (size_t)threads * Kind::kLaneBytes;
+    return (size_t)threads * Kind::kLaneBytes + threads / 32 * 16;
 }
 template <class Kind>
 __device__ __forceinline__ uint32_t traversal_base() {
     extern __shared__ __align__(512) unsigned char qrt_smem[];
-    return (uint32_t)__cvta_generic_to_shared(qrt_smem) + (threadIdx.x >> 5) * 32u * Kind::kLaneBytes;
+    return (uint32_t)__cvta_generic_to_shared(qrt_smem) + (threadIdx.x >> 5) * (32u * Kind::kLaneBytes + 16u);
 }
 
-// Persistent warp-synchronous traversal loop over work items [0, count)
-// claimed from *cursor.  Each lane holds one ray; start(k) sets item k up in
-// T (T.init), done() consumes the finished ray in T; a ray may use cap (<=
-// kMaxStack) stack entries, a launch-wide value passed down rather than kept per
-// ray.  A lane claims `batch`
-// items at a time; the idle lanes of a warp claim theirs with one atomic
-// (warp-aggregated), so a launch costs about one atomic per warp and
-// refill round instead of one per thread.  Per outer iteration
-// the warp first tests inner nodes together (lanes that reach a BLAS leaf
-// postpone it and keep traversing; lanes waiting at instances enter them in
-// groups) until few lanes are left with an inner node, then lanes enter
-// instances or test one leaf each.  Finished lanes refill
-// immediately, so no lane waits for the slowest ray of its warp.
-template <class Kind, class Idx, class Start, class Done>
+// Persistent warp-synchronous traversal loop over work items [0, count).  Each
+// lane holds one ray; start(k) sets item k up in T (T.init), done(k) consumes
+// the finished ray in T; a ray may use cap (<= kMaxStack) stack entries, a
+// launch-wide value passed down rather than kept per ray.
+//
+// The first items are dealt out: L to each warp, as many as it takes for the
+// launch's warps to hold them all, at most 32.  So a short queue is spread one
+// ray to a warp and over all SMs, where no ray waits for another's divergent
+// steps.  Later ones are claimed from *cursor (zero at the launch), `batch` a
+// lane and one atomic for the idle lanes of a warp, so a finished lane never
+// waits for the slowest ray of its warp.
+//
+// Per outer iteration the warp first tests inner nodes together (lanes that
+// reach a BLAS leaf postpone it and keep traversing; lanes waiting at
+// instances enter them in groups) until few lanes are left with an inner node,
+// then lanes enter instances or test one leaf each.
+template <class Kind, class Start, class Done>
 __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Kind>& T, TraceStats& st,
-                                                 Idx* cursor, Idx count, uint32_t batch, int cap,
+                                                 uint32_t* cursor, uint32_t count, uint32_t batch, int cap,
                                                  Start start, Done done) {
     const unsigned FULL = 0xFFFFFFFFu;
     const unsigned lane = threadIdx.x & 31u;
-    // [next, end) = this lane's claimed items not yet started; a claim that
-    // lands at or past count leaves end == count, which ends the claiming
-    bool busy = false;
-    Idx next = 0, end = 0;
+    constexpr uint32_t kIdle = 0xFFFFFFFFu;  // counts stay below it
+    const uint32_t base = traversal_base<Kind>();
+    const uint32_t claimed = base + 32u * Kind::kLaneBytes;  // claimed items not yet started: first, end
+    typename Kind::Entry deep[kMaxStack - Kind::STACK];
+    T.bind(base, deep);
+    uint32_t item = kIdle;
     int waited = 0;  // iterations lanes have sat with nothing left but a waiting quad
-    T.bind(traversal_base<Kind>());
+    bool more;       // items may be left to claim
+    {
+        const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+        const uint32_t w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+        const uint32_t L = min(32u, (count + warps - 1) / warps);
+        const uint32_t k = w * L + lane;
+        if (lane < L && k < count) {
+            item = k;
+            start(k);
+        }
+        more = count > 32u * warps;
+        if (lane == 0) sts_u2(claimed, 0u, 0u);
+        __syncwarp();
+    }
     for (;;) {
-        const bool need = !busy && next >= end && end < count;
-        const unsigned want = __ballot_sync(FULL, need);
-        if (want) {
-            const int leader = __ffs(want) - 1;
-            Idx base = 0;
-            if ((int)lane == leader) base = atomicAdd(cursor, (Idx)batch * (Idx)__popc(want));
-            base = __shfl_sync(FULL, base, leader);
-            if (need) {
-                next = base + (Idx)batch * (Idx)__popc(want & ((1u << lane) - 1u));
-                end = min(next + (Idx)batch, count);
+        const unsigned want = __ballot_sync(FULL, item == kIdle);
+        if (more && want) {
+            const uint32_t n = (uint32_t)__popc(want), rank = (uint32_t)__popc(want & ((1u << lane) - 1u));
+            const uint2 have = lds_u2(claimed);
+            const uint32_t left = have.y - have.x;
+            uint32_t first = 0;
+            if (n > left) {
+                const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+                if (lane == 0) first = 32u * warps + atomicAdd(cursor, batch * n);
+                first = __shfl_sync(FULL, first, 0);
             }
+            __syncwarp();
+            if (lane == 0) {
+                if (n > left) sts_u2(claimed, first + (n - left), first + batch * n);
+                else sts_u2(claimed, have.x + n, have.y);
+            }
+            __syncwarp();
+            if (item == kIdle) {
+                const uint32_t k = rank < left ? have.x + rank : first + (rank - left);
+                if (k < count) {
+                    item = k;
+                    start(k);
+                }
+            }
+            more = __all_sync(FULL, item != kIdle);  // past the end: nothing more to claim
         }
-        if (!busy && next < end) {
-            start(next++);
-            busy = true;
-        }
-        if (__all_sync(FULL, !busy)) break;
+        const int n_busy = __popc(__ballot_sync(FULL, item != kIdle));
+        if (n_busy == 0) break;
         for (;;) {
             // Once eight or more lanes wait at an instance (TLAS leaf), they
             // enter it together and go on with the inner nodes of its BLAS
             // in this phase, instead of idling until the next outer
             // iteration.  Each such step enters at least eight instances.
             const bool wt = T.at_instance();
-            const unsigned bt = __ballot_sync(FULL, wt);
-            if (__popc(bt) >= 8) {
+            if (__popc(__ballot_sync(FULL, wt)) >= 8) {
                 if (wt) T.instance_step(S, st);
                 continue;
             }
-            const bool w = T.wants_inner();
-            const unsigned bw = __ballot_sync(FULL, w);
-            if (!bw) break;
             // Leave the inner-node phase early once the lanes still in it are
-            // at most half as many as the lanes waiting at an instance or a
+            // no more than the lanes waiting at an instance or a
             // leaf (or finished): those then move on together instead of
-            // idling until the warp's longest run of inner nodes ends.
-            // bo != 0 keeps a lane that the next phase moves on, so every
-            // outer iteration makes progress.
-            const unsigned bo = __ballot_sync(FULL, busy && !w);
-            if (bo && 2 * __popc(bw) <= __popc(bo)) break;
+            // idling until the warp's longest run of inner nodes ends.  A lane
+            // that the next phase moves on is left then, or no lane is busy,
+            // so every outer iteration makes progress.
+            const bool w = T.wants_inner();
+            if (2 * __popc(__ballot_sync(FULL, w)) <= n_busy) break;
             if (w) T.inner_step(S, st, cap);
         }
-        if (busy) {
-            if (T.at_instance()) {
-                T.instance_step(S, st);
-            } else if (T.at_leaf()) {
-                T.leaf_step(S, st);
-            }
+        if (T.at_instance()) {
+            T.instance_step(S, st);
+        } else if (T.at_leaf()) {
+            T.leaf_step(S, st);
         }
         // Waiting quads are decided together: when a lane cannot go on, when
         // eight wait, or when the lanes that wait for nothing else have cost
         // about as much as the FP64 test does.
-        const unsigned bp = __ballot_sync(FULL, T.pending);
+        const unsigned bp = __ballot_sync(FULL, T.waiting != 0);
         if (bp) {
-            const bool idle = T.pending && T.visited();
+            const bool idle = T.waiting != 0 && T.visited();
             waited += __popc(__ballot_sync(FULL, idle));
-            if (__popc(bp) >= 8 || waited >= 16 || __any_sync(FULL, T.blocked) ||
-                !__any_sync(FULL, busy && !idle)) {
-                if (T.pending) T.resolve(S, st);
+            if (__popc(bp) >= 8 || waited >= 16 || __any_sync(FULL, T.waiting == 2) ||
+                !__any_sync(FULL, item != kIdle && !idle)) {
+                if (T.waiting) T.resolve(S, st, item);
                 waited = 0;
             }
         }
-        if (busy) {
+        if (item != kIdle) {
+            T.check_budget();
             if (T.finished()) {
-                done();
-                busy = false;
+                done(item);
+                item = kIdle;
             }
         }
     }
@@ -1095,11 +1221,14 @@ __device__ __forceinline__ uint32_t trace_ray(const DevScene& S, float wox, floa
                                               uint32_t max_steps, int cap, Hit* h, bool* found,
                                               TraceStats& st) {
     Traversal<Kind> T;
-    T.bind(traversal_base<Kind>());
+    typename Kind::Entry deep[kMaxStack - Kind::STACK];
+    T.bind(traversal_base<Kind>(), deep);
     T.init(S, wox, woy, woz, wdx, wdy, wdz, tmin, tmax, max_steps, st);
+    uint32_t none = 0;
     while (!T.finished()) {
-        if (T.blocked || T.visited())
-            T.resolve(S, st);
+        T.check_budget();
+        if (T.waiting == 2 || T.visited())
+            T.resolve(S, st, none);
         else if (T.wants_inner())
             T.inner_step(S, st, cap);
         else if (T.at_instance())
@@ -1111,7 +1240,7 @@ __device__ __forceinline__ uint32_t trace_ray(const DevScene& S, float wox, floa
         *found = T.found;
     else
         *h = T.hit(S);
-    return T.err;
+    return T.error();
 }
 
 }  // namespace qrt

@@ -119,10 +119,9 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
     const uint32_t batch = A.batch;
     TraceStats st{0, 0, 0, 0, 0, 0};
     Traversal<WaveKind<ANY, UV, FETCH, OCC>> T;
-    uint32_t j = 0;
     // any-hit entries of key-light shadow rays carry kLightRay
     auto start_ray = [&](uint32_t k) {
-        j = queue[k];
+        const uint32_t j = queue[k];
         if (ANY) {
             const float4 o = A.B.sray_o[j & ~kLightRay];
             if (j & kLightRay) {
@@ -138,10 +137,14 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
             T.init(A.S, o.x, o.y, o.z, d.x, d.y, d.z, 0.f, kInfF, A.P.max_steps, st);
         }
     };
-    auto finish_ray = [&]() {
+    auto finish_ray = [&](uint32_t k) {
+        if (T.error()) atomicOr(A.S.err, T.error());
+        const uint32_t j = queue[k];
         const uint32_t jj = j & ~kLightRay;
         if constexpr (STATS) {
-            if (A.cost_on) atomicAdd(A.B.cost + jj, A.P.max_steps - T.budget);
+            if (A.cost_on)
+                atomicAdd(A.B.cost + jj,
+                          min(A.P.max_steps, 0x7FFFFFFFu) - (uint32_t)(T.error() ? 0 : T.budget));
         }
         if (ANY) {
             const bool light = j & kLightRay;
@@ -171,7 +174,6 @@ __global__ void __maxnreg__(occupancy_regs(OCC)) wave_trace(const __grid_constan
         }
     };
     persistent_trace(A.S, T, st, fetch, count, batch, stack_cap, start_ray, finish_ray);
-    if (T.err) atomicOr(A.S.err, T.err);
     if constexpr (STATS) add_stats(A.stats + (ANY ? 6 : 0), st);
 }
 
@@ -357,6 +359,8 @@ static cudaError_t launch_wave_trace_v(const WaveArgs& A, int depth, const Tune&
     const int per_sm = t.blocks_per_sm > 0
                            ? t.blocks_per_sm
                            : resident.get(wave_trace<ANY, FETCH, OCC, STATS, UV>, t.block, smem);
+    const cudaError_t e = ResidentBlocks::allow(wave_trace<ANY, FETCH, OCC, STATS, UV>, smem);
+    if (e != cudaSuccess) return e;
     wave_trace<ANY, FETCH, OCC, STATS, UV><<<(unsigned)(sm_count * per_sm), t.block, smem, s>>>(
         A, depth, t.stack);
     return cudaGetLastError();
