@@ -39,9 +39,9 @@
 // Left to the compiler, the state spilled 476 bytes a thread at 48 registers,
 // the 64-entry stacks lay in local memory, a node test sorted its children and
 // the FP64 re-test sat in the leaf loop.  That against this on one GB300, ms:
-// 2 M diffuse bounces on the mid scene 5.58 -> 2.92, 1.5 M sun rays 1.60 ->
-// 0.83, 1 M rays of ambient occlusion on the island (0.42 re-tests a ray) 1.95
-// -> 0.91, the mid frame 17.9 -> 11.1, the island frame 34.2 -> 22.1.
+// 2 M diffuse bounces on the mid scene 5.6 -> 2.95, 1.5 M sun rays 1.60 ->
+// 0.81, 1 M rays of ambient occlusion on the island (0.42 re-tests a ray) 1.95
+// -> 0.86, the mid frame 17.7 -> 10.7, the island frame 33.9 -> 21.3.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -1073,6 +1073,59 @@ struct Traversal {
         return better;
     }
 
+    // ---- any-hit rays: parts of a ray's tree traversed by idle lanes ---------
+
+    // Shared-memory address of the stack's lowest entry (the subtree highest in
+    // the tree, as a rule the largest), 0 if there is none to give away.
+    __device__ __forceinline__ uint32_t spare_entry() const {
+        const uint32_t end = min(tip, bottom + kShared);
+        for (uint32_t a = bottom; a != end; a += kStride)
+            if (lds_u(a) != kRefNone) return a;
+        return 0;
+    }
+
+    // Takes the entry at address `entry` from the ray of the lane with records
+    // at `from` and makes this lane, which is idle, traverse it.  other, its
+    // other_base: that lane's ray and node_base; object_space: the entry lies
+    // in its instance.
+    __device__ __forceinline__ void take(const DevScene& S, uint32_t from, uint32_t entry, bool object_space,
+                                         const RaySetup& other, uint32_t other_base) {
+#pragma unroll
+        for (int k = 0; k < Kind::kRecs; ++k) {
+            const float4 v = lds4(from + 512u * k);
+            sts4(rec + 512u * k, v.x, v.y, v.z, v.w);
+        }
+        cur = lds_u(entry);
+        sts_u(entry, kRefNone);
+        pleaf = 0;
+        tip = inst_tip = bottom;
+        budget = kHelperBudget;
+        found = false;
+        waiting = 0;
+        if (object_space) {
+            r = other;
+            node_base = other_base;
+            lim = object_limit(tmax(), lds1(rec + kTe));
+        } else {
+            r.o = lds4(rec + kWorldO);
+            r.inv = lds4(rec + kWorldInv);
+            node_base = S.tlas_base;
+            lim = tmax();
+        }
+    }
+    static constexpr int kHelperBudget = 0x3FFFFFFF;
+
+    // Takes over what a helper lane found, its steps and its error.
+    __device__ __forceinline__ void absorb(bool its_found, int its_budget) {
+        const uint32_t e = (uint32_t)its_budget - (uint32_t)kStopped;
+        if (its_found && !error()) answer();
+        if (e < 16u) {
+            if (!error()) stop(e);
+        } else if (!error()) {
+            budget -= kHelperBudget - its_budget;
+        }
+    }
+
     // Order of two hits at the same distance.
     static __device__ __forceinline__ bool before(const DevScene& S, uint32_t inst, uint32_t slot,
                                                   uint32_t hinst, uint32_t hslot) {
@@ -1090,6 +1143,69 @@ template <class Kind>
 __device__ __forceinline__ uint32_t traversal_base() {
     extern __shared__ __align__(512) unsigned char qrt_smem[];
     return (uint32_t)__cvta_generic_to_shared(qrt_smem) + (threadIdx.x >> 5) * (32u * Kind::kLaneBytes + 16u);
+}
+
+// What a lane of the persistent loop works on: item k, the ray of lane l
+// (kHelper + l), nothing.
+constexpr uint32_t kHelper = 0xFFFFFF00u, kIdle = 0xFFFFFFFFu;
+
+// Each idle lane takes a subtree off the stack of a busy one, as long as one
+// has any to give.  An unoccluded any-hit ray visits every node its segment
+// meets, in whatever order, so its subtrees can go in parallel: at the end of
+// a queue, and from the start of one too short for every lane, where otherwise
+// the launch lasts as long as its longest ray.  Shadow rays of the mid frame
+// 2.83 -> 2.53 ms, 1.5 M sun rays 0.90 -> 0.82.  Closest-hit rays lost that way
+// (one ray on the mid scene 32 -> 80 us): the far subtrees are those which the
+// near ones' hit culls.
+template <class Kind>
+__device__ __forceinline__ void share_rays(const DevScene& S, Traversal<Kind>& T, uint32_t& item, uint32_t base) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned idle = __ballot_sync(FULL, item == kIdle);
+    if (idle == 0 || idle == FULL) return;
+    const uint32_t give = item != kIdle && !T.visited() ? T.spare_entry() : 0u;
+    const unsigned givers = __ballot_sync(FULL, give != 0u);
+    if (givers == 0) return;
+    __syncwarp();  // the givers' shared memory is read below
+    const int rank = __popc(idle & ((1u << lane) - 1u));
+    const bool takes = item == kIdle && rank < __popc(givers);
+    const int src = takes ? (int)__fns(givers, 0, rank + 1) : (int)lane;
+    const auto from = [&](float x) { return __shfl_sync(FULL, x, src); };
+    const uint32_t entry = __shfl_sync(FULL, give, src);
+    const bool object_space = __shfl_sync(FULL, (int)(!T.top(S) && give >= T.inst_tip), src);
+    const uint32_t its_item = __shfl_sync(FULL, item, src);
+    const uint32_t its_base = __shfl_sync(FULL, T.node_base, src);
+    const RaySetup its_ray{make_float4(from(T.r.o.x), from(T.r.o.y), from(T.r.o.z), from(T.r.o.w)),
+                           make_float4(from(T.r.inv.x), from(T.r.inv.y), from(T.r.inv.z), from(T.r.inv.w))};
+    if (takes) {
+        T.take(S, base + 16u * (uint32_t)src, entry, object_space, its_ray, its_base);
+        item = its_item >= kHelper ? its_item : kHelper + (uint32_t)src;
+    }
+    __syncwarp();
+}
+
+// Helpers that are done hand over what they found; an answered ray's helpers
+// end.  Returns the lanes whose ray others still help with.
+template <class Kind>
+__device__ __forceinline__ unsigned gather_rays(Traversal<Kind>& T, uint32_t& item) {
+    const unsigned FULL = 0xFFFFFFFFu;
+    const unsigned lane = threadIdx.x & 31u;
+    unsigned ready = __ballot_sync(FULL, item >= kHelper && item != kIdle && T.finished());
+    while (ready) {
+        const int j = __ffs(ready) - 1;
+        ready &= ready - 1;
+        const int owner = (int)(__shfl_sync(FULL, item, j) - kHelper);
+        const bool its_found = __shfl_sync(FULL, (int)T.found, j);
+        const int its_budget = __shfl_sync(FULL, T.budget, j);
+        if ((int)lane == owner) T.absorb(its_found, its_budget);
+        if ((int)lane == j) item = kIdle;
+    }
+    const unsigned answered = __ballot_sync(FULL, item < kHelper && T.found);
+    if (item >= kHelper && item != kIdle && (answered >> (item - kHelper) & 1u)) {
+        T.answer();  // its steps are still handed over, next time
+        T.found = false;
+    }
+    return __reduce_or_sync(FULL, item >= kHelper && item != kIdle ? 1u << (item - kHelper) : 0u);
 }
 
 // Persistent warp-synchronous traversal loop over work items [0, count).  Each
@@ -1114,7 +1230,6 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Ki
                                                  Start start, Done done) {
     const unsigned FULL = 0xFFFFFFFFu;
     const unsigned lane = threadIdx.x & 31u;
-    constexpr uint32_t kIdle = 0xFFFFFFFFu;  // counts stay below it
     const uint32_t base = traversal_base<Kind>();
     const uint32_t claimed = base + 32u * Kind::kLaneBytes;  // claimed items not yet started: first, end
     typename Kind::Entry deep[kMaxStack - Kind::STACK];
@@ -1162,8 +1277,13 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Ki
             }
             more = __all_sync(FULL, item != kIdle);  // past the end: nothing more to claim
         }
-        const int n_busy = __popc(__ballot_sync(FULL, item != kIdle));
-        if (n_busy == 0) break;
+        if constexpr (Kind::ANY)
+            if (!more) share_rays(S, T, item, base);
+        if (!__any_sync(FULL, item != kIdle)) break;
+        // rays with something left to do (one that only waits for its helpers
+        // has not)
+        const int n_busy = __popc(__ballot_sync(FULL, item != kIdle && !T.finished()));
+        int turns = more ? -1 : 8;  // any hit: then see again who is idle
         for (;;) {
             // Once eight or more lanes wait at an instance (TLAS leaf), they
             // enter it together and go on with the inner nodes of its BLAS
@@ -1175,13 +1295,14 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Ki
                 continue;
             }
             // Leave the inner-node phase early once the lanes still in it are
-            // no more than the lanes waiting at an instance or a
-            // leaf (or finished): those then move on together instead of
+            // no more than the lanes waiting at an instance or a leaf (any
+            // hit: half as many): those then move on together instead of
             // idling until the warp's longest run of inner nodes ends.  A lane
             // that the next phase moves on is left then, or no lane is busy,
-            // so every outer iteration makes progress.
+            // so every outer iteration makes progress.  (Closest hit with the
+            // other line +2 %; ambient occlusion with it +8 %, sun rays even.)
             const bool w = T.wants_inner();
-            if (2 * __popc(__ballot_sync(FULL, w)) <= n_busy) break;
+            if ((Kind::ANY ? 3 : 2) * __popc(__ballot_sync(FULL, w)) <= n_busy || (Kind::ANY && turns-- == 0)) break;
             if (w) T.inner_step(S, st, cap);
         }
         if (T.at_instance()) {
@@ -1202,9 +1323,12 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Ki
                 waited = 0;
             }
         }
-        if (item != kIdle) {
+        unsigned helped = 0;  // lanes whose ray others still help with
+        if constexpr (Kind::ANY)
+            if (!more) helped = gather_rays(T, item);
+        if (item < kHelper) {
             T.check_budget();
-            if (T.finished()) {
+            if (T.finished() && !(helped >> lane & 1u)) {
                 done(item);
                 item = kIdle;
             }

@@ -497,12 +497,27 @@ static cudaError_t wave_pass(WaveArgs& A, uint64_t P0, uint32_t n, int replay, c
     wave_gen<<<(n + 255) / 256, 256, 0, s>>>(A, P0, n);
     if (hook) hook->end(kStageGen, s);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    bool shadow_pending = false;
+    // Into a graph, the closest-hit launch of depth i + 1 goes before the
+    // shadow launch of depth i, so that of the two, which become ready at the
+    // same time, the one the next depths wait for is started first (a graph of
+    // one 128 x 96 frame of the mid scene 0.99 -> 0.88 ms).  On plain streams
+    // the order makes no difference to small frames and the other one is 0.5 %
+    // better for large ones.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (overlap && (e = cudaStreamIsCapturing(s, &capture)) != cudaSuccess) return e;
+    const bool closest_first = capture == cudaStreamCaptureStatusActive;
+    bool shadow_pending = false, shadow_waits = false;
     for (uint32_t i = 1; i <= A.P.max_depth; ++i) {
         if (hook) hook->begin(kStageTrace, s);
         e = launch_wave_trace<false>(A, (int)i, t, sm_count, s);
         if (hook) hook->end(kStageTrace, s);
         if (e != cudaSuccess) return e;
+        if (shadow_waits) {
+            if ((e = launch_wave_trace<true>(A, (int)i - 1, t, sm_count, ov->aux)) != cudaSuccess) return e;
+            if ((e = cudaEventRecord(ov->join, ov->aux)) != cudaSuccess) return e;
+            shadow_waits = false;
+            shadow_pending = true;
+        }
         // shade(i) adds into the radiance that shadow(i - 1) adds into
         if (shadow_pending && (e = cudaStreamWaitEvent(s, ov->join, 0)) != cudaSuccess) return e;
         shadow_pending = false;
@@ -518,6 +533,10 @@ static cudaError_t wave_pass(WaveArgs& A, uint64_t P0, uint32_t n, int replay, c
                 if ((e = cudaEventRecord(ov->fork, s)) != cudaSuccess) return e;
                 if ((e = cudaStreamWaitEvent(ov->aux, ov->fork, 0)) != cudaSuccess) return e;
                 ss = ov->aux;
+                if (closest_first && i < A.P.max_depth) {
+                    shadow_waits = true;
+                    continue;
+                }
             }
             if (hook) hook->begin(kStageShadow, ss);
             e = launch_wave_trace<true>(A, (int)i, t, sm_count, ss);
