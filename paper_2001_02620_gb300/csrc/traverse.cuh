@@ -1349,8 +1349,9 @@ __device__ __forceinline__ uint32_t trace_ray(const DevScene& S, float wox, floa
     T.bind(traversal_base<Kind>(), deep);
     T.init(S, wox, woy, woz, wdx, wdy, wdz, tmin, tmax, max_steps, st);
     uint32_t none = 0;
-    while (!T.finished()) {
-        T.check_budget();
+    for (;;) {
+        T.check_budget();  // may end the ray
+        if (T.finished()) break;
         if (T.waiting == 2 || T.visited())
             T.resolve(S, st, none);
         else if (T.wants_inner())
