@@ -505,6 +505,7 @@ struct TraversalKind {
     using Entry = std::conditional_t<ANY, uint32_t, uint64_t>;
     static constexpr int kRecs = ANY ? 6 : (UV || RANGE ? 8 : 6);
     static constexpr int kLaneBytes = kRecs * 16 + STACK * (int)sizeof(Entry);
+    static_assert(STACK >= 4 && STACK <= 32, "a node's pushes fit, the tuning's caps lie beyond");
 };
 
 // Stack entries in shared memory: what fits the 228 KB of an SM (less 1 KB a
@@ -513,7 +514,8 @@ struct TraversalKind {
 // beyond 9 in half of a closest-hit frame's node steps and beyond 12 in a
 // sixth, and a lane beyond takes its warp through the slower path.
 constexpr int shared_stack(bool any, int recs, int warps) {
-    return any ? 16 : ((warps > 40 ? 144 : warps > 32 ? 176 : 216) - 16 * recs) / 8;
+    const int fits = ((warps > 40 ? 144 : warps > 32 ? 176 : 216) - 16 * recs) / 8;
+    return any ? 16 : fits > 4 ? fits : 4;
 }
 
 // The ray-query kernels' rays, and the wavefront renderer's.
@@ -756,7 +758,7 @@ struct Traversal {
         const bool push[4] = {hit[0] && !next0, hit[1] && !next1, hit[2] && !next2, hit[3] && !next3};
         cur = next0 ? ref[0] : next1 ? ref[1] : next2 ? ref[2] : ref[3];
         if (!(hit[0] || hit[1] || hit[2] || hit[3])) cur = kRefNone;
-        if (tip - bottom <= kShared - 3 * kStride) {
+        if (tip - bottom + 3 * kStride <= kShared) {
 #pragma unroll
             for (int k = 3; k >= 0; --k)
                 if (push[k]) put_shared(t[k], ref[k]);

@@ -1,0 +1,113 @@
+"""The traversal's dispatch at its edges: short and long queries, deep stacks,
+frames small enough for a lane per sample, rays that are stopped.  Each is
+compared, bit for bit, with the same work done another way by the library;
+tests/test_gpu_tiny.py compares that with the oracle."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2001_02620_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2001_02620_gb300 import build as B
+    B.build()
+    from paper_2001_02620_gb300 import api as A
+    return A
+
+
+@pytest.fixture(scope="module")
+def tiny(api):
+    sc = I.tiny_scene()
+    return sc, api.Scene(sc)
+
+
+@pytest.fixture(scope="module")
+def rays(tiny):
+    lo, hi = I.scene_box(tiny[0])
+    r = np.concatenate([I.rays_toward(150_000, lo - 30, hi + 30, I.instance_origins(tiny[0]), 1.5, seed=5),
+                        I.rays_random(50_000, lo, hi, seed=6, tmax=60.0)])
+    return torch.from_numpy(r[np.random.default_rng(7).permutation(len(r))]).cuda()
+
+
+# warps of a full launch: 152 SMs x 32; its lanes 155,648
+@pytest.mark.parametrize("n", [1, 31, 33, 1000, 4865, 60_000, 155_649])
+@pytest.mark.parametrize("tuning", [dict(), dict(batch=3, block=64), dict(occupancy=48, fetch=16)])
+def test_a_query_does_not_depend_on_its_company(tiny, rays, n, tuning):
+    _, gs = tiny
+    all_hits, all_bits = gs.trace_closest(rays), gs.trace_any(rays)
+    hits, bits = gs.trace_closest(rays[:n], tuning=tuning), gs.trace_any(rays[:n], tuning=tuning)
+    gs.check()
+    assert torch.equal(hits, all_hits[:n])
+    occ = (bits[:, None] >> torch.arange(32, device="cuda", dtype=torch.int32) & 1).reshape(-1)[:n]
+    ref = (all_bits[:, None] >> torch.arange(32, device="cuda", dtype=torch.int32) & 1).reshape(-1)[:n]
+    assert torch.equal(occ, ref)
+    assert torch.equal(occ.bool(), hits[:, 1] != -1)  # the same interval: occluded means hit
+
+
+def test_stacks_deeper_than_shared_memory(api):
+    """A chain-shaped tree over coincident quads keeps three entries per level:
+    64 of its quads stack some 60, four times what shared memory holds."""
+    vv = np.array([[0, 0, 0], [1, 0, 0], [1, 1, 0], [0, 1, 0]], dtype=np.float32)
+    q = np.tile(np.array([[0, 1, 2, 3]], dtype=np.uint32), (60, 1))
+    sc = I.Scene([(vv, q)], I.IDENTITY_XFORM[None].copy(), np.zeros(1, dtype=np.uint32))
+    rng = np.random.default_rng(3)
+    o = np.concatenate([rng.uniform(-0.5, 1.5, size=(500, 2)), np.full((500, 1), 5.0)], 1)
+    r = torch.from_numpy(I.ray_array(o, np.tile([[0.0, 0.0, -1.0]], (500, 1)))).cuda()
+    deep, flat = api.Scene(sc, build_opts=dict(degenerate=1)), api.Scene(sc)
+    for tuning in (dict(), dict(occupancy=48), dict(occupancy=16, fetch=16)):
+        a, b = deep.trace_closest(r, tuning=tuning), deep.trace_any(r, tuning=tuning)
+        deep.check()
+        assert torch.equal(a, flat.trace_closest(r))
+        assert torch.equal(b, flat.trace_any(r))
+    assert (a[:, 1] != -1).sum() > 50
+
+
+def _views(sizes, spps):
+    base, views = 0, []
+    for (w, h), spp in zip(sizes, spps):
+        views.append(dataclasses.replace(I.tiny_view(), w=w, h=h, spp=spp, pixel_base=base))
+        base += w * h
+    return views
+
+
+@pytest.mark.parametrize("sizes,spps", [
+    ([(1, 1)], [1]), ([(61, 47)], [1]), ([(5, 7)], [3]), ([(31, 33)], [8]), ([(31, 33)], [9]),
+    ([(17, 3), (40, 21), (1, 1)], [2, 2, 2]), ([(17, 3), (40, 21)], [2, 3]), ([(192, 152)], [1]),
+    ([(193, 152)], [1])])
+def test_small_frames_equal_the_wavefront(api, tiny, sizes, spps):
+    """Around the rule that takes small frames to the single kernel: images and
+    path logs are those of the wavefront renderer."""
+    sc, gs = tiny
+    views = _views(sizes, spps)
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    params = I.Params(max_depth=4, sun_dir=I.MID_SUN_DIR, sun_E=(2.0, 2.0, 2.0), lights=I.tiny_lights())
+    log = [torch.zeros(api.path_log_words(views, 4), dtype=torch.int32, device="cuda") for _ in range(2)]
+    a = gs.render(views, alb, params, path_log=log[0])
+    b = gs.render(views, alb, params, path_log=log[1], tuning=dict(mode=2))
+    g = api.RenderGraph(gs, views, alb, params)
+    c = g.launch()
+    gs.check()
+    for x, y, z in zip(a, b, c):
+        assert torch.equal(x, y) and torch.equal(x, z)
+    assert torch.equal(log[0], log[1])
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_stopped_rays_are_reported_by_every_renderer(api, tiny, mode):
+    sc, gs = tiny
+    view = dataclasses.replace(I.tiny_view(), w=300, h=200)
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    gs.render([view], alb, I.tiny_params(), max_steps=3, tuning=dict(mode=mode))
+    with pytest.raises(api.N.QrtError) as e:
+        gs.check()
+    assert e.value.code == api.N.QRT_ERR_STEP_LIMIT
+    gs.check()  # cleared after reading
