@@ -137,7 +137,9 @@ typedef struct {
  *                  16 (up to 128 registers a thread), 24 (80), 32 (64,
  *                  default), 40 (48) or 48 (40); more warps hide the latency
  *                  of the dependent node loads, at the price of spills
- *   mode           renderer: 0 = default (wavefront), 1 = single persistent
+ *   mode           renderer: 0 = default (wavefront; small frames, of a
+ *                  few ten thousand paths, the single kernel with a lane per
+ *                  sample), 1 = single persistent
  *                  kernel (a lane renders whole pixels), 2 = wavefront (stages
  *                  gen / trace / shade / shadow / accumulate over queues; a
  *                  lane of a trace kernel takes a new ray as soon as its own

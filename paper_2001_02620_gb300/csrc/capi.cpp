@@ -885,6 +885,21 @@ int wave_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const
     return rc;
 }
 
+// The samples per pixel of a call small enough for the single-kernel renderer
+// with a lane per sample (kSpreadPathsPerSm); 0: the call is not.
+uint32_t spread_samples(qrt_scene scene, const qrt_view* views, uint32_t n_views, const qrt_params* params) {
+    const qrt_tuning& t = params->tuning;
+    if (t.mode != 0 || t.chunk_log2 != 0 || (params->flags & QRT_FLAG_STAGE_TIMES)) return 0;
+    uint64_t paths = 0;
+    for (uint32_t v = 0; v < n_views; ++v) {
+        if (views[v].spp != views[0].spp) return 0;
+        paths += region_pixels(views[v]) * views[v].spp;
+    }
+    const uint32_t spp = views[0].spp;
+    const uint64_t limit = spp == 1 ? kSpreadPathsPerSm : kSpreadSamplesPerSm;
+    return spp <= 8 && paths <= limit * (uint64_t)scene->sm_count ? spp : 0;
+}
+
 // Enqueues the render (or adjoint) of all views on stream s.  counter serves
 // the single-kernel renderer, workspace (bytes) the wavefront one.
 int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const float* d_albedo,
@@ -897,7 +912,9 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
     int rc = validate_tuning(t);
     if (rc) return rc;
     const bool adjoint = d_grad != nullptr;
-    if (t.mode == 1) {
+    const uint32_t spread =
+        params && !adjoint && !stats && !d_cost ? spread_samples(scene, views, n_views, params) : 0;
+    if (t.mode == 1 || spread) {
         static_assert(sizeof(RenderArgs) < 32000, "kernel parameter block too large");
         RenderArgs* A = new RenderArgs();
         std::memset(A, 0, sizeof(RenderArgs));
@@ -907,6 +924,7 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
         A->counter = counter;
         A->stats = stats;
         A->batch = (uint32_t)t.batch;
+        A->spread = spread;
         rc = make_params(params, A->P);
         if (adjoint) {
             A->P.path_log = nullptr;
@@ -919,7 +937,8 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
             if (rc) break;
             for (uint32_t k = 0; k < cnt; ++k)
                 paths += region_pixels(views[first + k]) * views[first + k].spp;
-            cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+            cudaError_t e = cudaSuccess;
+            if (!spread) e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
             if (e == cudaSuccess) e = launch_render(*A, t, scene->sm_count, s);
             if (e != cudaSuccess) rc = cuda_fail(e, "render launch");
         }

@@ -126,8 +126,21 @@ struct RenderArgs {
     uint64_t n_items;
     uint32_t n_views;
     uint32_t batch;
+    uint32_t spread;  // 0, or the samples per pixel of every view (at most 8): a lane per sample, no counter
     ViewDev views[kMaxViewsPerLaunch];
 };
+
+// Frames of at most this many paths per SM take the single-kernel renderer, a
+// lane per sample, unless the tuning names a renderer.  Measured on one GB300,
+// us, wavefront / single kernel on the tiny, mid and island scenes, depth 5: one
+// sample per pixel, 128 x 96 257 / 161, 929 / 720, 907 / 616; 192 x 144 (182 paths
+// per SM) 285 / 193, 982 / 877, 1053 / 849; 256 x 192 (323 per SM) 318 / 275, 1225
+// / 1169, 1166 / 1249, where the wavefront's warps, full of like rays, draw level.
+// With several samples per pixel they do so sooner: 48 x 40 x 4 (51 per SM) 256
+// / 162, 754 / 529, 739 / 640; 64 x 48 x 4 (81 per SM) 262 / 195, 793 / 850, 795 /
+// 684; 24 x 24 x 16 227 / 186, 703 / 772, 673 / 697 (at most 8 samples, then).
+constexpr uint64_t kSpreadPathsPerSm = 192;
+constexpr uint64_t kSpreadSamplesPerSm = 64;
 
 // Persistent ray-query launch; cursor is a device counter the launch resets.
 cudaError_t launch_trace(bool any, const DevScene& S, const void* rays, uint64_t n, void* hits,

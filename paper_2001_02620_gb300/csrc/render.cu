@@ -5,7 +5,10 @@
 // claims 32*batch consecutive pixels at a time from a global counter, each
 // lane renders all spp samples of its pixel and writes the mean, so the
 // primal needs no atomics and a pixel's value does not depend on how views
-// are batched.  Random numbers: Philox4x32-10 keyed by the render seed with
+// are batched.  Small frames (kSpreadPathsPerSm) are rendered here too, with
+// a lane per sample and few of them to a warp: such a frame lasts as long as
+// its longest path, here once instead of a longest ray per depth, and without
+// the wavefront's dozen launches.  Random numbers: Philox4x32-10 keyed by the render seed with
 // counter (global pixel lo, global pixel hi, sample, bounce).
 //
 // Per path (Section 5.4, "Shading": a path tracer with progressive
@@ -198,63 +201,100 @@ __device__ __forceinline__ int find_view(const RenderArgs& A, uint64_t item) {
 
 template <int STACK, int FETCH, bool ADJ>
 __global__ void __launch_bounds__(256) render_kernel(const __grid_constant__ RenderArgs A) {
-    const int lane = threadIdx.x & 31;
+    const uint32_t lane = threadIdx.x & 31;
     const uint32_t D = A.P.max_depth;
     uint32_t err = 0;
     uint64_t bad = ~0ull;
     TraceStats st{0, 0, 0, 0, 0, 0};
+    // Either a warp claims 32 * batch pixels at a time and a lane renders all
+    // samples of its pixel; or (A.spread = samples per pixel, for small frames)
+    // pixels are dealt out, as few to a warp as it takes for the launch's warps
+    // to hold them all, and each sample has a lane of its own, so that few
+    // paths wait for another's divergent steps.
+    const uint32_t U = ADJ ? 0u : A.spread;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    uint64_t base = 0;
+    uint32_t take = 32u * A.batch;  // pixels per claim
+    if (U) {
+        take = (uint32_t)min((uint64_t)(32u / U), (A.n_items + warps - 1) / warps);
+        base = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * take;
+    }
     for (;;) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(A.counter, 32ull * A.batch);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (!U) {
+            if (lane == 0) base = atomicAdd(A.counter, (unsigned long long)take);
+            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        }
         if (base >= A.n_items) break;
-        for (uint32_t k = 0; k < A.batch; ++k) {
-            const uint64_t item = base + 32ull * k + lane;
-            if (item >= A.n_items) break;
-            const ViewDev& V = A.views[find_view(A, item)];
-            const uint64_t pix = item - V.item_begin;
-            uint32_t x, y;
-            const uint64_t gpix = view_pixel(V, pix, &x, &y);
-            const float inv_spp = __frcp_rn((float)V.spp);
-            if (!ADJ) {
-                float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f;
-                for (uint32_t s = 0; s < V.spp; ++s) {
-                    float L[3];
-                    const uint64_t g = V.path_begin + pix * V.spp + s;
-                    uint32_t* log = A.P.path_log ? A.P.path_log + g * path_log_words(D) : nullptr;
-                    float* rlog = A.P.ray_log ? ray_log_rec(A.P, g, 1) : nullptr;
-                    const uint32_t e = path_sample<STACK, FETCH>(A, V, x, y, gpix, V.sample_base + s, 0, L, nullptr,
-                                                                 nullptr, log, rlog, &st);
-                    if (e) {
-                        err |= e;
-                        bad = min(bad, item);
+        for (uint32_t k = 0; k < take; k += 32) {
+            const uint32_t in = U ? lane / U : k + lane;
+            const uint64_t item = base + in;
+            const bool valid = in < take && item < A.n_items;
+            float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f;
+            uint32_t spp = 1;
+            float* out = nullptr;
+            if (valid) {
+                const ViewDev& V = A.views[find_view(A, item)];
+                const uint64_t pix = item - V.item_begin;
+                uint32_t x, y;
+                const uint64_t gpix = view_pixel(V, pix, &x, &y);
+                spp = V.spp;
+                if (!ADJ) {
+                    out = V.out + 3 * pix;
+                    const uint32_t s0 = U ? lane % U : 0u, s1 = U ? s0 + 1u : spp;
+                    for (uint32_t s = s0; s < s1; ++s) {
+                        float L[3];
+                        const uint64_t g = V.path_begin + pix * spp + s;
+                        uint32_t* log = A.P.path_log ? A.P.path_log + g * path_log_words(D) : nullptr;
+                        float* rlog = A.P.ray_log ? ray_log_rec(A.P, g, 1) : nullptr;
+                        const uint32_t e = path_sample<STACK, FETCH>(A, V, x, y, gpix, V.sample_base + s, 0, L, nullptr,
+                                                                     nullptr, log, rlog, &st);
+                        if (e) {
+                            err |= e;
+                            bad = min(bad, item);
+                        }
+                        acc0 = __fadd_rn(acc0, L[0]);
+                        acc1 = __fadd_rn(acc1, L[1]);
+                        acc2 = __fadd_rn(acc2, L[2]);
                     }
-                    acc0 = __fadd_rn(acc0, L[0]);
-                    acc1 = __fadd_rn(acc1, L[1]);
-                    acc2 = __fadd_rn(acc2, L[2]);
-                }
-                float* out = V.out + 3 * pix;
-                out[0] = __fdiv_rn(acc0, (float)V.spp);
-                out[1] = __fdiv_rn(acc1, (float)V.spp);
-                out[2] = __fdiv_rn(acc2, (float)V.spp);
-            } else {
-                const float* di = V.dimage + 3 * pix;
-                const float w[3] = {__fmul_rn(__ldg(di), inv_spp), __fmul_rn(__ldg(di + 1), inv_spp),
-                                    __fmul_rn(__ldg(di + 2), inv_spp)};
-                if (w[0] == 0.f && w[1] == 0.f && w[2] == 0.f) continue;
-                for (uint32_t s = 0; s < V.spp; ++s) {
-                    float L[3], L2[3];
-                    uint32_t e = path_sample<STACK, FETCH>(A, V, x, y, gpix, V.sample_base + s, 0, L, nullptr,
-                                                           nullptr, nullptr, nullptr, &st);
-                    e |= path_sample<STACK, FETCH>(A, V, x, y, gpix, V.sample_base + s, 1, L2, L, w, nullptr,
-                                                   nullptr, &st);
-                    if (e) {
-                        err |= e;
-                        bad = min(bad, item);
+                } else {
+                    const float inv_spp = __frcp_rn((float)spp);
+                    const float* di = V.dimage + 3 * pix;
+                    const float w[3] = {__fmul_rn(__ldg(di), inv_spp), __fmul_rn(__ldg(di + 1), inv_spp),
+                                        __fmul_rn(__ldg(di + 2), inv_spp)};
+                    if (w[0] == 0.f && w[1] == 0.f && w[2] == 0.f) continue;
+                    for (uint32_t s = 0; s < spp; ++s) {
+                        float L[3], L2[3];
+                        uint32_t e = path_sample<STACK, FETCH>(A, V, x, y, gpix, V.sample_base + s, 0, L, nullptr,
+                                                               nullptr, nullptr, nullptr, &st);
+                        e |= path_sample<STACK, FETCH>(A, V, x, y, gpix, V.sample_base + s, 1, L2, L, w, nullptr,
+                                                       nullptr, &st);
+                        if (e) {
+                            err |= e;
+                            bad = min(bad, item);
+                        }
                     }
                 }
             }
+            if (U > 1) {  // the samples' sum in sample order, as one lane forms it
+                __syncwarp();
+                float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+                for (uint32_t s = 0; s < U; ++s) {
+                    const int src = (int)min(31u, in * U + s);
+                    s0 = __fadd_rn(s0, __shfl_sync(0xFFFFFFFFu, acc0, src));
+                    s1 = __fadd_rn(s1, __shfl_sync(0xFFFFFFFFu, acc1, src));
+                    s2 = __fadd_rn(s2, __shfl_sync(0xFFFFFFFFu, acc2, src));
+                }
+                acc0 = s0;
+                acc1 = s1;
+                acc2 = s2;
+            }
+            if (!ADJ && valid && (U <= 1 || lane % U == 0)) {
+                out[0] = __fdiv_rn(acc0, (float)spp);
+                out[1] = __fdiv_rn(acc1, (float)spp);
+                out[2] = __fdiv_rn(acc2, (float)spp);
+            }
         }
+        if (U) base += warps * take;
     }
     if (err) {
         atomicOr(A.S.err, err);
@@ -284,8 +324,8 @@ cudaError_t launch_render(const RenderArgs& A, const Tune& t, int sm_count, cuda
     const bool adj = A.grad != nullptr;
     int per_sm = t.blocks_per_sm > 0 ? t.blocks_per_sm : render_occupancy(t, adj);
     if (per_sm < 1) per_sm = 1;
-    uint64_t want = (A.n_items + (uint64_t)t.block - 1) / (uint64_t)t.block;
     uint64_t grid = (uint64_t)sm_count * (uint64_t)per_sm;
+    const uint64_t want = A.spread ? A.n_items : (A.n_items + (uint64_t)t.block - 1) / (uint64_t)t.block;
     if (want < grid) grid = want;
     if (grid < 1) grid = 1;
     const dim3 g((unsigned)grid), b((unsigned)t.block);
