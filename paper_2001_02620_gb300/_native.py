@@ -128,6 +128,8 @@ class QrtError(RuntimeError):
 def lib():
     """The loaded libqrt.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):

@@ -11,14 +11,30 @@ from . import _native as N
 from .inputs import Params, View
 
 
+# The current stream's handle without the Stream object that
+# torch.cuda.current_stream() makes around it: a ray query over a few rays is
+# bound by the host, and of its 27 us that took 3.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _ptr(t: torch.Tensor | None) -> int | None:
     return None if t is None else t.data_ptr()
+
+
+_NO_TUNING = C.byref(N.qrt_tuning())  # all defaults; the library only reads it
+
+
+def _tuning_ref(tuning: dict | None):
+    return C.byref(make_tuning(tuning)) if tuning else _NO_TUNING
 
 
 def make_tuning(tuning: dict | None) -> N.qrt_tuning:
@@ -153,8 +169,7 @@ class Scene:
         n = rays.shape[0]
         if hits is None:
             hits = torch.empty((n, 4), dtype=torch.int32, device=rays.device)
-        t = make_tuning(tuning)
-        N.check(N.lib().qrt_trace_closest(self.handle, _ptr(rays), n, _ptr(hits), C.byref(t),
+        N.check(N.lib().qrt_trace_closest(self.handle, _ptr(rays), n, _ptr(hits), _tuning_ref(tuning),
                                           _stream(stream)))
         return hits
 
@@ -164,8 +179,7 @@ class Scene:
         n = rays.shape[0]
         if bits is None:
             bits = torch.empty(((n + 31) // 32,), dtype=torch.int32, device=rays.device)
-        t = make_tuning(tuning)
-        N.check(N.lib().qrt_trace_any(self.handle, _ptr(rays), n, _ptr(bits), C.byref(t),
+        N.check(N.lib().qrt_trace_any(self.handle, _ptr(rays), n, _ptr(bits), _tuning_ref(tuning),
                                       _stream(stream)))
         return bits
 

@@ -57,10 +57,13 @@ static cudaError_t launch_variant(const DevScene& S, const float4* rays, uint64_
     // 32-bit item numbers: more rays than kMaxItems go in several launches
     for (uint64_t k = 0; k < n; k += kMaxItems) {
         const uint32_t m = (uint32_t)std::min(n - k, kMaxItems);
-        if ((e = cudaMemsetAsync(cursor, 0, sizeof(*cursor), s)) != cudaSuccess) return e;
         // at most one block per ray: a short query has each ray in a warp and
         // mostly on an SM of its own
         const unsigned grid = std::min((uint32_t)(sm_count * per_sm), m);
+        // rays beyond the launch's lanes are claimed from the cursor
+        if (m > (uint64_t)grid * t.block &&
+            (e = cudaMemsetAsync(cursor, 0, sizeof(*cursor), s)) != cudaSuccess)
+            return e;
         trace_kernel<ANY, FETCH, OCC, STATS><<<grid, t.block, smem, s>>>(
             S, rays + 2 * k, m, k, ANY ? nullptr : hits + k, ANY ? occ + k / 32 : nullptr, max_steps,
             reinterpret_cast<uint32_t*>(cursor), (uint32_t)t.batch, stats, t.stack);

@@ -72,7 +72,11 @@ __device__ __forceinline__ void push(uint32_t* queue, uint32_t* count, uint32_t 
 __global__ void __launch_bounds__(256) wave_gen(const __grid_constant__ WaveArgs A, uint64_t P0,
                                                 uint32_t n) {
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j == 0) A.B.ctr[kCtrStride * 1 + kCtrClosest] = n;  // queue of depth 1 holds every path
+    // the counters of every depth start at zero; the queue of depth 1 holds
+    // every path
+    if (blockIdx.x == 0)
+        for (uint32_t k = threadIdx.x; k < kCtrStride * (A.P.max_depth + 2); k += blockDim.x)
+            A.B.ctr[k] = k == kCtrStride * 1 + kCtrClosest ? n : 0u;
     if (j >= n) return;
     const uint64_t g = P0 + j;
     const ViewDev& V = A.views[find_view_by_path(A, g)];
@@ -491,8 +495,7 @@ static cudaError_t wave_pass(WaveArgs& A, uint64_t P0, uint32_t n, int replay, c
                              int sm_count, cudaStream_t s, StageHook* hook, const WaveStreams* ov) {
     const bool overlap = ov && ov->aux && (A.P.sun_on || A.P.n_lights);
     A.P0 = P0;
-    cudaError_t e = cudaMemsetAsync(A.B.ctr, 0, sizeof(uint32_t) * kCtrStride * (A.P.max_depth + 2), s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     if (hook) hook->begin(kStageGen, s);
     wave_gen<<<(n + 255) / 256, 256, 0, s>>>(A, P0, n);
     if (hook) hook->end(kStageGen, s);
