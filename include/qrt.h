@@ -147,7 +147,8 @@ typedef struct {
  *   chunk_log2     wavefront: paths per chunk = 2^chunk_log2 (10..26); 0 =
  *                  fit the call: the smallest 2^k >= its paths, k in
  *                  10..25.  Sets the size of the per-stream workspace
- *                  (about 164 B per path; it grows when a call needs more) */
+ *                  (about 164 B per path, and the adjoint's kept hits; it
+ *                  grows when a call needs more) */
 typedef struct {
     uint32_t block;
     uint32_t blocks_per_sm;
@@ -338,10 +339,11 @@ int qrt_render_spp_static(qrt_scene scene, const qrt_view* views, uint32_t n_vie
  * into d_grad_albedo (DEVICE float [n_quads*3], accumulated, not cleared).
  * Paths are recomputed from their random streams instead of being stored
  * (path replay); contributions are added with FP32 atomics.  Per path the
- * wavefront renderer keeps only its radiance and one visibility bit per
- * shadow ray of depths 1..32, so its replay traces the closest-hit rays again
- * but not those shadow rays.  d_dimage: host array of n_views DEVICE
- * pointers, each float [h*w*3]. */
+ * wavefront renderer keeps its radiance, one visibility bit per sun shadow ray
+ * of depths 1..32 and, for as many depths as 8 GB of the per-stream workspace
+ * hold (16 bytes per path and depth, 24 with textures; none where that memory
+ * cannot be had), the closest hits; its replay traces the other rays again.
+ * d_dimage: host array of n_views DEVICE pointers, each float [h*w*3]. */
 int qrt_render_adjoint(qrt_scene scene, const qrt_view* views, uint32_t n_views,
                        const float* d_albedo, const float* const* d_dimage,
                        float* d_grad_albedo, const qrt_params* params, qrt_stream stream);

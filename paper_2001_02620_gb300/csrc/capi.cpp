@@ -117,6 +117,7 @@ struct StreamSlot {
     unsigned long long* counter = nullptr;
     void* ws = nullptr;
     size_t ws_bytes = 0;
+    size_t ws_refused = ~size_t(0);  // the least optional size that could not be had
     WaveStreams ov;  // second stream for overlapping shadow and closest-hit launches
 };
 
@@ -805,13 +806,16 @@ int make_params(const qrt_params* p, ParamsDev& P) {
     return QRT_OK;
 }
 
-// Ensures sl holds a wavefront workspace of at least `bytes`.  Allocation is
-// refused while the stream is being captured.
-int ensure_workspace(StreamSlot& sl, size_t bytes, cudaStream_t s) {
-    if (sl.ws_bytes >= bytes) return QRT_OK;
+// Ensures sl holds a wavefront workspace of at least `bytes`, and of `bytes` +
+// `more` where it has to be allocated anew anyway or the memory is there.
+// Allocation is refused while the stream is being captured.
+int ensure_workspace(StreamSlot& sl, size_t bytes, size_t more, cudaStream_t s) {
+    if (bytes + more >= sl.ws_refused) more = 0;
+    if (sl.ws_bytes >= bytes + more) return QRT_OK;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(s, &cs);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
+    if (cs != cudaStreamCaptureStatusNone && sl.ws_bytes >= bytes) return QRT_OK;
     if (cs != cudaStreamCaptureStatusNone)
         return fail(QRT_ERR_NOT_READY,
                     "wavefront workspace must be allocated before capture: render once on this "
@@ -822,9 +826,15 @@ int ensure_workspace(StreamSlot& sl, size_t bytes, cudaStream_t s) {
     cudaFree(sl.ws);
     sl.ws = nullptr;
     sl.ws_bytes = 0;
-    e = cudaMalloc(&sl.ws, bytes);
+    e = cudaMalloc(&sl.ws, bytes + more);
+    if (e == cudaErrorMemoryAllocation && more) {
+        cudaGetLastError();
+        sl.ws_refused = bytes + more;
+        more = 0;
+        e = cudaMalloc(&sl.ws, bytes);
+    }
     if (e != cudaSuccess) return cuda_fail(e, "wavefront workspace");
-    sl.ws_bytes = bytes;
+    sl.ws_bytes = bytes + more;
     return QRT_OK;
 }
 
@@ -859,8 +869,14 @@ int wave_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const
     W.capacity = cap;
     W.batch = (uint32_t)t.batch;
     W.cost_on = d_cost != nullptr;
-    wave_carve(workspace, cap, adjoint, W.B);
     int rc = make_params(params, W.P);
+    uint32_t stored = 0;  // depths whose hits the workspace has room for
+    const bool tex = rc == QRT_OK && W.P.tex_res != 0;
+    if (adjoint && rc == QRT_OK) {
+        stored = wave_stored_depths(cap, W.P.max_depth);
+        while (stored && wave_workspace_bytes(cap, true) + wave_stored_bytes(cap, stored, tex) > ws_bytes) --stored;
+    }
+    wave_carve(workspace, cap, adjoint, stored, tex, W.B);
     if (adjoint) {
         W.P.path_log = nullptr;
         W.P.ray_log = nullptr;
@@ -967,7 +983,12 @@ int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* vi
     if (rc) return rc;
     if (t.mode == 2) {
         // one workspace per stream, sized for the adjoint so both fit
-        rc = ensure_workspace(sl, wave_workspace_bytes(1ull << t.chunk_log2, true), s);
+        const uint64_t cap = 1ull << t.chunk_log2;
+        size_t more = 0;
+        if (adjoint && params && params->max_depth >= 1 && params->max_depth <= 256)
+            more = wave_stored_bytes(cap, wave_stored_depths(cap, params->max_depth),
+                                     params->d_tex && params->tex_res);
+        rc = ensure_workspace(sl, wave_workspace_bytes(cap, true), more, s);
         if (rc) return rc;
         // the second stream is made outside capture; a capture started
         // before the first render on this stream runs the stages in order
@@ -980,7 +1001,6 @@ int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* vi
         }
         if (sl.ov.aux) *ov = &sl.ov;
     }
-    (void)adjoint;
     *ws = sl.ws;
     *ws_bytes = sl.ws_bytes;
     return QRT_OK;

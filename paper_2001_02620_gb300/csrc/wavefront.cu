@@ -16,7 +16,8 @@
 //              timed stage by stage; shade i+1 waits for it)
 //   accumulate mean over each pixel's samples, summed in sample order
 // The adjoint runs the chunk twice: a primal pass that leaves each path's
-// radiance in Ltot, then a replay pass whose shade stage adds
+// radiance in Ltot and its hits in hits[], then a replay pass whose shade stage
+// follows the paths through those hits again and adds
 // w * (Ltot - sun terms before vertex i) / a_i into the albedo gradient.
 // The primal also records which of the path's shadow rays of depths 1..32
 // were unoccluded (bit i-1 in the spare w lane of its radiance), so the
@@ -401,7 +402,7 @@ static cudaError_t launch_wave_trace(const WaveArgs& A, int depth, const Tune& t
     return launch_wave_trace_uv<ANY, false>(A, depth, t, sm_count, s);
 }
 
-void wave_carve(void* base, uint64_t C, bool adjoint, WaveBufs& B) {
+void wave_carve(void* base, uint64_t C, bool adjoint, uint32_t stored, bool tex, WaveBufs& B) {
     char* p = static_cast<char*>(base);
     auto take = [&](size_t bytes) {
         char* r = p;
@@ -425,6 +426,10 @@ void wave_carve(void* base, uint64_t C, bool adjoint, WaveBufs& B) {
     B.cost = reinterpret_cast<uint32_t*>(take(4 * C));
     B.Ltot = adjoint ? reinterpret_cast<float4*>(take(16 * C)) : nullptr;
     B.ctr = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * kCtrStride * 258));
+    B.stored = stored;
+    B.stride = C;  // a multiple of 1024
+    B.hits = stored ? reinterpret_cast<uint4*>(take(16 * C * stored)) : nullptr;
+    B.uvs = stored && tex ? reinterpret_cast<float2*>(take(8 * C * stored)) : nullptr;
 }
 
 // Scratch of qrt_render_spp_static.  It lives as long as the library is
@@ -510,11 +515,27 @@ static cudaError_t wave_pass(WaveArgs& A, uint64_t P0, uint32_t n, int replay, c
     if (overlap && (e = cudaStreamIsCapturing(s, &capture)) != cudaSuccess) return e;
     const bool closest_first = capture == cudaStreamCaptureStatusActive;
     bool shadow_pending = false, shadow_waits = false;
+    uint4* const hit = A.B.hit;
+    float2* const hit_uv = A.B.hit_uv;
+    struct Restore {  // of the buffers that depths beyond the stored ones share
+        WaveBufs& B;
+        uint4* hit;
+        float2* uv;
+        ~Restore() {
+            B.hit = hit;
+            B.hit_uv = uv;
+        }
+    } restore{A.B, hit, hit_uv};
     for (uint32_t i = 1; i <= A.P.max_depth; ++i) {
-        if (hook) hook->begin(kStageTrace, s);
-        e = launch_wave_trace<false>(A, (int)i, t, sm_count, s);
-        if (hook) hook->end(kStageTrace, s);
-        if (e != cudaSuccess) return e;
+        const bool kept = i <= A.B.stored;  // by the first pass, for the replay
+        A.B.hit = kept ? A.B.hits + (i - 1) * A.B.stride : hit;
+        A.B.hit_uv = kept && A.B.uvs ? A.B.uvs + (i - 1) * A.B.stride : hit_uv;
+        if (!(replay && kept)) {
+            if (hook) hook->begin(kStageTrace, s);
+            e = launch_wave_trace<false>(A, (int)i, t, sm_count, s);
+            if (hook) hook->end(kStageTrace, s);
+            if (e != cudaSuccess) return e;
+        }
         if (shadow_waits) {
             if ((e = launch_wave_trace<true>(A, (int)i - 1, t, sm_count, ov->aux)) != cudaSuccess) return e;
             if ((e = cudaEventRecord(ov->join, ov->aux)) != cudaSuccess) return e;

@@ -111,3 +111,44 @@ def test_stopped_rays_are_reported_by_every_renderer(api, tiny, mode):
         gs.check()
     assert e.value.code == api.N.QRT_ERR_STEP_LIMIT
     gs.check()  # cleared after reading
+
+
+@pytest.mark.parametrize("tex", [False, True])
+def test_adjoint_with_hits_kept_for_some_depths(api, tiny, tex):
+    """The adjoint's replay follows the hits of its first pass for as many depths
+    as the workspace has room for and traces the others: a workspace made by a
+    render (no room) or by a shallower adjoint, which a captured call may not
+    grow, gives the gradient of one with room for every depth."""
+    sc, gs = tiny
+    view = dataclasses.replace(I.tiny_view(), w=96, h=80, spp=3)
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    dimg = torch.from_numpy(np.random.default_rng(9).normal(size=(80, 96, 3)).astype(np.float32)).cuda()
+
+    def params(depth):
+        p = I.Params(max_depth=depth, sun_dir=I.MID_SUN_DIR, sun_E=(2.0, 2.0, 2.0), lights=I.tiny_lights())
+        if tex:
+            p.tex = torch.from_numpy(I.face_textures(sc.n_quads)).cuda()
+        return p
+
+    deep = params(4)
+    ref = gs.adjoint([view], alb, [dimg], torch.zeros_like(alb), deep)
+    gs.check()
+    assert float(ref.abs().max()) > 0
+    for before in (None, 2):
+        s = torch.cuda.Stream()
+        grad = torch.zeros_like(alb)
+        with torch.cuda.stream(s):
+            gs.render([view], alb, deep, tuning=dict(mode=2))
+            if before:
+                gs.adjoint([view], alb, [dimg], torch.zeros_like(alb), params(before))
+            s.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                gs.adjoint([view], alb, [dimg], grad, deep)
+            grad.zero_()
+            g.replay()
+        torch.cuda.synchronize()
+        gs.check()
+        # the same terms added by FP32 atomics in another order: at most a few
+        # hundred terms to a quad, each rounded to 2^-24 of the sum of their sizes
+        torch.testing.assert_close(grad, ref, rtol=1e-4, atol=1e-5 * float(ref.abs().max()))
