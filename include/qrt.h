@@ -136,7 +136,9 @@ typedef struct {
  *   occupancy      trace kernels' register budget as resident warps per SM:
  *                  16 (up to 128 registers a thread), 24 (80), 32 (64,
  *                  default), 40 (48) or 48 (40); more warps hide the latency
- *                  of the dependent node loads, at the price of spills
+ *                  of the dependent node loads, at the price of spills.
+ *                  With block and occupancy both 0, closest-hit ray queries run
+ *                  28 warps (72 registers) in blocks of 128
  *   mode           renderer: 0 = default (wavefront; small frames, of a
  *                  few ten thousand paths, the single kernel with a lane per
  *                  sample), 1 = single persistent

@@ -215,6 +215,8 @@ int check_device(const qrt_scene_s* s) {
 Tune resolve_tuning(const qrt_tuning* t) {
     Tune r;
     if (!t) return r;
+    r.block_given = t->block != 0;
+    r.occupancy_given = t->occupancy != 0;
     if (t->block) r.block = (int)t->block;
     if (t->blocks_per_sm) r.blocks_per_sm = (int)t->blocks_per_sm;
     if (t->batch) r.batch = (int)t->batch;

@@ -63,6 +63,7 @@ struct Tune {
     int stack = 64;         // 32 or 64
     int fetch = 32;         // node fetch bytes per load: 16 or 32
     int occupancy = 32;     // trace kernels: target resident warps per SM (16, 24, 32, 40 or 48)
+    bool block_given = false, occupancy_given = false;  // by the caller; else a kernel's own default may differ
     int mode = 2;           // 1 = single persistent kernel, 2 = wavefront
     int chunk_log2 = 0;     // wavefront paths per chunk = 2^chunk_log2; 0 = fit the call
 };
