@@ -254,7 +254,7 @@ def bench_trace(api, scene, view, d_alb, params, dev, tuning=None, n=1 << 22):
     of the workload's view: camera rays, first diffuse bounces, shadow rays.
     The query kernels return each hit's (u, v), which the render's
     closest-hit kernel drops, so they carry more state: each query is timed
-    with the render's register budget and with 32 warps/SM, the faster
+    with the render's register budget and with 40 warps/SM, the faster
     reported (both budgets give the same hits)."""
     import torch
     out = {}

@@ -133,8 +133,9 @@ def tune(scene, view, albedo, params, space: dict | None = None, reps: int = 3,
     Every candidate is timed on a proxy view of at most proxy_paths paths; when the
     view is larger, the `finalists` fastest are timed again on the view
     itself and the fastest there wins.  (A proxy renders from a warm L2 and
-    a smaller working set: on a scene of tens of GB the full frame preferred
-    40 resident warps per SM, 2.6 % faster, where the proxy chose 32.)"""
+    a smaller working set: with kernels that spilled at 64 registers, the full
+    frame of a scene of tens of GB ran 2.6 % faster at 40 resident warps per
+    SM, where the proxy chose 32.)"""
     import torch
 
     from . import _native as N

@@ -59,7 +59,7 @@ constexpr int occupancy_regs(int warps) { return (65536 / (32 * warps)) & ~7; }
 struct Tune {
     int block = 256;
     int blocks_per_sm = 0;  // 0 = occupancy maximum
-    int batch = 1;          // single kernel: 32-pixel groups a warp claims; trace kernels: rays a lane claims
+    int batch = 1;          // single kernel: 32-pixel groups a warp claims; trace kernels: rays claimed for each idle lane near a queue's end
     int stack = 64;         // 32 or 64
     int fetch = 32;         // node fetch bytes per load: 16 or 32
     int occupancy = 32;     // trace kernels: target resident warps per SM (16, 24, 32, 40 or 48)

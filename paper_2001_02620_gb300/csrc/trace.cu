@@ -1,7 +1,7 @@
 // Ray-query kernels behind qrt_trace_closest / qrt_trace_any.  Persistent:
 // a grid of SMs x resident blocks running the warp-synchronous traversal loop
-// (persistent_trace); each lane claims `batch` rays at a time from a global
-// cursor and starts its next ray as soon as its own is done.
+// (persistent_trace); the first rays are dealt out, a warp claims the others
+// from a global cursor, and a lane starts its next ray as soon as its own is done.
 #include <algorithm>
 
 #include "launch.h"

@@ -30,18 +30,18 @@
 // Execution.  Persistent kernels run persistent_trace: each lane of a warp
 // holds one ray; the warp tests inner nodes together, enters instances in
 // groups, then lets every other lane enter its instance or test one leaf;
-// finished lanes take the next ray at once (claimed one atomic per warp).
-// What bounds it is the issue slots (65 to 75 % busy at 13 to 17 active lanes
-// of 32; some 430 warp instructions per node step, all phases counted) and,
+// finished lanes take the next ray at once (claimed for the warp, see there).
+// What bounds it is the issue slots (60 to 70 % busy at 13 to 16 active lanes
+// of 32; some 410 warp instructions per node step, all phases counted) and,
 // behind them, each ray's chain of dependent node loads, hidden by resident
 // warps.  So the registers hold what a node test reads and shared memory the
 // rest of a ray and its stack: 64 registers (32 warps an SM) without spills.
 // Left to the compiler, the state spilled 476 bytes a thread at 48 registers,
 // the 64-entry stacks lay in local memory, a node test sorted its children and
 // the FP64 re-test sat in the leaf loop.  That against this on one GB300, ms:
-// 2 M diffuse bounces on the mid scene 5.6 -> 2.95, 1.5 M sun rays 1.60 ->
-// 0.81, 1 M rays of ambient occlusion on the island (0.42 re-tests a ray) 1.95
-// -> 0.86, the mid frame 17.7 -> 10.7, the island frame 33.9 -> 21.3.
+// 2 M diffuse bounces on the mid scene 5.62 -> 2.88, 1.5 M sun rays 1.63 ->
+// 0.81, 1 M rays of ambient occlusion on the island (0.40 re-tests a ray) 1.98
+// -> 0.84, the mid frame 17.9 -> 10.4, the island frame 33.6 -> 20.1.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -1218,9 +1218,10 @@ __device__ __forceinline__ unsigned gather_rays(Traversal<Kind>& T, uint32_t& it
 // The first items are dealt out: L to each warp, as many as it takes for the
 // launch's warps to hold them all, at most 32.  So a short queue is spread one
 // ray to a warp and over all SMs, where no ray waits for another's divergent
-// steps.  Later ones are claimed from *cursor (zero at the launch), `batch` a
-// lane and one atomic for the idle lanes of a warp, so a finished lane never
-// waits for the slowest ray of its warp.
+// steps.  Later ones are claimed from *cursor (zero at the launch), one atomic
+// for a warp: 32 items while plenty are left, then `batch` for each idle lane.
+// A finished lane takes the next of them at once and never waits for the
+// slowest ray of its warp.
 //
 // Per outer iteration the warp first tests inner nodes together (lanes that
 // reach a BLAS leaf postpone it and keep traversing; lanes waiting at
