@@ -71,6 +71,52 @@ def test_stacks_deeper_than_shared_memory(api):
     assert (a[:, 1] != -1).sum() > 50
 
 
+@pytest.mark.parametrize("quad", ["folded", "triangle"])
+@pytest.mark.parametrize("side", [1.0, -1.0])
+def test_retests_of_a_quad_by_the_triangles_it_hits(api, quad, side):
+    """Rays along z on a grid over a quad (0,0,0) (1,0,0) (1,1,0) v3, its edges
+    and diagonal included, which FP32 leaves to FP64.  Folded, v3 = (1,0,1): a
+    ray with y <= x meets triangle 0 at z = 0 and triangle 1 at z = x - y.
+    Triangle, v3 = v2: only triangle 0 has area.  All numbers are dyadic, so a
+    re-test is exact; FP32 decisions are off by a few units in the last place
+    of 5, and (u, v) are kept in 16 bits (half a step, 7.7e-6)."""
+    v3 = [1, 0, 1] if quad == "folded" else [1, 1, 0]
+    vv = np.array([[0, 0, 0], [1, 0, 0], [1, 1, 0], v3], dtype=np.float32)
+    q = np.array([[0, 1, 2, 3]], dtype=np.uint32)
+    gs = api.Scene(I.Scene([(vv, q)], I.IDENTITY_XFORM[None].copy(), np.zeros(1, dtype=np.uint32)))
+    x, y = (a.ravel() for a in np.meshgrid(np.arange(-2, 19) / 16.0, np.arange(-2, 19) / 16.0))
+    n = len(x)
+    o = np.stack([x, y, np.full(n, 5.0 * side)], 1)
+    r = I.ray_array(o, np.tile([[0.0, 0.0, -side]], (n, 1)))
+    inside = (y >= 0) & (x <= 1) & (y <= x)
+    only0 = quad == "triangle"
+    far = 5.0 - side * (x - y)  # where triangle 1 is met, if it is there
+    for skip in (False, True):  # skip: the interval starts beyond the nearer triangle
+        near = np.full(n, 5.0) if only0 else np.minimum(5.0, far)
+        other = np.full(n, np.inf) if only0 else np.maximum(5.0, far)
+        ok = inside & (np.abs(x - y) >= 1 / 16) if skip else inside
+        if skip:
+            r[:, 3] = np.where(ok, near + 1 / 32, 0.0)
+        t_ref = other if skip else near
+        rt = torch.from_numpy(r).cuda()
+        h = gs.trace_closest(rt).cpu().numpy()
+        bits = gs.trace_any(rt).cpu().numpy()
+        gs.check()
+        hit = h[:, 1] != -1
+        sel = ok if skip else np.ones(n, dtype=bool)
+        want = ok & np.isfinite(t_ref)
+        assert np.array_equal(hit[sel], want[sel])
+        any_hit = (bits[:, None] >> np.arange(32) & 1).reshape(-1)[:n].astype(bool)
+        assert np.array_equal(any_hit[sel], want[sel])
+        w = want & sel
+        t = h[:, 0].copy().view(np.float32)
+        assert np.abs(t[w] - t_ref[w]).max(initial=0.0) <= 8 * 5 * 2.0**-23
+        tri1 = (np.abs(t_ref - 5.0) > 1e-3) & (not only0)
+        u, v = (h[:, 3] & 0xFFFF) / 65535.0, (h[:, 3] >> 16 & 0xFFFF) / 65535.0
+        assert np.abs(u - np.where(tri1, y, x))[w].max(initial=0.0) <= 1e-5
+        assert np.abs(v - np.where(tri1, x, y))[w].max(initial=0.0) <= 1e-5
+
+
 def _views(sizes, spps):
     base, views = 0, []
     for (w, h), spp in zip(sizes, spps):
