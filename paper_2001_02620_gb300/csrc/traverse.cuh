@@ -39,9 +39,9 @@
 // Left to the compiler, the state spilled 476 bytes a thread at 48 registers,
 // the 64-entry stacks lay in local memory, a node test sorted its children and
 // the FP64 re-test sat in the leaf loop.  That against this on one GB300, ms:
-// 2 M diffuse bounces on the mid scene 5.62 -> 2.88, 1.5 M sun rays 1.63 ->
-// 0.81, 1 M rays of ambient occlusion on the island (0.40 re-tests a ray) 1.98
-// -> 0.84, the mid frame 17.9 -> 10.4, the island frame 33.6 -> 20.1.
+// 2 M diffuse bounces on the mid scene 5.59 -> 2.80, 1.5 M sun rays 1.62 ->
+// 0.81, 1 M rays of ambient occlusion on the island (0.40 re-tests a ray) 1.95
+// -> 0.79, the mid frame 16.9 -> 9.9, the island frame 33.1 -> 19.7.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
