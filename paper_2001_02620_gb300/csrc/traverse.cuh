@@ -953,7 +953,11 @@ struct Traversal {
     // Tests the quads of BLAS leaf ref; returns true when an any-hit query is
     // answered.  A quad that FP32 cannot decide, or whose distance is within
     // its error bound of the best hit's, waits for resolve(); while one waits
-    // the traversal goes on, and a second one puts the rest of its leaf back.
+    // the traversal goes on, and the next one puts the rest of its leaf back.
+    // So does a closest-hit ray's next hit of any kind: which of two near hits
+    // keeps its FP32 distance and which gets an FP64 one depends on the order
+    // they are compared in, and that must be the order of the traversal, not
+    // the moment at which the warp came to resolve().
     __device__ __forceinline__ bool leaf(const DevScene& S, TraceStats& st, uint32_t ref) {
         const float4 od = lds4(rec + kObjD);
         const float4 oo = ANY ? lds4(rec + kObjO) : r.o;
@@ -971,6 +975,8 @@ struct Traversal {
                 float u = __int_as_float(0x7fffffff), v = 0.f;
                 if constexpr (ANY) {
                     if (!wait && t > t0 && t < t1) return true;
+                } else if (!wait && t > t0 && t < t1 && waiting) {
+                    wait = true;
                 } else if (!wait && t > t0 && t < t1) {
                     const float ht = lds1(rec + kHT);
                     const float4 hr = lds4(rec + kHit);

@@ -198,3 +198,32 @@ def test_adjoint_with_hits_kept_for_some_depths(api, tiny, tex):
         # the same terms added by FP32 atomics in another order: at most a few
         # hundred terms to a quad, each rounded to 2^-24 of the sum of their sizes
         torch.testing.assert_close(grad, ref, rtol=1e-4, atol=1e-5 * float(ref.abs().max()))
+
+
+def _nearly_coincident(copies, jitter):
+    """The tiny scene with every instance `copies` times, a few units of FP32
+    rounding apart: most rays have several nearest hits within their error
+    bounds of each other."""
+    sc = I.tiny_scene()
+    x = np.repeat(sc.xforms, copies, axis=0).astype(np.float64)
+    x += np.random.default_rng(1).uniform(-jitter, jitter, size=x.shape) * (np.abs(x) + 1.0)
+    return I.Scene(sc.meshes, x.astype(np.float32), np.repeat(sc.mesh_ids, copies))
+
+
+@pytest.mark.parametrize("copies,jitter", [(3, 1e-7), (4, 3e-7), (4, 1e-6)])
+def test_near_ties_do_not_depend_on_the_company(api, copies, jitter):
+    """A hit's bits, its distance included, are the same whatever other rays
+    share the warp and whenever it gets to the FP64 tests."""
+    sc = _nearly_coincident(copies, jitter)
+    gs = api.Scene(sc)
+    lo, hi = I.scene_box(sc)
+    r = torch.from_numpy(I.rays_toward(300_000, lo - 30, hi + 30, I.instance_origins(sc), 1.5, seed=5)).cuda()
+    ref = gs.trace_closest(r)
+    for tuning in (dict(), dict(batch=8), dict(occupancy=32), dict(occupancy=32, block=64), dict(occupancy=24)):
+        assert torch.equal(gs.trace_closest(r, tuning=tuning), ref)
+    for seed in range(3):
+        at = torch.randperm(len(r), device="cuda", generator=torch.Generator("cuda").manual_seed(seed))
+        assert torch.equal(gs.trace_closest(r[at].contiguous()), ref[at])
+    few = torch.cat([gs.trace_closest(r[k:k + 1].contiguous()) for k in range(3000)])
+    gs.check()
+    assert torch.equal(few, ref[:3000])
