@@ -149,8 +149,10 @@ typedef struct {
  *   chunk_log2     wavefront: paths per chunk = 2^chunk_log2 (10..26); 0 =
  *                  fit the call: the smallest 2^k >= its paths, k in
  *                  10..25.  Sets the size of the per-stream workspace
- *                  (about 164 B per path, and the adjoint's kept hits; it
- *                  grows when a call needs more) */
+ *                  (about 192 B per path).  It grows when a call needs more,
+ *                  outside stream capture; one that a captured call used stays
+ *                  until the scene is destroyed, so the capture can be
+ *                  replayed whatever is called on the stream after it */
 typedef struct {
     uint32_t block;
     uint32_t blocks_per_sm;
@@ -342,9 +344,10 @@ int qrt_render_spp_static(qrt_scene scene, const qrt_view* views, uint32_t n_vie
  * Paths are recomputed from their random streams instead of being stored
  * (path replay); contributions are added with FP32 atomics.  Per path the
  * wavefront renderer keeps its radiance, one visibility bit per sun shadow ray
- * of depths 1..32 and, for as many depths as 8 GB of the per-stream workspace
- * hold (16 bytes per path and depth, 24 with textures; none where that memory
- * cannot be had), the closest hits; its replay traces the other rays again.
+ * of depths 1..32 and, for as many depths as 8 GB kept for the stream hold (16
+ * bytes per path and depth, 24 with textures; fewer or none where that memory
+ * cannot be had, or in a capture that would have to allocate it), the closest
+ * hits; its replay traces the other rays again.
  * d_dimage: host array of n_views DEVICE pointers, each float [h*w*3]. */
 int qrt_render_adjoint(qrt_scene scene, const qrt_view* views, uint32_t n_views,
                        const float* d_albedo, const float* const* d_dimage,

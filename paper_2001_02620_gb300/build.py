@@ -21,7 +21,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["trace.cu", "render.cu", "wavefront.cu", "lbvh.cu", "radix_sort.cu"]
 CPP_SOURCES = ["capi.cpp", "bvh_build.cpp"]
 HEADERS = ["qrt_layout.h", "launch.h", "traverse.cuh", "shading.cuh", "wavefront.h", "bvh_build.h",
-           "lbvh.h", "radix_sort.h", "node_quant.h"]
+           "lbvh.h", "radix_sort.h", "node_quant.h", "stream_memory.h"]
 
 
 def _inputs():

@@ -22,6 +22,7 @@
 #include "lbvh.h"
 #include "launch.h"
 #include "radix_sort.h"
+#include "stream_memory.h"
 #include "wavefront.h"
 
 using namespace qrt;
@@ -111,14 +112,24 @@ struct StageTimer : StageHook {
     }
 };
 
-// Scratch of one stream: a work counter for the single-kernel renderer and
-// the wavefront workspace (grown on demand, outside stream capture).
+// Scratch of one stream: a work counter for the single-kernel renderer, the
+// wavefront workspace and the adjoint's kept hits (each grown on demand, outside
+// stream capture; apart, so that the workspace never moves for the hits).
 struct StreamSlot {
+    unsigned long long* counter = nullptr;
+    StreamBuffer ws, hits;
+    std::vector<void*> retired;  // buffers of captured calls, outgrown: freed with the scene
+    WaveStreams ov;  // second stream for overlapping shadow and closest-hit launches
+};
+
+// What a call uses of it (or of a graph's own scratch).
+struct Scratch {
     unsigned long long* counter = nullptr;
     void* ws = nullptr;
     size_t ws_bytes = 0;
-    size_t ws_refused = ~size_t(0);  // the least optional size that could not be had
-    WaveStreams ov;  // second stream for overlapping shadow and closest-hit launches
+    void* hits = nullptr;
+    size_t hits_bytes = 0;
+    const WaveStreams* ov = nullptr;
 };
 
 void destroy_streams(WaveStreams& w) {
@@ -194,7 +205,9 @@ void free_scene(qrt_scene_s* s) {
     cudaFree(s->d_err);
     cudaFree(s->d_counters);
     for (StreamSlot& sl : s->slots) {
-        cudaFree(sl.ws);
+        cudaFree(sl.ws.ptr);
+        cudaFree(sl.hits.ptr);
+        for (void* p : sl.retired) cudaFree(p);
         destroy_streams(sl.ov);
     }
     delete s;
@@ -808,50 +821,54 @@ int make_params(const qrt_params* p, ParamsDev& P) {
     return QRT_OK;
 }
 
-// Ensures sl holds a wavefront workspace of at least `bytes`, and of `bytes` +
-// `more` where it has to be allocated anew anyway or the memory is there.
-// Allocation is refused while the stream is being captured.
-int ensure_workspace(StreamSlot& sl, size_t bytes, size_t more, cudaStream_t s) {
-    if (bytes + more >= sl.ws_refused) more = 0;
-    if (sl.ws_bytes >= bytes + more) return QRT_OK;
+// Device memory for a StreamBuffer of stream s; keeps the CUDA error behind a
+// failure.
+struct DeviceMem {
+    cudaStream_t s;
+    cudaError_t error = cudaSuccess;
+
+    int alloc(void** p, size_t bytes) {
+        error = cudaMalloc(p, bytes);
+        if (error == cudaErrorMemoryAllocation) {
+            cudaGetLastError();  // the caller may go on without
+            return kNoMemory;
+        }
+        return (int)error;
+    }
+    void release(void* p) { cudaFree(p); }
+    int drain() { return (int)(error = cudaStreamSynchronize(s)); }
+};
+
+// Makes sl hold a wavefront workspace of `bytes` and, where that memory can be
+// had, `hits` bytes for kept hits.  Allocation is refused while the stream is
+// being captured.
+int ensure_workspace(StreamSlot& sl, size_t bytes, size_t hits, cudaStream_t s) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaError_t e = cudaStreamIsCapturing(s, &cs);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
-    if (cs != cudaStreamCaptureStatusNone && sl.ws_bytes >= bytes) return QRT_OK;
-    if (cs != cudaStreamCaptureStatusNone)
+    cudaError_t ce = cudaStreamIsCapturing(s, &cs);
+    if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamIsCapturing");
+    const bool capturing = cs != cudaStreamCaptureStatusNone;
+    DeviceMem mem{s};
+    int e = need(sl.ws, bytes, capturing, sl.retired, mem);
+    if (e == kCapturing)
         return fail(QRT_ERR_NOT_READY,
                     "wavefront workspace must be allocated before capture: render once on this "
                     "stream outside capture, or use qrt_render_graph_create");
-    // the old workspace may still be in use by queued work on this stream
-    e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "stream synchronize");
-    cudaFree(sl.ws);
-    sl.ws = nullptr;
-    sl.ws_bytes = 0;
-    e = cudaMalloc(&sl.ws, bytes + more);
-    if (e == cudaErrorMemoryAllocation && more) {
-        cudaGetLastError();
-        sl.ws_refused = bytes + more;
-        more = 0;
-        e = cudaMalloc(&sl.ws, bytes);
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "wavefront workspace");
-    sl.ws_bytes = bytes + more;
+    if (!e && hits) e = want(sl.hits, hits, capturing, sl.retired, mem);
+    if (e) return cuda_fail(mem.error, "wavefront workspace");
     return QRT_OK;
 }
 
 // Enqueues the wavefront render (or adjoint) of all views on stream s in
-// the given workspace; W and R are the caller's storage for the launch
+// the given scratch; W and R are the caller's storage for the launch
 // parameter blocks (so this function allocates nothing).
 int wave_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const float* d_albedo,
                  const float* const* d_dimage, float* d_grad, const qrt_params* params,
-                 const Tune& t, void* workspace, size_t ws_bytes, unsigned long long* stats,
-                 cudaStream_t s, WaveArgs& W, RenderArgs& R, const WaveStreams* ov,
-                 float* const* d_cost = nullptr) {
+                 const Tune& t, const Scratch& scratch, unsigned long long* stats,
+                 cudaStream_t s, WaveArgs& W, RenderArgs& R, float* const* d_cost = nullptr) {
     static_assert(sizeof(WaveArgs) < 32000, "kernel parameter block too large");
     const bool adjoint = d_grad != nullptr;
     const uint64_t cap = 1ull << t.chunk_log2;
-    if (wave_workspace_bytes(cap, adjoint) > ws_bytes)
+    if (wave_workspace_bytes(cap, adjoint) > scratch.ws_bytes)
         return fail(QRT_ERR_INVALID_ARG, "wavefront workspace too small for chunk_log2");
     // a chunk is cut at pixel boundaries, so it must hold all of a pixel's samples
     for (uint32_t v = 0; v < n_views; ++v)
@@ -872,13 +889,13 @@ int wave_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const
     W.batch = (uint32_t)t.batch;
     W.cost_on = d_cost != nullptr;
     int rc = make_params(params, W.P);
-    uint32_t stored = 0;  // depths whose hits the workspace has room for
+    uint32_t stored = 0;  // depths whose hits there is room for
     const bool tex = rc == QRT_OK && W.P.tex_res != 0;
     if (adjoint && rc == QRT_OK) {
         stored = wave_stored_depths(cap, W.P.max_depth);
-        while (stored && wave_workspace_bytes(cap, true) + wave_stored_bytes(cap, stored, tex) > ws_bytes) --stored;
+        while (stored && wave_stored_bytes(cap, stored, tex) > scratch.hits_bytes) --stored;
     }
-    wave_carve(workspace, cap, adjoint, stored, tex, W.B);
+    wave_carve(scratch.ws, cap, adjoint, scratch.hits, stored, tex, W.B);
     if (adjoint) {
         W.P.path_log = nullptr;
         W.P.ray_log = nullptr;
@@ -897,7 +914,7 @@ int wave_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const
         W.n_views = cnt;
         StageHook* hook = (params && (params->flags & QRT_FLAG_STAGE_TIMES)) ? &scene->timer : nullptr;
         // timed stages run in order: overlapping kernels would blur their times
-        cudaError_t e = launch_wave(W, t, scene->sm_count, s, hook, hook ? nullptr : ov);
+        cudaError_t e = launch_wave(W, t, scene->sm_count, s, hook, hook ? nullptr : scratch.ov);
         if (e != cudaSuccess) rc = cuda_fail(e, "wavefront launch");
     }
     return rc;
@@ -918,12 +935,10 @@ uint32_t spread_samples(qrt_scene scene, const qrt_view* views, uint32_t n_views
     return spp <= 8 && paths <= limit * (uint64_t)scene->sm_count ? spp : 0;
 }
 
-// Enqueues the render (or adjoint) of all views on stream s.  counter serves
-// the single-kernel renderer, workspace (bytes) the wavefront one.
+// Enqueues the render (or adjoint) of all views on stream s.
 int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const float* d_albedo,
                    const float* const* d_dimage, float* d_grad, const qrt_params* params,
-                   unsigned long long* counter, void* workspace, size_t ws_bytes,
-                   unsigned long long* stats, cudaStream_t s, const WaveStreams* ov,
+                   const Scratch& scratch, unsigned long long* stats, cudaStream_t s,
                    float* const* d_cost = nullptr) {
     Tune t = resolve_tuning(params ? &params->tuning : nullptr);
     fit_chunk(t, views, n_views);
@@ -939,7 +954,7 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
         A->S = scene->S;
         A->albedo = d_albedo;
         A->grad = d_grad;
-        A->counter = counter;
+        A->counter = scratch.counter;
         A->stats = stats;
         A->batch = (uint32_t)t.batch;
         A->spread = spread;
@@ -956,7 +971,7 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
             for (uint32_t k = 0; k < cnt; ++k)
                 paths += region_pixels(views[first + k]) * views[first + k].spp;
             cudaError_t e = cudaSuccess;
-            if (!spread) e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+            if (!spread) e = cudaMemsetAsync(scratch.counter, 0, sizeof(unsigned long long), s);
             if (e == cudaSuccess) e = launch_render(*A, t, scene->sm_count, s);
             if (e != cudaSuccess) rc = cuda_fail(e, "render launch");
         }
@@ -965,8 +980,8 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
     }
     WaveArgs* W = new WaveArgs();
     RenderArgs* R = new RenderArgs();
-    rc = wave_enqueue(scene, views, n_views, d_albedo, d_dimage, d_grad, params, t, workspace,
-                      ws_bytes, stats, s, *W, *R, ov, d_cost);
+    rc = wave_enqueue(scene, views, n_views, d_albedo, d_dimage, d_grad, params, t, scratch, stats, s,
+                      *W, *R, d_cost);
     delete R;
     delete W;
     return rc;
@@ -974,11 +989,10 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
 
 // Scratch for a plain (non-graph) call on stream s.
 int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* views,
-                   uint32_t n_views, bool adjoint, cudaStream_t s, unsigned long long** counter,
-                   void** ws, size_t* ws_bytes, const WaveStreams** ov) {
+                   uint32_t n_views, bool adjoint, cudaStream_t s, Scratch& out) {
     StreamSlot& sl = scene->slot_for(s);
-    *counter = sl.counter;
-    *ov = nullptr;
+    out = Scratch{};
+    out.counter = sl.counter;
     Tune t = resolve_tuning(params ? &params->tuning : nullptr);
     fit_chunk(t, views, n_views);
     int rc = validate_tuning(t);
@@ -986,11 +1000,11 @@ int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* vi
     if (t.mode == 2) {
         // one workspace per stream, sized for the adjoint so both fit
         const uint64_t cap = 1ull << t.chunk_log2;
-        size_t more = 0;
+        size_t hits = 0;
         if (adjoint && params && params->max_depth >= 1 && params->max_depth <= 256)
-            more = wave_stored_bytes(cap, wave_stored_depths(cap, params->max_depth),
+            hits = wave_stored_bytes(cap, wave_stored_depths(cap, params->max_depth),
                                      params->d_tex && params->tex_res);
-        rc = ensure_workspace(sl, wave_workspace_bytes(cap, true), more, s);
+        rc = ensure_workspace(sl, wave_workspace_bytes(cap, true), hits, s);
         if (rc) return rc;
         // the second stream is made outside capture; a capture started
         // before the first render on this stream runs the stages in order
@@ -1001,10 +1015,12 @@ int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* vi
                 if (e != cudaSuccess) return cuda_fail(e, "overlap stream");
             }
         }
-        if (sl.ov.aux) *ov = &sl.ov;
+        if (sl.ov.aux) out.ov = &sl.ov;
     }
-    *ws = sl.ws;
-    *ws_bytes = sl.ws_bytes;
+    out.ws = sl.ws.ptr;
+    out.ws_bytes = sl.ws.bytes;
+    out.hits = sl.hits.ptr;
+    out.hits_bytes = sl.hits.bytes;
     return QRT_OK;
 }
 
@@ -1026,14 +1042,10 @@ int qrt_render_spp(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
     if (rc) return rc;
     if (n_views == 0) return QRT_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    unsigned long long* ctr;
-    void* ws;
-    size_t wsb;
-    const WaveStreams* ov = nullptr;
-    rc = stream_scratch(scene, params, views, n_views, false, s, &ctr, &ws, &wsb, &ov);
+    Scratch scratch;
+    rc = stream_scratch(scene, params, views, n_views, false, s, scratch);
     if (rc) return rc;
-    return render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, ctr, ws, wsb,
-                          nullptr, s, ov);
+    return render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, scratch, nullptr, s);
 }
 
 // qrt_render_spp without any allocation: the wavefront renderer with its
@@ -1056,14 +1068,14 @@ int qrt_render_spp_static(qrt_scene scene, const qrt_view* views, uint32_t n_vie
     Tune t = resolve_tuning(&tt);
     rc = validate_tuning(t);
     if (rc) return rc;
-    void* ws = nullptr;
-    cudaError_t e = static_workspace(&ws);
+    Scratch scratch;
+    cudaError_t e = static_workspace(&scratch.ws);
     if (e != cudaSuccess) return cuda_fail(e, "static workspace address");
+    scratch.ws_bytes = kStaticWorkspaceBytes;
     WaveArgs W;  // parameter blocks on the stack: nothing is allocated
     RenderArgs R;
-    return wave_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, t, ws,
-                        kStaticWorkspaceBytes, nullptr, reinterpret_cast<cudaStream_t>(stream), W, R,
-                        nullptr);
+    return wave_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, t, scratch, nullptr,
+                        reinterpret_cast<cudaStream_t>(stream), W, R);
 }
 
 // Same as qrt_render_spp with traversal counters added into d_stats (device
@@ -1077,14 +1089,10 @@ int qrt_render_spp_stats(qrt_scene scene, const qrt_view* views, uint32_t n_view
     if (!d_stats || !aligned(d_stats, 8)) return fail(QRT_ERR_INVALID_ARG, "d_stats NULL or unaligned");
     if (n_views == 0) return QRT_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    unsigned long long* ctr;
-    void* ws;
-    size_t wsb;
-    const WaveStreams* ov = nullptr;
-    rc = stream_scratch(scene, params, views, n_views, false, s, &ctr, &ws, &wsb, &ov);
+    Scratch scratch;
+    rc = stream_scratch(scene, params, views, n_views, false, s, scratch);
     if (rc) return rc;
-    return render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, ctr, ws, wsb,
-                          d_stats, s, ov);
+    return render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, scratch, d_stats, s);
 }
 
 int qrt_render_cost(qrt_scene scene, const qrt_view* views, uint32_t n_views, const float* d_albedo,
@@ -1103,14 +1111,10 @@ int qrt_render_cost(qrt_scene scene, const qrt_view* views, uint32_t n_views, co
     if (params && params->tuning.mode == 1)
         return fail(QRT_ERR_INVALID_ARG, "cost maps come from the wavefront renderer (tuning.mode 0 or 2)");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    unsigned long long* ctr;
-    void* ws;
-    size_t wsb;
-    const WaveStreams* ov = nullptr;
-    rc = stream_scratch(scene, params, views, n_views, false, s, &ctr, &ws, &wsb, &ov);
+    Scratch scratch;
+    rc = stream_scratch(scene, params, views, n_views, false, s, scratch);
     if (rc) return rc;
-    return render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, ctr, ws, wsb,
-                          d_stats, s, ov, d_cost);
+    return render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, scratch, d_stats, s, d_cost);
 }
 
 int qrt_trace_stats(qrt_scene scene, int any, const qrt_ray* d_rays, uint64_t n, void* d_out,
@@ -1143,14 +1147,11 @@ int qrt_render_adjoint(qrt_scene scene, const qrt_view* views, uint32_t n_views,
     if (!d_grad_albedo || !aligned(d_grad_albedo, 4))
         return fail(QRT_ERR_INVALID_ARG, "d_grad_albedo is NULL or unaligned");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    unsigned long long* ctr;
-    void* ws;
-    size_t wsb;
-    const WaveStreams* ov = nullptr;
-    rc = stream_scratch(scene, params, views, n_views, true, s, &ctr, &ws, &wsb, &ov);
+    Scratch scratch;
+    rc = stream_scratch(scene, params, views, n_views, true, s, scratch);
     if (rc) return rc;
-    return render_enqueue(scene, views, n_views, d_albedo, d_dimage, d_grad_albedo, params, ctr, ws,
-                          wsb, nullptr, s, ov);
+    return render_enqueue(scene, views, n_views, d_albedo, d_dimage, d_grad_albedo, params, scratch,
+                          nullptr, s);
 }
 
 int qrt_accumulate(float* d_sum, const float* d_frame, float* d_mean, uint64_t n, uint32_t frames,
@@ -1228,8 +1229,12 @@ int qrt_render_graph_create(qrt_scene scene, const qrt_view* views, uint32_t n_v
         delete g;
         return cuda_fail(e, "graph capture");
     }
-    rc = render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, g->d_counter,
-                        g->ws, wsb, nullptr, cs, ov.aux ? &ov : nullptr);
+    Scratch scratch;
+    scratch.counter = g->d_counter;
+    scratch.ws = g->ws;
+    scratch.ws_bytes = wsb;
+    scratch.ov = ov.aux ? &ov : nullptr;
+    rc = render_enqueue(scene, views, n_views, d_albedo, nullptr, nullptr, params, scratch, nullptr, cs);
     cudaGraph_t graph = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
     cudaStreamDestroy(cs);

@@ -443,7 +443,7 @@ static cudaError_t launch_wave_trace(const WaveArgs& A, int depth, const Tune& t
     return launch_wave_trace_uv<ANY, false>(A, depth, t, sm_count, s);
 }
 
-void wave_carve(void* base, uint64_t C, bool adjoint, uint32_t stored, bool tex, WaveBufs& B) {
+void wave_carve(void* base, uint64_t C, bool adjoint, void* hits, uint32_t stored, bool tex, WaveBufs& B) {
     char* p = static_cast<char*>(base);
     auto take = [&](size_t bytes) {
         char* r = p;
@@ -469,6 +469,7 @@ void wave_carve(void* base, uint64_t C, bool adjoint, uint32_t stored, bool tex,
     B.ctr = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * kCtrStride * 258));
     B.stored = stored;
     B.stride = C;  // a multiple of 1024
+    p = static_cast<char*>(hits);
     B.hits = stored ? reinterpret_cast<uint4*>(take(16 * C * stored)) : nullptr;
     B.uvs = stored && tex ? reinterpret_cast<float2*>(take(8 * C * stored)) : nullptr;
 }

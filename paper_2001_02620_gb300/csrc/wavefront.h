@@ -111,8 +111,9 @@ constexpr size_t kStaticWorkspaceBytes = wave_workspace_bytes(1ull << kStaticChu
 // Device address of that array on the current device (looked up once per
 // device with cudaGetSymbolAddress; allocates nothing).
 cudaError_t static_workspace(void** ptr);
-// stored, tex: wave_stored_bytes() more at the end (adjoint)
-void wave_carve(void* base, uint64_t capacity, bool adjoint, uint32_t stored, bool tex, WaveBufs& B);
+// hits: wave_stored_bytes(capacity, stored, tex) apart (adjoint)
+void wave_carve(void* base, uint64_t capacity, bool adjoint, void* hits, uint32_t stored, bool tex,
+                WaveBufs& B);
 cudaError_t launch_wave(WaveArgs& A, const Tune& t, int sm_count, cudaStream_t s, StageHook* hook,
                         const WaveStreams* ov);
 

@@ -227,3 +227,51 @@ def test_near_ties_do_not_depend_on_the_company(api, copies, jitter):
     few = torch.cat([gs.trace_closest(r[k:k + 1].contiguous()) for k in range(3000)])
     gs.check()
     assert torch.equal(few, ref[:3000])
+
+
+def test_captured_calls_outlive_larger_ones(api, tiny):
+    """A render and an adjoint captured on a stream are replayed after calls that
+    take more memory there: an adjoint of the same frame, a deeper one, one with
+    textures, a larger frame."""
+    sc, gs = tiny
+    view = dataclasses.replace(I.tiny_view(), w=96, h=80, spp=3)
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    dimg = torch.from_numpy(np.random.default_rng(9).normal(size=(80, 96, 3)).astype(np.float32)).cuda()
+    wave = dict(mode=2)
+
+    def params(depth, tex=False):
+        p = I.Params(max_depth=depth, sun_dir=I.MID_SUN_DIR, sun_E=(2.0, 2.0, 2.0), lights=I.tiny_lights())
+        if tex:
+            p.tex = torch.from_numpy(I.face_textures(sc.n_quads)).cuda()
+        return p
+
+    p2, p5, p5t = params(2), params(5), params(5, True)
+    (ref,) = gs.render([view], alb, p5, tuning=wave)
+    ref_grad = gs.adjoint([view], alb, [dimg], torch.zeros_like(alb), p2)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        out, grad, scratch = torch.zeros_like(ref), torch.zeros_like(alb), torch.zeros_like(alb)
+        gs.render([view], alb, p5, outs=[out], tuning=wave)
+        s.synchronize()
+        g1, g2 = torch.cuda.CUDAGraph(), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g1, stream=s):
+            gs.render([view], alb, p5, outs=[out], tuning=wave)
+        gs.adjoint([view], alb, [dimg], scratch, p2)
+        s.synchronize()
+        with torch.cuda.graph(g2, stream=s):
+            gs.adjoint([view], alb, [dimg], grad, p2)
+        more = [lambda: gs.adjoint([view], alb, [dimg], scratch, p5),
+                lambda: gs.adjoint([view], alb, [dimg], scratch, p5t),
+                lambda: gs.render([dataclasses.replace(view, w=400, h=300)], alb, p5, tuning=wave)]
+        for call in more:
+            call()
+            out.zero_()
+            grad.zero_()
+            g1.replay()
+            g2.replay()
+            s.synchronize()
+            assert torch.equal(out, ref)
+            # the same terms, added by FP32 atomics in another order
+            torch.testing.assert_close(grad, ref_grad, rtol=1e-4, atol=1e-5 * float(ref_grad.abs().max()))
+    gs.check()
