@@ -149,7 +149,7 @@ typedef struct {
  *   chunk_log2     wavefront: paths per chunk = 2^chunk_log2 (10..26); 0 =
  *                  fit the call: the smallest 2^k >= its paths, k in
  *                  10..25.  Sets the size of the per-stream workspace
- *                  (about 192 B per path).  It grows when a call needs more,
+ *                  (about 196 B per path).  It grows when a call needs more,
  *                  outside stream capture; one that a captured call used stays
  *                  until the scene is destroyed, so the capture can be
  *                  replayed whatever is called on the stream after it */
@@ -320,7 +320,7 @@ int qrt_render_spp(qrt_scene scene, const qrt_view* views, uint32_t n_views,
  * results as qrt_render_spp.
  *
  * It renders with the wavefront renderer, using as scratch a fixed array of
- * about 17 MB compiled into the library (device global memory held on every
+ * about 24 MB compiled into the library (device global memory held on every
  * GPU that loads the library, until the process exits), enough for chunks of
  * 2^17 paths; any number of views and paths is processed chunk by chunk, so
  * a view's spp may be at most 2^17 (larger is rejected with

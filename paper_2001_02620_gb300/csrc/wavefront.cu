@@ -463,7 +463,7 @@ void wave_carve(void* base, uint64_t C, bool adjoint, void* hits, uint32_t store
     B.meta = reinterpret_cast<uint2*>(take(8 * C));
     B.q[0] = reinterpret_cast<uint32_t*>(take(4 * C));
     B.q[1] = reinterpret_cast<uint32_t*>(take(4 * C));
-    B.qs = reinterpret_cast<uint32_t*>(take(4 * C));
+    B.qs = reinterpret_cast<uint32_t*>(take(8 * C));
     B.cost = reinterpret_cast<uint32_t*>(take(4 * C));
     B.Ltot = adjoint ? reinterpret_cast<float4*>(take(16 * C)) : nullptr;
     B.ctr = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * kCtrStride * 258));

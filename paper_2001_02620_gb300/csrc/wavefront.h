@@ -37,7 +37,7 @@ struct WaveBufs {
     float2* hit_uv;  // quad-space (u, v) of the hit (per-face textures)
     uint2* meta;     // (pixel item, sample)
     uint32_t* q[2];  // closest-ray queues, ping-pong by depth parity
-    uint32_t* qs;    // shadow-ray queue
+    uint32_t* qs;    // shadow-ray queue: up to two rays of a path, toward the sun and a key light
     uint32_t* cost;  // cost maps: inner BVH nodes visited by each path's rays
     float4* Ltot;    // adjoint: radiance of the first pass
     uint4* hits;     // adjoint: hit[] of depths 1..stored, `stride` entries apart, kept by
@@ -97,8 +97,8 @@ constexpr size_t wave_stored_bytes(uint64_t capacity, uint32_t stored, bool tex)
                      (tex ? (((8 * capacity) + 255) & ~uint64_t(255)) : 0));
 }
 constexpr size_t wave_workspace_bytes(uint64_t capacity, bool adjoint) {
-    return 9 * (((16 * capacity) + 255) & ~uint64_t(255)) + 2 * (((8 * capacity) + 255) & ~uint64_t(255)) +
-           4 * (((4 * capacity) + 255) & ~uint64_t(255)) +
+    return 9 * (((16 * capacity) + 255) & ~uint64_t(255)) + 3 * (((8 * capacity) + 255) & ~uint64_t(255)) +
+           3 * (((4 * capacity) + 255) & ~uint64_t(255)) +
            ((sizeof(uint32_t) * kCtrStride * 258 + 255) & ~uint64_t(255)) +
            (adjoint ? (((16 * capacity) + 255) & ~uint64_t(255)) : 0);
 }

@@ -275,3 +275,38 @@ def test_captured_calls_outlive_larger_ones(api, tiny):
             # the same terms, added by FP32 atomics in another order
             torch.testing.assert_close(grad, ref_grad, rtol=1e-4, atol=1e-5 * float(ref_grad.abs().max()))
     gs.check()
+
+
+def test_two_shadow_rays_of_every_path_fit_their_queue(api):
+    """A frame of exactly one chunk (2^13 paths) that looks straight down on a
+    ground under a sun and a key light: every path queues two shadow rays, twice
+    the paths of the chunk.  The cost map's own counters, which lie behind the
+    queue, and the image stay what they are in sixteen chunks and in the
+    single-kernel renderer."""
+    rng = np.random.default_rng(4)
+    c = rng.uniform(-20, 20, size=(300, 1, 3)) * [1, 1, 0] + [0, 0, 4]
+    e = np.array([[-1, -1, 0], [1, -1, 0], [1, 1, 0], [-1, 1, 0]]) * rng.uniform(0.2, 0.8, size=(300, 1, 1))
+    ground = np.array([[[-60, -60, 0], [60, -60, 0], [60, 60, 0], [-60, 60, 0]]])
+    v = np.concatenate([c + e, ground]).astype(np.float32).reshape(-1, 3)
+    sc = I.Scene([(v, np.arange(len(v), dtype=np.uint32).reshape(-1, 4))], I.IDENTITY_XFORM[None].copy(),
+                 np.zeros(1, dtype=np.uint32))
+    gs = api.Scene(sc)
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    view = I.View(eye=(0.0, 0.0, 50.0), look=(0.0, 0.0, 0.0), up=(0.0, 1.0, 0.0), vfov_deg=40.0, w=64, h=64, spp=2)
+    light = np.array([[-5, -5, 30, 0, 10, 0, 10, 0, 0, 9, 8, 7]], dtype=np.float32)  # edge1 x edge2 points down
+    params = I.Params(max_depth=2, sun_dir=(0.1, 0.2, 1.0), sun_E=(2.0, 2.0, 2.0), lights=light)
+    n = 64 * 64 * 2
+    maps, images = [], []
+    for tuning in (dict(chunk_log2=13), dict(chunk_log2=10)):
+        stats = torch.zeros(12, dtype=torch.int64, device="cuda")
+        img = torch.empty((64, 64, 3), device="cuda")
+        (cost,) = gs.cost_maps([view], alb, params, stats, outs=[img], tuning=tuning)
+        gs.check()
+        st = stats.cpu().numpy()
+        assert st[6] == 2 * n and st[0] == 2 * n  # two shadow rays at depth 1; bounces leave upward or hit a quad's back
+        assert int(torch.round(cost.double() * 2).sum()) == int(st[1] + st[7])
+        maps.append(cost)
+        images.append(img)
+    (single,) = gs.render([view], alb, params, tuning=dict(mode=1))
+    assert torch.equal(images[0], images[1]) and torch.equal(images[0], single)
+    assert float((maps[0] - maps[1]).abs().mean()) <= 0.05 * float(maps[0].mean())
