@@ -182,7 +182,9 @@ typedef struct {
  *               the pixel within the view's rendered region, each path taking
  *               2*max_depth + 2 words.
  *   max_steps   traversal step limit per ray (0 = 2^20); exceeding it stops
- *               that ray and raises QRT_ERR_STEP_LIMIT.
+ *               that ray and raises QRT_ERR_STEP_LIMIT.  An occluded shadow
+ *               ray that several lanes share may be answered where one lane
+ *               would have exceeded the limit, never the other way round.
  *   tuning      launch tuning (zeros = defaults).
  *   d_ray_log   optional DEVICE float buffer for diagnostics (NULL = off),
  *               16-byte aligned, indexed by path like d_path_log: per path

@@ -39,7 +39,7 @@ namespace qrt {
 template <int FETCH>
 using PathRay = TraversalKind<false, true, false, FETCH, 10>;
 template <int FETCH>
-using PathShadow = TraversalKind<true, false, true, FETCH, 28>;
+using PathShadow = TraversalKind<true, false, true, FETCH, 27>;
 static_assert(PathShadow<32>::kLaneBytes == PathRay<32>::kLaneBytes, "a warp's part must be the same");
 
 template <int STACK, int FETCH>

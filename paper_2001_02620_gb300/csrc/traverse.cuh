@@ -524,16 +524,17 @@ __device__ __forceinline__ uint32_t keep_register(uint32_t a, uint32_t v) {
 // Per thread kRecs 16-byte records and the stack's entries: 64 bits (distance,
 // reference) for closest-hit rays, whose pops drop entries beyond the best
 // hit; 32 bits (reference) for any-hit rays, which never drop one (tmax stays
-// put until the ray ends).  Per warp, record k of lane l lies at 512 k + 16 l
-// and stack entry k after the records at (32 sizeof(Entry)) k + sizeof(Entry)
-// l: lanes never conflict for a bank, however far apart their stacks are.
+// put until the ray ends) and have one word for the node tests of a shared ray
+// behind them.  Per warp, record k of lane l lies at 512 k + 16 l and stack
+// entry k after the records at (32 sizeof(Entry)) k + sizeof(Entry) l: lanes
+// never conflict for a bank, however far apart their stacks are.
 template <bool ANY_, bool UV_, bool RANGE_, int FETCH_, int STACK_>
 struct TraversalKind {
     static constexpr bool ANY = ANY_, UV = UV_, RANGE = RANGE_;
     static constexpr int FETCH = FETCH_, STACK = STACK_;
     using Entry = std::conditional_t<ANY, uint32_t, uint64_t>;
     static constexpr int kRecs = ANY ? 6 : (UV || RANGE ? 8 : 6);
-    static constexpr int kLaneBytes = kRecs * 16 + STACK * (int)sizeof(Entry);
+    static constexpr int kLaneBytes = kRecs * 16 + STACK * (int)sizeof(Entry) + (ANY ? 4 : 0);
     static_assert(STACK >= 4 && STACK <= 32, "a node's pushes fit, the tuning's caps lie beyond");
 };
 
@@ -616,6 +617,7 @@ struct Traversal {
         rec = keep_register(own, own);
         bottom = keep_register(own, base + 512u * Kind::kRecs + (uint32_t)sizeof(Entry) * lane);
         plane_exp = keep_register(own, 0x3F000000u);
+        if constexpr (ANY) sts_u(steps_word(), 0u);
         cur = kRefNone;
         pleaf = 0;
         found = false;
@@ -807,7 +809,7 @@ struct Traversal {
     // Whether the ray has tested more nodes than it may; such a ray ends here.
     // Asked between steps and not in them, which saves two instructions of
     // every node test: a ray may go some nodes beyond its limit, but never ends
-    // beyond it unreported.
+    // beyond it unreported.  (An any-hit ray shared with other lanes: share_rays.)
     __device__ __forceinline__ void check_budget() {
         if (budget < 0 && !error()) stop(kErrStepLimit);
     }
@@ -1123,10 +1125,10 @@ struct Traversal {
 
     // Takes the entry at address `entry` from the ray of the lane with records
     // at `from` and makes this lane, which is idle, traverse it.  other, its
-    // other_base: that lane's ray and node_base; object_space: the entry lies
-    // in its instance.
+    // other_base, other_budget: that lane's ray, node_base and budget;
+    // object_space: the entry lies in its instance.
     __device__ __forceinline__ void take(const DevScene& S, uint32_t from, uint32_t entry, bool object_space,
-                                         const RaySetup& other, uint32_t other_base) {
+                                         const RaySetup& other, uint32_t other_base, int other_budget) {
 #pragma unroll
         for (int k = 0; k < Kind::kRecs; ++k) {
             const float4 v = lds4(from + 512u * k);
@@ -1136,7 +1138,8 @@ struct Traversal {
         sts_u(entry, kRefNone);
         pleaf = 0;
         tip = inst_tip = bottom;
-        budget = kHelperBudget;
+        budget = other_budget;
+        sts_u(steps_word(), (uint32_t)other_budget);
         found = false;
         waiting = 0;
         if (object_space) {
@@ -1150,17 +1153,37 @@ struct Traversal {
             lim = tmax();
         }
     }
-    static constexpr int kHelperBudget = 0x3FFFFFFF;
 
-    // Takes over what a helper lane found, its steps and its error.
-    __device__ __forceinline__ void absorb(bool its_found, int its_budget) {
-        const uint32_t e = (uint32_t)its_budget - (uint32_t)kStopped;
+    // Of a ray's own lane: the node tests that its helpers made, kFailed and
+    // error bits if one of them was stopped.  Of a helper: its budget when it
+    // began.  Zeroed once: rays are shared when none is left to start, and a
+    // lane that has been a helper never starts one.
+    static constexpr uint32_t kFailed = 0xFFFFFFF0u;
+    __device__ __forceinline__ uint32_t steps_word() const { return bottom + kShared; }
+    // What a helper that is done has to add to its ray's word.
+    __device__ __forceinline__ uint32_t spent() const {
+        return error() ? kFailed | error() : lds_u(steps_word()) - (uint32_t)budget;
+    }
+
+    // Takes over what a helper lane found and spent.
+    __device__ __forceinline__ void absorb(bool its_found, uint32_t its_spent) {
+        const uint32_t had = lds_u(steps_word()), sum = had + its_spent;
+        uint32_t now = sum < had || sum >= kFailed ? kFailed | kErrStepLimit : sum;
+        if (had >= kFailed || its_spent >= kFailed)
+            now = (had >= kFailed ? had : kFailed) | (its_spent >= kFailed ? its_spent : kFailed);
+        sts_u(steps_word(), now);
         if (its_found && !error()) answer();
-        if (e < 16u) {
-            if (!error()) stop(e);
-        } else if (!error()) {
-            budget -= kHelperBudget - its_budget;
-        }
+    }
+
+    // The end of a shared ray (precondition: finished(), no helpers left): one
+    // that is not answered is stopped if its lanes together made more tests than
+    // it may, or one of them was.  The budget then counts them all (cost maps),
+    // but an answered ray's does not go below 0.
+    __device__ __forceinline__ void settle() {
+        const uint32_t c = lds_u(steps_word());
+        if (budget < 0) return;  // beyond the limit by itself
+        if (c <= (uint32_t)budget) budget -= (int)c;
+        else budget = found ? 0 : kStopped | (int)(c >= kFailed ? c & 15u : kErrStepLimit);
     }
 
     // Order of two hits at the same distance.
@@ -1194,6 +1217,16 @@ constexpr uint32_t kHelper = 0xFFFFFF00u, kIdle = 0xFFFFFFFFu;
 // 2.83 -> 2.53 ms, 1.5 M sun rays 0.90 -> 0.82.  Closest-hit rays lost that way
 // (one ray on the mid scene 32 -> 80 us): the far subtrees are those which the
 // near ones' hit culls.
+//
+// The step limit.  The lane that gives goes on as it would alone, from the top
+// of its stack, and what it gives away lies at the bottom, which it would come
+// to last.  So its own tests are those of a ray alone, in order; a helper begins
+// with the budget left to its giver, so that a ray alone is beyond its limit
+// wherever the helper is; and only the end of an unanswered ray adds them up
+// (settle).  An unoccluded ray is reported exactly if it takes more tests than it
+// may, as it is alone; an occluded one that is answered within its limit alone
+// is answered here, whatever its helpers spend.  A ray that is stopped or
+// answered ends its helpers.
 template <class Kind>
 __device__ __forceinline__ void share_rays(const DevScene& S, Traversal<Kind>& T, uint32_t& item, uint32_t base) {
     const unsigned FULL = 0xFFFFFFFFu;
@@ -1212,33 +1245,36 @@ __device__ __forceinline__ void share_rays(const DevScene& S, Traversal<Kind>& T
     const bool object_space = __shfl_sync(FULL, (int)(!T.top(S) && give >= T.inst_tip), src);
     const uint32_t its_item = __shfl_sync(FULL, item, src);
     const uint32_t its_base = __shfl_sync(FULL, T.node_base, src);
+    const int its_budget = __shfl_sync(FULL, T.budget, src);
     const RaySetup its_ray{make_float4(from(T.r.o.x), from(T.r.o.y), from(T.r.o.z), from(T.r.o.w)),
                            make_float4(from(T.r.inv.x), from(T.r.inv.y), from(T.r.inv.z), from(T.r.inv.w))};
     if (takes) {
-        T.take(S, base + 16u * (uint32_t)src, entry, object_space, its_ray, its_base);
+        T.take(S, base + 16u * (uint32_t)src, entry, object_space, its_ray, its_base, its_budget);
         item = its_item >= kHelper ? its_item : kHelper + (uint32_t)src;
     }
     __syncwarp();
 }
 
-// Helpers that are done hand over what they found; an answered ray's helpers
-// end.  Returns the lanes whose ray others still help with.
+// Helpers that are done hand over what they found and spent; the helpers of a
+// ray that is answered or stopped end.  Returns the lanes whose ray others
+// still help with.
 template <class Kind>
 __device__ __forceinline__ unsigned gather_rays(Traversal<Kind>& T, uint32_t& item) {
     const unsigned FULL = 0xFFFFFFFFu;
     const unsigned lane = threadIdx.x & 31u;
     unsigned ready = __ballot_sync(FULL, item >= kHelper && item != kIdle && T.finished());
+    const uint32_t spent = ready >> lane & 1u ? T.spent() : 0u;
     while (ready) {
         const int j = __ffs(ready) - 1;
         ready &= ready - 1;
         const int owner = (int)(__shfl_sync(FULL, item, j) - kHelper);
-        const bool its_found = __shfl_sync(FULL, (int)T.found, j);
-        const int its_budget = __shfl_sync(FULL, T.budget, j);
-        if ((int)lane == owner) T.absorb(its_found, its_budget);
+        const bool its_found = __shfl_sync(FULL, (int)(T.found && !T.error()), j);
+        const uint32_t its_spent = __shfl_sync(FULL, spent, j);
+        if ((int)lane == owner) T.absorb(its_found, its_spent);
         if ((int)lane == j) item = kIdle;
     }
-    const unsigned answered = __ballot_sync(FULL, item < kHelper && T.found);
-    if (item >= kHelper && item != kIdle && (answered >> (item - kHelper) & 1u)) {
+    const unsigned over = __ballot_sync(FULL, item < kHelper && (T.found || T.error()));
+    if (item >= kHelper && item != kIdle && (over >> (item - kHelper) & 1u)) {
         T.answer();  // its steps are still handed over, next time
         T.found = false;
     }
@@ -1370,12 +1406,12 @@ __device__ __forceinline__ void persistent_trace(const DevScene& S, Traversal<Ki
         unsigned helped = 0;  // lanes whose ray others still help with
         if constexpr (Kind::ANY)
             if (!more) helped = gather_rays(T, item);
-        if (item < kHelper) {
-            T.check_budget();
-            if (T.finished() && !(helped >> lane & 1u)) {
-                done(item);
-                item = kIdle;
-            }
+        if (item != kIdle) T.check_budget();
+        if (item < kHelper && T.finished() && !(helped >> lane & 1u)) {
+            if constexpr (Kind::ANY)
+                if (!more) T.settle();
+            done(item);
+            item = kIdle;
         }
     }
 }

@@ -310,3 +310,95 @@ def test_two_shadow_rays_of_every_path_fit_their_queue(api):
     (single,) = gs.render([view], alb, params, tuning=dict(mode=1))
     assert torch.equal(images[0], images[1]) and torch.equal(images[0], single)
     assert float((maps[0] - maps[1]).abs().mean()) <= 0.05 * float(maps[0].mean())
+
+
+def _canopy(n, occluder_z=None):
+    """Ground under n sheets parallel to the sun's direction (1, 0, 1), through
+    whose overlapping boxes a shadow ray from the ground runs without a hit;
+    optionally one quad across those rays, occluder_z above the ground.  Dyadic
+    numbers: the sheets are exactly parallel to the rays."""
+    rng = np.random.default_rng(1)
+    c = np.stack([rng.uniform(-60, 36, n), rng.uniform(-20, 12, n), rng.uniform(20, 24, n)], 1)
+    c = np.round(c * 64) / 64
+    a, b = np.array([24.0, 0, 24]), np.array([0, 8.0, 0])
+    q = np.stack([c, c + a, c + a + b, c + b], 1)
+    if occluder_z is not None:
+        p, u, w = np.array([occluder_z, 0, occluder_z]), np.array([3.0, 0, -3]), np.array([0, 3.0, 0])
+        q = np.concatenate([q, np.stack([p - u - w, p + u - w, p + u + w, p - u + w])[None]])
+    ground = np.array([[[-9, -9, 0], [9, -9, 0], [9, 9, 0], [-9, 9, 0]]])
+    meshes = [(v.astype(np.float32).reshape(-1, 3), np.arange(4 * len(v), dtype=np.uint32).reshape(-1, 4))
+              for v in (q, ground)]
+    return I.Scene(meshes, np.stack([I.IDENTITY_XFORM] * 2), np.arange(2, dtype=np.uint32))
+
+
+class _Limited:
+    """Camera rays at the ground of a _canopy, shadow rays through its sheets."""
+
+    def __init__(self, api, n, occluder_z=None):
+        sc = _canopy(n, occluder_z)
+        self.api, self.gs = api, api.Scene(sc)
+        self.alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+        self.params = I.Params(max_depth=1, sun_dir=(1.0, 0.0, 1.0), sun_E=(2.0, 2.0, 2.0))
+
+    def view(self, side):
+        return I.View(eye=(0.0, 0.0, 10.0), look=(0.0, 0.0, 0.0), up=(0.0, 1.0, 0.0), vfov_deg=20.0, w=side, h=side,
+                      spp=1)
+
+    def stopped(self, side, steps, mode):
+        (img,) = self.gs.render([self.view(side)], self.alb, self.params, max_steps=steps, tuning=dict(mode=mode))
+        try:
+            self.gs.check()
+        except self.api.N.QrtError as e:
+            assert e.code == self.api.N.QRT_ERR_STEP_LIMIT
+            return True, img
+        return False, img
+
+    def least(self, side):
+        """The least limit that stops no ray of the single-kernel renderer, where
+        each ray has one lane."""
+        lo, hi = 1, 1 << 14
+        while lo < hi:
+            m = (lo + hi) // 2
+            if self.stopped(side, m, 1)[0]:
+                lo = m + 1
+            else:
+                hi = m
+        return lo
+
+
+@pytest.mark.parametrize("side", [1, 8])
+def test_step_limit_of_shared_rays(api, side):
+    """An unoccluded any-hit ray is stopped exactly where it is without help, and
+    the lanes that help it stop with it: each of a warp's lanes makes at most the
+    limit and a few turns more."""
+    s = _Limited(api, 20_000)
+    least = s.least(side)
+    assert least > 500
+    for mode in (1, 2):
+        assert s.stopped(side, least - 1, mode)[0]
+        assert not s.stopped(side, least, mode)[0]
+    stats = torch.zeros(12, dtype=torch.int64, device="cuda")
+    limit = 16
+    for steps, most in ((0, side * side * least), (limit, side * side * 32 * (limit + 32))):
+        if steps and least < 32 * (limit + 32) and side == 1:
+            most = least // 2  # one ray alone: its helpers end far from the end of its tree
+        stats.zero_()
+        s.gs.render([s.view(side)], s.alb, s.params, max_steps=steps, tuning=dict(mode=2), stats=stats)
+        if steps:
+            with pytest.raises(api.N.QrtError):
+                s.gs.check()
+        else:
+            s.gs.check()
+        assert int(stats[7]) <= most
+
+
+@pytest.mark.parametrize("z", [21.0, 23.0, 31.0, 45.0])
+def test_an_answered_ray_is_not_charged_for_its_helpers(api, z):
+    """An occluded ray that is answered within its limit without help is answered
+    within it by a warp, whatever other lanes spend on the rest of its tree."""
+    s = _Limited(api, 20_000, z)
+    least = s.least(1)
+    assert least > 200
+    stopped, img = s.stopped(1, least, 2)
+    assert not stopped
+    assert torch.equal(img, s.stopped(1, 0, 1)[1])
