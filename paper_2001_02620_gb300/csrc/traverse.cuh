@@ -977,15 +977,13 @@ struct Traversal {
                 float u = __int_as_float(0x7fffffff), v = 0.f;
                 if constexpr (ANY) {
                     if (!wait && t > t0 && t < t1) return true;
-                } else if (!wait && t > t0 && t < t1 && waiting) {
-                    wait = true;
                 } else if (!wait && t > t0 && t < t1) {
                     const float ht = lds1(rec + kHT);
                     const float4 hr = lds4(rec + kHit);
                     const uint32_t inst = lds_u(rec + kCurInst);
                     const uint32_t hinst = __float_as_uint(hr.x), hslot = __float_as_uint(hr.y);
-                    wait = fabsf(t - ht) <= fmaxf(sh.eps_t, hr.z) && hinst != 0xFFFFFFFFu &&
-                           !(hslot == slot && hinst == inst);
+                    wait = waiting != 0 || (fabsf(t - ht) <= fmaxf(sh.eps_t, hr.z) && hinst != 0xFFFFFFFFu &&
+                           !(hslot == slot && hinst == inst));
                     if (wait || t <= ht) {
                         if constexpr (UV) {
                             u = __fdiv_rn(q.u_num, q.det);
