@@ -137,6 +137,8 @@ typedef struct {
  *                  16 (up to 128 registers a thread), 24 (80), 32 (64,
  *                  default), 40 (48) or 48 (40); more warps hide the latency
  *                  of the dependent node loads, at the price of spills.
+ *                  Shared memory holds closest-hit rays that carry (u, v)
+ *                  (queries, textured renders) to 40 warps.
  *                  With block and occupancy both 0, closest-hit ray queries run
  *                  28 warps (72 registers) in blocks of 128
  *   mode           renderer: 0 = default (wavefront; small frames, of a

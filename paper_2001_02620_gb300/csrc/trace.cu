@@ -48,6 +48,7 @@ static cudaError_t launch_variant(const DevScene& S, const float4* rays, uint64_
                                   uint32_t* occ, uint32_t max_steps, unsigned long long* cursor,
                                   unsigned long long* stats, const Tune& t, int sm_count,
                                   cudaStream_t s) {
+    static_assert(reaches<QueryKind<ANY, FETCH, OCC>>(OCC), "shared memory beyond the resident warps'");
     static ResidentBlocks resident;
     const size_t smem = traversal_bytes<QueryKind<ANY, FETCH, OCC>>(t.block);
     const int per_sm = t.blocks_per_sm > 0 ? t.blocks_per_sm

@@ -539,13 +539,27 @@ struct TraversalKind {
 };
 
 // Stack entries in shared memory: what fits the 228 KB of an SM (less 1 KB a
-// block) at the kernel's resident warps, in blocks of 256 threads.  A ray's
+// block) at the kernel's resident warps, in blocks of 256 threads (at 28 warps
+// of 128), at most 16 for any-hit rays.  A ray's
 // stack seldom holds more than 9 entries, but the deepest of a warp's lanes is
 // beyond 9 in half of a closest-hit frame's node steps and beyond 12 in a
 // sixth, and a lane beyond takes its warp through the slower path.
+constexpr int lane_room(int warps) { return warps > 40 ? 144 : warps > 32 ? 176 : warps > 28 ? 216 : 240; }
 constexpr int shared_stack(bool any, int recs, int warps) {
-    const int fits = ((warps > 40 ? 144 : warps > 32 ? 176 : warps > 28 ? 216 : 240) - 16 * recs) / 8;
-    return any ? 16 : fits > 4 ? fits : 4;
+    const int fits = any ? (lane_room(warps) - 16 * 6 - 4) / 4 : (lane_room(warps) - 16 * recs) / 8;
+    return any && fits > 16 ? 16 : fits < 4 ? 4 : fits;
+}
+
+// Whether a kernel of this kind reaches its resident warps in those blocks.  At
+// 48 warps closest-hit rays with (u, v) have room for two entries only and take
+// four, at 40 warps (2 M diffuse bounces on the mid scene 5.30 ms against 5.74).
+// Any-hit rays have eleven there: sun rays 1.48 -> 1.50 ms against sixteen at
+// 40 warps, the mid frame 19.6 -> 18.8.
+template <class Kind>
+constexpr bool reaches(int warps) {
+    if (warps > 40 && Kind::kRecs == 8) warps = 40;
+    const int block = warps == 28 ? 128 : 256, blocks = 32 * warps / block;
+    return blocks * (block * Kind::kLaneBytes + block / 32 * 16 + 1024) <= 228 * 1024;
 }
 
 // The ray-query kernels' rays, and the wavefront renderer's.

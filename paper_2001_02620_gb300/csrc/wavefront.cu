@@ -400,6 +400,7 @@ __global__ void __launch_bounds__(256) wave_accumulate(const __grid_constant__ W
 template <bool ANY, int FETCH, int OCC, bool STATS, bool UV>
 static cudaError_t launch_wave_trace_v(const WaveArgs& A, int depth, const Tune& t, int sm_count,
                                        cudaStream_t s) {
+    static_assert(reaches<WaveKind<ANY, UV, FETCH, OCC>>(OCC), "shared memory beyond the resident warps'");
     static ResidentBlocks resident;
     const size_t smem = traversal_bytes<WaveKind<ANY, UV, FETCH, OCC>>(t.block);
     const int per_sm = t.blocks_per_sm > 0
