@@ -108,8 +108,12 @@ def proxy_view(view, max_paths: int = 1 << 22):
 
 
 def _time_render(scene, view, albedo, params, out, cand, reps: int) -> float:
-    """Best of `reps` timed renders (after one untimed) with CUDA events."""
+    """Best of `reps` timed renders (after one untimed) with CUDA events, on the
+    wavefront renderer unless the candidate names another: small views take the
+    single kernel by default, which reads neither occupancy nor batch, and the
+    choice is for larger frames of the scene too."""
     import torch
+    cand = {"mode": 2, **cand}
     scene.render([view], albedo, params, outs=[out], tuning=cand)
     scene.check()
     ts = []
