@@ -42,7 +42,9 @@ extern "C" {
 #define QRT_VERSION 1
 
 /* qrt_params.flags */
-#define QRT_FLAG_STAGE_TIMES 1u /* record GPU time of each wavefront stage (qrt_stage_times) */
+#define QRT_FLAG_STAGE_TIMES 1u  /* record GPU time of each wavefront stage (qrt_stage_times) */
+#define QRT_FLAG_NO_KEPT_HITS 2u /* qrt_render_adjoint: keep no hits, and give back what earlier calls
+                                    on the stream keep for them */
 
 /* Most key lights one render takes (qrt_params.n_lights). */
 #define QRT_MAX_LIGHTS 32
@@ -348,10 +350,13 @@ int qrt_render_spp_static(qrt_scene scene, const qrt_view* views, uint32_t n_vie
  * Paths are recomputed from their random streams instead of being stored
  * (path replay); contributions are added with FP32 atomics.  Per path the
  * wavefront renderer keeps its radiance, one visibility bit per sun shadow ray
- * of depths 1..32 and, for as many depths as 8 GB kept for the stream hold (16
- * bytes per path and depth, 24 with textures; fewer or none where that memory
- * cannot be had, or in a capture that would have to allocate it), the closest
- * hits; its replay traces the other rays again.
+ * of depths 1..32 and the closest hits of as many depths as 8 GB hold, or an
+ * eighth of the device memory free at the time if that is less (16 bytes per
+ * path and depth, 24 with textures; fewer or none where that memory cannot be
+ * had, or in a capture that would have to allocate it); its replay traces the
+ * other rays again.  That memory is kept for the stream's next adjoint until
+ * the scene is destroyed, a larger render needs it or a call with
+ * QRT_FLAG_NO_KEPT_HITS gives it back.
  * d_dimage: host array of n_views DEVICE pointers, each float [h*w*3]. */
 int qrt_render_adjoint(qrt_scene scene, const qrt_view* views, uint32_t n_views,
                        const float* d_albedo, const float* const* d_dimage,

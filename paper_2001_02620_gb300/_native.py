@@ -22,6 +22,7 @@ QRT_ERR_STEP_LIMIT = -6
 QRT_ERR_NOT_READY = -7
 
 QRT_FLAG_STAGE_TIMES = 1
+QRT_FLAG_NO_KEPT_HITS = 2
 STAGES = ("gen", "trace_closest", "shade", "trace_shadow", "accumulate")
 
 ERROR_NAMES = {

@@ -232,12 +232,18 @@ class Scene:
         return costs
 
     def adjoint(self, views, albedo: torch.Tensor, dimages, grad: torch.Tensor, params: Params,
-                tuning: dict | None = None, stream=None) -> torch.Tensor:
-        """Adds the albedo gradient of sum(dimage * image) into grad [n_quads, 3]."""
+                tuning: dict | None = None, stream=None, keep_hits: bool = True) -> torch.Tensor:
+        """Adds the albedo gradient of sum(dimage * image) into grad [n_quads, 3].
+
+        keep_hits: the replay follows the hits of the first pass, in device
+        memory that stays with the stream (at most 8 GB); False traces them
+        again and gives that memory back."""
         if isinstance(views, View):
             views = [views]
         cv = make_views(views, [None] * len(views))
         cp = make_params(params, tuning)
+        if not keep_hits:
+            cp.flags |= N.QRT_FLAG_NO_KEPT_HITS
         dptr = (C.c_void_p * len(views))(*[_ptr(d) for d in dimages])
         N.check(N.lib().qrt_render_adjoint(self.handle, cv, len(views), _ptr(albedo), dptr,
                                            _ptr(grad), C.byref(cp), _stream(stream)))

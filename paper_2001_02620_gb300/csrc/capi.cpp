@@ -837,12 +837,17 @@ struct DeviceMem {
     }
     void release(void* p) { cudaFree(p); }
     int drain() { return (int)(error = cudaStreamSynchronize(s)); }
+    // An eighth of what is free: the caller's own allocations come after this one.
+    size_t spare() {
+        size_t free = 0, total = 0;
+        return cudaMemGetInfo(&free, &total) == cudaSuccess ? free / 8 : 0;
+    }
 };
 
 // Makes sl hold a wavefront workspace of `bytes` and, where that memory can be
-// had, `hits` bytes for kept hits.  Allocation is refused while the stream is
-// being captured.
-int ensure_workspace(StreamSlot& sl, size_t bytes, size_t hits, cudaStream_t s) {
+// had, kept hits of `depths` depths of `hits` bytes each.  Allocation is
+// refused while the stream is being captured.
+int ensure_workspace(StreamSlot& sl, size_t bytes, size_t hits, uint32_t depths, cudaStream_t s) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t ce = cudaStreamIsCapturing(s, &cs);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaStreamIsCapturing");
@@ -853,7 +858,14 @@ int ensure_workspace(StreamSlot& sl, size_t bytes, size_t hits, cudaStream_t s) 
         return fail(QRT_ERR_NOT_READY,
                     "wavefront workspace must be allocated before capture: render once on this "
                     "stream outside capture, or use qrt_render_graph_create");
-    if (!e && hits) e = want(sl.hits, hits, capturing, sl.retired, mem);
+    if (e == kNoMemory && sl.hits.ptr && !sl.hits.captured) {  // it comes first
+        e = mem.drain();
+        if (!e) {
+            let_go(sl.hits, sl.retired, mem);
+            e = need(sl.ws, bytes, capturing, sl.retired, mem);
+        }
+    }
+    if (!e && depths) e = want(sl.hits, hits, depths, capturing, sl.retired, mem);
     if (e) return cuda_fail(mem.error, "wavefront workspace");
     return QRT_OK;
 }
@@ -891,7 +903,7 @@ int wave_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, const
     int rc = make_params(params, W.P);
     uint32_t stored = 0;  // depths whose hits there is room for
     const bool tex = rc == QRT_OK && W.P.tex_res != 0;
-    if (adjoint && rc == QRT_OK) {
+    if (adjoint && rc == QRT_OK && !(params->flags & QRT_FLAG_NO_KEPT_HITS)) {
         stored = wave_stored_depths(cap, W.P.max_depth);
         while (stored && wave_stored_bytes(cap, stored, tex) > scratch.hits_bytes) --stored;
     }
@@ -987,6 +999,19 @@ int render_enqueue(qrt_scene scene, const qrt_view* views, uint32_t n_views, con
     return rc;
 }
 
+// Gives the kept hits of stream s back, outside a capture (one that a captured
+// call uses stays until the scene is destroyed).
+int drop_hits(StreamSlot& sl, cudaStream_t s) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &cs);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing");
+    if (!sl.hits.ptr || cs != cudaStreamCaptureStatusNone) return QRT_OK;
+    DeviceMem mem{s};
+    if (mem.drain()) return cuda_fail(mem.error, "stream synchronize");
+    let_go(sl.hits, sl.retired, mem);
+    return QRT_OK;
+}
+
 // Scratch for a plain (non-graph) call on stream s.
 int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* views,
                    uint32_t n_views, bool adjoint, cudaStream_t s, Scratch& out) {
@@ -1000,11 +1025,13 @@ int stream_scratch(qrt_scene scene, const qrt_params* params, const qrt_view* vi
     if (t.mode == 2) {
         // one workspace per stream, sized for the adjoint so both fit
         const uint64_t cap = 1ull << t.chunk_log2;
-        size_t hits = 0;
-        if (adjoint && params && params->max_depth >= 1 && params->max_depth <= 256)
-            hits = wave_stored_bytes(cap, wave_stored_depths(cap, params->max_depth),
-                                     params->d_tex && params->tex_res);
-        rc = ensure_workspace(sl, wave_workspace_bytes(cap, true), hits, s);
+        const bool keep = !params || !(params->flags & QRT_FLAG_NO_KEPT_HITS);
+        uint32_t depths = 0;
+        if (adjoint && keep && params && params->max_depth >= 1 && params->max_depth <= 256)
+            depths = wave_stored_depths(cap, params->max_depth);
+        if (adjoint && !keep && (rc = drop_hits(sl, s))) return rc;
+        rc = ensure_workspace(sl, wave_workspace_bytes(cap, true),
+                              wave_stored_bytes(cap, 1, params && params->d_tex && params->tex_res), depths, s);
         if (rc) return rc;
         // the second stream is made outside capture; a capture started
         // before the first render on this stream runs the stages in order

@@ -9,7 +9,8 @@
 //
 // Mem is where the memory comes from: int alloc(void**, size_t) (0, kNoMemory
 // or another error of its own), void release(void*), int drain() (waits for
-// the stream's queued work; 0 or an error).
+// the stream's queued work; 0 or an error), size_t spare() (what optional
+// memory may take now).
 #pragma once
 #include <stddef.h>
 
@@ -64,18 +65,26 @@ int need(StreamBuffer& b, size_t bytes, bool capturing, std::vector<void*>& reti
     return 0;
 }
 
-// Makes b hold `bytes` if that memory can be had outside a capture, and leaves
-// it as it is otherwise.  A size that was refused is not tried again.
+// Makes b hold `count` times `unit` bytes, or as many as may be spared, if that
+// memory can be had outside a capture, and leaves it as it is otherwise.  A
+// size that was refused, or cut, is not tried again.
 template <class Mem>
-int want(StreamBuffer& b, size_t bytes, bool capturing, std::vector<void*>& retired, Mem& mem) {
+int want(StreamBuffer& b, size_t unit, size_t count, bool capturing, std::vector<void*>& retired, Mem& mem) {
+    size_t bytes = unit * count;
     if (b.bytes >= bytes || capturing || bytes >= b.refused) {
         b.captured = b.captured || (capturing && b.ptr);
         return 0;
     }
+    const size_t spare = mem.spare();
+    if (bytes > spare) {
+        b.refused = bytes;
+        bytes = spare / unit * unit;
+        if (bytes <= b.bytes) return 0;
+    }
     void* p = nullptr;
     int e = mem.alloc(&p, bytes);
     if (e == kNoMemory) {
-        b.refused = bytes;
+        b.refused = bytes < b.refused ? bytes : b.refused;
         return 0;
     }
     if (e) return e;

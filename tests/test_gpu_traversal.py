@@ -402,3 +402,33 @@ def test_an_answered_ray_is_not_charged_for_its_helpers(api, z):
     stopped, img = s.stopped(1, least, 2)
     assert not stopped
     assert torch.equal(img, s.stopped(1, 0, 1)[1])
+
+
+def test_kept_hits_can_be_refused_and_are_given_back(api, tiny):
+    """A large adjoint keeps its hits on the device (128 MiB here) until a call
+    without them gives the memory back; the gradient is the same."""
+    sc, gs = tiny
+    view = dataclasses.replace(I.tiny_view(), w=512, h=512, spp=8)
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    dimg = torch.from_numpy(np.random.default_rng(9).normal(size=(512, 512, 3)).astype(np.float32)).cuda()
+    p = I.Params(max_depth=4, sun_dir=I.MID_SUN_DIR, sun_E=(2.0, 2.0, 2.0))
+    hits = 16 * 512 * 512 * 8 * 4
+    s = torch.cuda.Stream()
+
+    def grad(keep):
+        g = torch.zeros_like(alb)
+        gs.adjoint([view], alb, [dimg], g, p, keep_hits=keep)
+        s.synchronize()
+        return g, torch.cuda.mem_get_info()[0]
+
+    with torch.cuda.stream(s):
+        grad(False)  # the workspace
+        without, free = grad(False)
+        kept, less = grad(True)
+        again, back = grad(False)
+    gs.check()
+    assert free - less >= hits and back - less >= hits
+    # the same terms, added by FP32 atomics in another order
+    tol = dict(rtol=1e-4, atol=1e-5 * float(kept.abs().max()))
+    torch.testing.assert_close(without, kept, **tol)
+    torch.testing.assert_close(again, kept, **tol)
