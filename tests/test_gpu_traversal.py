@@ -432,3 +432,20 @@ def test_kept_hits_can_be_refused_and_are_given_back(api, tiny):
     tol = dict(rtol=1e-4, atol=1e-5 * float(kept.abs().max()))
     torch.testing.assert_close(without, kept, **tol)
     torch.testing.assert_close(again, kept, **tol)
+
+
+def test_wavefront_splits_many_views(api, tiny):
+    """More small views than one launch holds, by the wavefront (by default they
+    take the single kernel), in one chunk and in several."""
+    sc, gs = tiny
+    views = _views([(16, 8 + k % 3) for k in range(70)], [1 + k % 2 for k in range(70)])
+    alb = torch.from_numpy(I.albedo(sc.n_quads)).cuda()
+    params = I.Params(max_depth=4, sun_dir=I.MID_SUN_DIR, sun_E=(2.0, 2.0, 2.0), lights=I.tiny_lights())
+    whole = gs.render(views, alb, params, tuning=dict(mode=2))
+    parts = gs.render(views, alb, params, tuning=dict(mode=2, chunk_log2=10))
+    single = gs.render(views, alb, params, tuning=dict(mode=1))
+    gs.check()
+    for v, a, b, c in zip(views, whole, parts, single):
+        assert torch.equal(a, b) and torch.equal(a, c)
+    for k in (0, 63, 64, 69):
+        assert torch.equal(gs.render([views[k]], alb, params, tuning=dict(mode=2))[0], whole[k])
