@@ -254,19 +254,20 @@ def bench_trace(api, scene, view, d_alb, params, dev, tuning=None, n=1 << 22):
     of the workload's view: camera rays, first diffuse bounces, shadow rays.
     The query kernels return each hit's (u, v), which the render's
     closest-hit kernel drops, so they carry more state: each query is timed
-    with the render's register budget and with 40 warps/SM, the faster
-    reported (both budgets give the same hits)."""
+    with the library's own choice of block and register budget, with the
+    render's budget and with 40 warps/SM, the fastest reported (all give the
+    same hits)."""
     import torch
     out = {}
     base = dict(tuning or {})
-    budgets = sorted({base.get("occupancy", 32), 40})
+    own = {k: v for k, v in base.items() if k not in ("block", "occupancy")}
+    budgets = {"default": own, **{o: dict(base, occupancy=o) for o in sorted({base.get("occupancy", 32), 40})}}
     for name, d in dumped_rays(api, scene, view, d_alb, params, n, tuning).items():
         m = d.shape[0]
         hits = torch.empty((m, 4), dtype=torch.int32, device=dev)
         bits = torch.empty(((m + 31) // 32,), dtype=torch.int32, device=dev)
         tc = ta = None
-        for occ in budgets:
-            t = dict(base, occupancy=occ)
+        for occ, t in budgets.items():
             c = _time(lambda: scene.trace_closest(d, hits, tuning=t), 5)
             a = _time(lambda: scene.trace_any(d, bits, tuning=t), 5)
             if tc is None or c < tc[0]:
