@@ -130,8 +130,9 @@ typedef struct {
  *   blocks_per_sm  resident blocks per SM for persistent kernels (default:
  *                  as many as the register budget allows)
  *   batch          single kernel: pixels a warp claims per fetch, in units
- *                  of 32; wavefront and ray queries: rays a lane claims per
- *                  fetch (1..64, default 1)
+ *                  of 32; wavefront and ray queries: rays claimed for each
+ *                  idle lane near a queue's end, before which a warp claims
+ *                  32 at a time (1..64, default 1)
  *   stack          traversal stack entries per ray (32 or 64)
  *   fetch          node fetch width in bytes (16: 4x128-bit, 32: 2x256-bit
  *                  loads, default)

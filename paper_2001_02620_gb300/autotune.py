@@ -1,8 +1,8 @@
 """Autotuner for the launch parameters of the renderer.
 
 Searches node-fetch width, block size, the trace kernels' register budget
-(resident warps per SM), the rays a lane claims per fetch (`batch`) and the
-traversal stack depth, by timing renders of a proxy view (the target view at
+(resident warps per SM), the rays claimed for each idle lane near a queue's
+end (`batch`) and the traversal stack depth, by timing renders of a proxy view (the target view at
 reduced resolution, same spp and depth), and keeps the fastest
 configuration that raised no device error.
 
@@ -15,9 +15,8 @@ qrt_scene_stats).  A depth that merely sufficed on the proxy view could
 overflow on another view, and an overflow changes results.  Where no
 candidate below the library's 64 entries is proven, 64 is kept (overflows
 there are still detected and reported by qrt_check).  The stack's place is
-not searched: the per-thread stack in local memory (cached in L1) beat a
-stack whose bottom 4-16 entries sit in shared memory in every measured
-configuration, and the shared-memory branch cost 9 % even when switched off.
+not searched: its first entries, as many as each register budget leaves room
+for, are in shared memory.
 
 Results are cached as JSON keyed by (GPU name, SM count, scene class), so
 later runs skip the search.  None of the parameters changes a rendered

@@ -245,7 +245,7 @@ Tune resolve_tuning(const qrt_tuning* t) {
 // [10, kFitChunkMax].  One chunk per call where it fits: every chunk pays
 // its own run of draining launches, and a whole mid frame (2^22 paths) in
 // one chunk renders 1.12x faster than in two (a Moana-scale frame of 2^25
-// paths: 1.03x faster than in two).  2^25 paths of workspace is about 5.5 GB
+// paths: 1.03x faster than in two).  2^25 paths of workspace is about 6.6 GB
 // (adjoint included) per stream, 2 % of GB300's memory.
 constexpr int kFitChunkMax = 25;
 

@@ -35,13 +35,16 @@
 // of 32; some 410 warp instructions per node step, all phases counted) and,
 // behind them, each ray's chain of dependent node loads, hidden by resident
 // warps.  So the registers hold what a node test reads and shared memory the
-// rest of a ray and its stack: 64 registers (32 warps an SM) without spills.
-// Left to the compiler, the state spilled 476 bytes a thread at 48 registers,
-// the 64-entry stacks lay in local memory, a node test sorted its children and
-// the FP64 re-test sat in the leaf loop.  That against this on one GB300, ms:
-// 2 M diffuse bounces on the mid scene 5.59 -> 2.80, 1.5 M sun rays 1.62 ->
-// 0.81, 1 M rays of ambient occlusion on the island (0.40 re-tests a ray) 1.95
-// -> 0.79, the mid frame 16.9 -> 9.9, the island frame 33.1 -> 19.7.
+// rest of a ray and its stack: 64 registers (32 warps an SM) with few spills
+// (bytes stored a thread: 16 for the renderer's closest-hit rays, 64 with
+// textures, 4 for its any-hit rays, 24 for any-hit queries; none for
+// closest-hit queries, at 72 registers).  Left to the compiler, the state
+// spilled 476 bytes a thread at 48 registers, the 64-entry stacks lay in local
+// memory, a node test sorted its children and the FP64 re-test sat in the leaf
+// loop.  That against this on one GB300, ms: 2 M diffuse bounces on the mid
+// scene 5.59 -> 2.82, 1.5 M sun rays 1.63 -> 0.81, 1 M rays of ambient
+// occlusion on the island (0.40 re-tests a ray) 1.94 -> 0.80, the mid frame
+// 18.0 -> 10.5, the island frame 34.5 -> 20.4.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -137,11 +140,9 @@ __device__ __forceinline__ float maxabs3(float a, float b, float c) {
 
 // --------------------------------------------------------------------------
 // Node fetch: 64 bytes as four 128-bit or two 256-bit read-only loads.  The
-// loads do not allocate in L1: with 32 or more warps per SM the per-ray
-// local memory (spilled values and traversal stacks) needs L1, and node
-// lines, which are seldom reused by the same SM soon enough, would only
-// evict it (the mid frame measured 657 -> 674 Mrays/s with the hint, 678
-// with quads read the same way; L2 still caches both).
+// loads do not allocate in L1: shared memory leaves it little room, and node
+// lines are seldom reused by the same SM soon enough (nodes, or everything,
+// allocating there: 0 to 3 % slower; L2 caches both).
 // --------------------------------------------------------------------------
 __device__ __forceinline__ uint4 ld_nc_na(const void* p) {
     uint4 v;

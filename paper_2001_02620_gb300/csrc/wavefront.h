@@ -86,7 +86,7 @@ struct WaveArgs {
     uint64_t P0;        // first path of the current chunk
     uint64_t capacity;  // paths per chunk
     uint32_t n_views;
-    uint32_t batch;     // rays a lane claims per fetch
+    uint32_t batch;     // rays claimed for each idle lane near a queue's end
     uint32_t cost_on;   // record per-path traversal cost (counting launches only)
     ViewDev views[kMaxViewsPerLaunch];
 };
